@@ -115,13 +115,14 @@ sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const
   a.q_pitch = p->q_pitch;
   a.copies = p->d_presum_copies;
   a.copies_max = p->presum_copies_max;
-  a.data_bytes = p->presum_data_bytes;
+  a.stage_bytes = p->presum_stage_bytes;
+  a.chunk_rows = p->d_presum_chunks;
   a.offs = p->d_presum_offs;
   a.di_pad = presum_di_pad(cfg);
   a.n_dm = rows;
   a.n_groups = p->channels / per;
   a.group_units = (per + K - 1) / K;
-  a.fold_units = 65535 / (255 * K);
+  a.fold_units = presum_fold_units(cfg);
   a.max_start = (int32_t)(p->n_in - p->n_t);
   a.n_out = n_out;
   a.out_pitch = out_pitch;
@@ -196,7 +197,7 @@ sps_status run_dedisperse(const sps_plan* p, const uint8_t* x, int64_t pitch, in
   uint8_t* x4 = static_cast<uint8_t*>(ws);
   if ((s = prepare_input(p, &x, &pitch, &x4, st))) return s;
   if (p->mode == SPS_MODE_BRUTE)
-    return run_u8_pass(p, p->cfg.brute, x, pitch, x4, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
+    return run_u8_pass(p, p->brute_tile, x, pitch, x4, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
                        p->dmax_brute, D, 0, st);
   uint16_t* Y = reinterpret_cast<uint16_t*>(x4 + y_offset(p));
   if ((s = run_step1(p, x, pitch, x4, Y, st))) return s;
@@ -253,7 +254,7 @@ sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int
   if ((s = check_workspace(p, ws, ws_bytes))) return s;
   uint8_t* w = static_cast<uint8_t*>(ws);
   if ((s = prepare_input(p, &x, &pitch, &w, st))) return s;
-  return presum_prepass(p, p->cfg.brute, x, pitch, w, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
+  return presum_prepass(p, p->brute_tile, x, pitch, w, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
                         p->dmax_brute, D, 0, st, args);
 }
 
@@ -289,6 +290,7 @@ sps_status sps_plan_destroy(sps_plan* p) {
   cudaFree(p->d_presum_series);
   cudaFree(p->d_presum_units);
   cudaFree(p->d_zap);
+  cudaFree(p->d_presum_chunks);
   cudaFree(p->d_presum_copies);
   cudaFree(p->d_presum_offs);
   if (swap) cudaSetDevice(cur);
@@ -443,10 +445,21 @@ sps_status sps_presum_tables_verify(const int32_t* delays, int32_t rows, int32_t
   std::string why;
   if (!presum_config_supported(*cfg, &why)) return fail(SPS_ERR_INVALID_ARG, why);
   const std::vector<int32_t> d(delays, delays + (size_t)rows * channels);
-  PresumTables t;
-  if (sps_status s = build_presum_tables(d, rows, channels, per, build_n_out, *cfg, &t)) return s;
-  if (!verify_presum_tables(d, rows, channels, per, read_n_out, *cfg, t, &why)) return fail(SPS_ERR_INVALID_ARG, why);
-  return SPS_OK;
+  // a stage holds the configured chunk of units, or, for the wide tile that may
+  // take the default tile's place, is fixed
+  auto check = [&](const sps_dedisp_config& c, int32_t units, int32_t fixed) {
+    const int32_t Di = c.warps_dm * c.dms_per_thread, Tt = c.warps_time * 32 * c.samples_per_thread;
+    const int32_t need = presum_stage_data(d, rows, channels, per, 1 << c.presum, Di, units, Tt) +
+                         units * presum_di_pad(c) * 2;
+    if (fixed && need > fixed) return SPS_OK;  // not taken
+    PresumTables t;
+    if (sps_status s = build_presum_tables(d, rows, channels, per, build_n_out, c, fixed ? fixed : need, &t)) return s;
+    if (!verify_presum_tables(d, rows, channels, per, read_n_out, c, t, &why)) return fail(SPS_ERR_INVALID_ARG, why);
+    return SPS_OK;
+  };
+  if (sps_status s = check(*cfg, presum_chunk(*cfg), 0)) return s;
+  sps_dedisp_config wide;
+  return per == channels && wide_form(*cfg, channels, &wide) ? check(wide, 1, kWideStage) : SPS_OK;
 }
 
 sps_status sps_plan_status(const sps_plan* p, uint32_t* host_status, int32_t clear) {

@@ -48,8 +48,8 @@ double beam_work(const sps_plan* p) { return (double)p->dms.size() * p->n_t * p-
 using ConfigKey = std::tuple<int32_t, int32_t, int32_t, int32_t, int32_t, int32_t, int32_t>;
 
 ConfigKey key_of(const sps_plan* p, int32_t smem_per_sm) {
-  const sps_dedisp_config& c = p->cfg.brute;
-  const size_t per_block = presum_smem_bytes(c, p->presum_data_bytes) + 1024;  // + the block's reserved share
+  const sps_dedisp_config& c = p->brute_tile;
+  const size_t per_block = presum_smem_bytes(p->presum_stage_bytes) + 1024;  // + the block's reserved share
   const int32_t resident = (int32_t)std::max<size_t>(1, (size_t)smem_per_sm / per_block);
   return ConfigKey{c.dms_per_thread, c.samples_per_thread, c.warps_dm, c.warps_time, c.chunk, c.presum, resident};
 }
@@ -173,7 +173,7 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
     int64_t n_work = 0;
     for (int32_t b = 0; b < n_beams; b++) {
       if (!L.batched[b]) continue;
-      const sps_dedisp_config& c = plans[b]->cfg.brute;
+      const sps_dedisp_config& c = plans[b]->brute_tile;
       PresumPassArgs shape{};
       shape.n_dm = (int32_t)plans[b]->dms.size();
       shape.n_out = plans[b]->n_t;
@@ -217,15 +217,15 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
       cudaStream_t sg = streams[gi % B];
       const int32_t first = pass_of[beams[0]];
       const size_t w0 = work.size();
-      int32_t max_data = 0;
+      int32_t max_stage = 0;
       for (int32_t b : beams) {
         cuda_ok(cudaStreamWaitEvent(sg, pre_done[b], 0), "cudaStreamWaitEvent");
-        presum_pass_work(passes[pass_of[b]], plans[b]->cfg.brute, pass_of[b] - first, &work);
-        max_data = std::max(max_data, passes[pass_of[b]].data_bytes);
+        presum_pass_work(passes[pass_of[b]], plans[b]->brute_tile, pass_of[b] - first, &work);
+        max_stage = std::max(max_stage, passes[pass_of[b]].stage_bytes);
       }
       if (st == SPS_OK)
         st = launch_presum_pass_list(batch->d_passes + first, batch->d_work + w0, (int64_t)(work.size() - w0),
-                                     plans[beams[0]]->cfg.brute, max_data, sg);
+                                     plans[beams[0]]->brute_tile, max_stage, sg);
       batch->list_launches++;
       if (st == SPS_OK) cuda_ok(cudaEventRecord(group_done[gi], sg), "cudaEventRecord");
     }
@@ -251,7 +251,7 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
   if (st == SPS_OK && n_passes) {
     int64_t n_work = 0;
     for (int32_t b = 0; b < n_beams; b++)
-      if (L.batched[b]) n_work += presum_pass_blocks(passes[pass_of[b]], plans[b]->cfg.brute);
+      if (L.batched[b]) n_work += presum_pass_blocks(passes[pass_of[b]], plans[b]->brute_tile);
     if ((int64_t)work.size() != n_work) st = fail(SPS_ERR_INVALID_ARG, "batched work list size changed");
   }
   if (st == SPS_OK && n_passes) {

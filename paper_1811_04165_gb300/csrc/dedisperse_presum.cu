@@ -21,6 +21,15 @@
 // are <= 255 K, so 16-bit lanes are exact for 65535 / (255 K) units (128 pairs,
 // 64 quads); partial sums fold into int32 registers that often.  A group whose
 // size is not a multiple of K ends in a shorter unit.
+//
+// The wide tile (8 trials x 7 words per thread) keeps no int32 sums: a fold moves
+// the lanes' multiples of 4096 into 8-bit counts, four to a register, so a thread
+// holds 112 outputs in 84 registers where int32 sums take 192.  It is bound by
+// the shared-memory loads: with 64 trials x 448 samples per block the windows
+// staged per output (L2 -> shared, which alone took 0.6 ms of a 2048-trial pass
+// with 32 x 512 tiles) fall by 40 %, and loads run at 81 % of the LSU peak.  On
+// 1536 channels x 12500 samples x 2048 trials the pass takes 597 us (800 us with
+// the 4 x 8 tile, 825 before chunks were packed by size).
 #include <algorithm>
 
 #include "sps_internal.h"
@@ -38,6 +47,18 @@ __device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
   if constexpr (M < NW) {
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(w[M]) : "r"(addr), "n"(M * 128));
     lds_row<NW, M + 1>(addr, w);
+  }
+}
+
+// The same into `w` only where `load` is set (uniform over the warp); otherwise
+// `w` keeps its words.
+template <int NW, int M = 0>
+__device__ __forceinline__ void lds_row_if(bool load, uint32_t addr, uint32_t (&w)[NW]) {
+  if constexpr (M < NW) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u32 %0, [%1+%3];\n\t}"
+                 : "+r"(w[M])
+                 : "r"(addr), "r"((uint32_t)load), "n"(M * 128));
+    lds_row_if<NW, M + 1>(load, addr, w);
   }
 }
 
@@ -67,33 +88,34 @@ __device__ __forceinline__ void load_offs(const uint16_t* p, uint32_t (&o)[ND]) 
 }
 
 // One block's tile: DM tile `tile`, time tile `ty`, group `g` of the pass `a`.
-template <int ND, int NW>
+// WIDE: 8-bit counts instead of int32 sums (see the top of the file).
+template <int ND, int NW, bool WIDE>
 __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int tile, int ty, int g, int wd,
-                                                  int cp_max, int wb) {
+                                                  int wb) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int wt = (int)(blockDim.x >> 5) / wd;
   const int Tt = wt * 64 * NW;
   const int Di = wd * ND;
   const int copies_max = a.copies_max;
-  const int stage_bytes = a.data_bytes + cp_max * a.di_pad * 2;
+  const int stage_bytes = a.stage_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * stage_bytes);
   uint64_t* empty = full + kStages;
   __shared__ volatile int aborted;
   __shared__ volatile int issued_upto;  // chunks [0, issued_upto) have been issued
+  __shared__ volatile int chunk_units[kStages];  // units of the chunk in a stage
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nwarps = (int)(blockDim.x >> 5);
   const int dm_sub = warp % wd, t_sub = warp / wd;
   const int i0 = tile * Di;
   const int t0 = ty * Tt;
-  const int P = a.group_units;
-  const int n_chunks = (P + cp_max - 1) / cp_max;
+  const int4 chunks = __ldg(&a.chunk_rows[(int64_t)tile * a.n_groups + g]);
+  const int n_chunks = chunks.y;
   const uint32_t toff = (uint32_t)(t_sub * 128 * NW + lane * 4);  // bytes
-  const int64_t chunk_row = ((int64_t)tile * a.n_groups + g) * n_chunks;
   const bool clip = t0 + wb / 2 + a.max_start > a.q_pitch;  // windows may be cut at the row end
   // bounds-checked build: the largest staged offset whose NW words fit the
   // stage's windows, and the warp's trials inside a row of the offset table
-  const int64_t lim = (int64_t)a.data_bytes - (int64_t)(toff + 128 * (NW - 1) + 4);
+  const int64_t lim = (int64_t)stage_bytes - (int64_t)(toff + 128 * (NW - 1) + 4);
   if (kBoundsCheck && (dm_sub + 1) * ND > a.di_pad) stage_read_ok(1u, -1, a.status);
 
   if (tid == 0) {
@@ -112,13 +134,14 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   // byte in the stage and its length; lane 0 also copies the chunk's offset
   // table and arrives on the stage's "full" barrier with the byte count (the
   // list's last entry, unless a window may be cut at the end of a row).  The
-  // issuing warp fetches the count and its first list entry per lane a chunk
-  // early (`fetch`).
+  // issuing warp asks for its list a chunk early (`fetch`): the wide tile
+  // loads the head and its first entry per lane; the narrow ones, whose sums
+  // leave no registers to hold them over a chunk, bring the list into L1.
   // A list entry is {row, start, (stage byte / 16) | (bytes / 16) << 16, 0};
-  // the last is {count, total bytes}.
+  // the last is {count, total bytes, units, offset table / 8 entries}.
   struct Fetched { uint32_t nt; int row, start, at; };  // nt = count | total << 14
-  auto fetch = [&](int ch) {
-    const int4* list = a.copies + (chunk_row + ch) * (copies_max + 1);
+  auto load_list = [&](int ch) {
+    const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
     Fetched f;
     const int4 h = __ldg(&list[copies_max]);
     f.nt = (uint32_t)h.x | ((uint32_t)h.y << 14);
@@ -128,12 +151,21 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
     f.at = e.z;
     return f;
   };
-  auto issue = [&](int ch, const Fetched& f) {
+  auto fetch = [&](int ch) {
+    if constexpr (WIDE) return load_list(ch);
+    const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
+    // a 128-byte line holds eight entries
+    const int at = min(8 * lane, copies_max);
+    if (at < copies_max || lane == 31) asm volatile("prefetch.global.L1 [%0];" ::"l"(list + at));
+    return Fetched{};
+  };
+  auto issue = [&](int ch, const Fetched& fetched) {
     const int st = ch % kStages;
     uint8_t* sb = smem + st * stage_bytes;
-    const int pb = ch * cp_max, cp = min(cp_max, P - pb);
-    const int4* list = a.copies + (chunk_row + ch) * (copies_max + 1);
-    const uint32_t tbl_bytes = (uint32_t)(cp * a.di_pad * 2);
+    const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
+    const Fetched f = WIDE ? fetched : load_list(ch);
+    const int4 head = __ldg(&list[copies_max]);
+    const uint32_t tbl_bytes = (uint32_t)(head.z * a.di_pad * 2);
     const int n = (int)(f.nt & 0x3FFFu);
     auto entry = [&](int q) {
       if (q == lane) return make_int3(f.row, f.start, f.at);
@@ -151,7 +183,10 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) bytes_all += __shfl_xor_sync(0xffffffffu, bytes_all, o);
     }
-    if (lane == 0) mbar_arrive_expect_tx(&full[st], bytes_all + tbl_bytes);
+    if (lane == 0) {
+      chunk_units[st] = head.z;
+      mbar_arrive_expect_tx(&full[st], bytes_all + tbl_bytes);
+    }
     __syncwarp();
     for (int q = lane; q < n; q += 32) {
       const int3 e = entry(q);
@@ -159,19 +194,38 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
       bulk_g2s(sb + ((uint32_t)e.z & 0xFFFFu) * 16, src, (uint32_t)length(e), &full[st]);
     }
     if (lane == 0) {
-      const uint16_t* src = a.offs + (((int64_t)tile * a.n_groups + g) * P + pb) * a.di_pad;
-      bulk_g2s(sb + a.data_bytes, src, tbl_bytes, &full[st]);
+      bulk_g2s(sb, a.offs + (int64_t)head.w * 8, tbl_bytes, &full[st]);
       issued_upto = ch + 1;
     }
   };
 
   uint32_t lanes[ND][NW];
-  int32_t acc[ND][NW][2];
+  int32_t acc[WIDE ? 1 : ND][WIDE ? 1 : NW][2];
+  uint32_t cnt[WIDE ? ND * NW / 2 : 1];  // counts of two words' four samples
 #pragma unroll
   for (int r = 0; r < ND; r++)
 #pragma unroll
-    for (int m = 0; m < NW; m++) { lanes[r][m] = 0u; acc[r][m][0] = 0; acc[r][m][1] = 0; }
+    for (int m = 0; m < NW; m++) {
+      lanes[r][m] = 0u;
+      if constexpr (!WIDE) { acc[r][m][0] = 0; acc[r][m][1] = 0; }
+    }
+  if constexpr (WIDE) {
+#pragma unroll
+    for (int k = 0; k < ND * NW / 2; k++) cnt[k] = 0u;
+  }
   auto fold = [&]() {
+    if constexpr (WIDE) {
+      // the lanes' multiples of kWideCount move to the counts
+#pragma unroll
+      for (int k = 0; k < ND * NW / 2; k++) {
+        uint32_t& x = lanes[2 * k / NW][2 * k % NW];
+        uint32_t& y = lanes[(2 * k + 1) / NW][(2 * k + 1) % NW];
+        cnt[k] += ((x >> 12) & 0x000F000Fu) + (((y >> 12) & 0x000F000Fu) << 8);
+        x &= 0x0FFF0FFFu;
+        y &= 0x0FFF0FFFu;
+      }
+      return;
+    } else {
 #pragma unroll
     for (int r = 0; r < ND; r++)
 #pragma unroll
@@ -180,6 +234,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
         acc[r][m][1] += (int32_t)(lanes[r][m] >> 16);
         lanes[r][m] = 0u;
       }
+    }
   };
 
   // Chunks 0 and 1 go out first; after computing chunk ch, warp (ch mod
@@ -197,32 +252,50 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   bool bad = false;
   for (; ch < n_chunks; ch++) {
     const int st = ch % kStages;
-    const int cp = min(cp_max, P - ch * cp_max);
     const bool issuer = turn == warp && ch + kStages - 1 < n_chunks;
     if (++turn == nwarps) turn = 0;
-    if (pending + cp > a.fold_units) { fold(); pending = 0; }
     Fetched next{};
     if (issuer) next = fetch(ch + kStages - 1);
     if (!bad && !mbar_wait(&full[st], (ch / kStages) & 1, a.status)) {
       bad = true;
       aborted = 1;
     }
+    const int cp = bad ? 0 : chunk_units[st];
+    if (pending + cp > a.fold_units) { fold(); pending = 0; }
     if (!bad) {
       const uint32_t base = smem_u32(smem) + (uint32_t)(st * stage_bytes) + toff;
       const uint16_t* tb =
-          reinterpret_cast<const uint16_t*>(smem + st * stage_bytes + a.data_bytes) + dm_sub * ND;
+          reinterpret_cast<const uint16_t*>(smem + st * stage_bytes) + dm_sub * ND;
       int p = 0;
       for (; p + 1 < cp; p += 2) {
         uint32_t e0[ND], e1[ND];
         load_offs<ND>(tb + p * a.di_pad, e0);
         load_offs<ND>(tb + (p + 1) * a.di_pad, e1);
+        if constexpr (WIDE && !kBoundsCheck) {
+          // a trial that reads the words of the trial before it (the same series
+          // at the same delay: 11 % of the reads at 0.2 pc cm^-3 per trial, 21 %
+          // at 0.1) takes them from the registers
+          uint32_t A[NW], B[NW];
+          lds_row<NW>(base + e0[0], A);
+          lds_row<NW>(base + e1[0], B);
 #pragma unroll
-        for (int r = 0; r < ND; r++) {
-          uint32_t A[NW] = {}, B[NW] = {};
-          if (stage_read_ok(e0[r], lim, a.status)) lds_row<NW>(base + e0[r], A);
-          if (stage_read_ok(e1[r], lim, a.status)) lds_row<NW>(base + e1[r], B);
+          for (int r = 0; r < ND; r++) {
+            if (r > 0) {
+              lds_row_if<NW>(e0[r] != e0[r - 1], base + e0[r], A);
+              lds_row_if<NW>(e1[r] != e1[r - 1], base + e1[r], B);
+            }
 #pragma unroll
-          for (int m = 0; m < NW; m++) lanes[r][m] += A[m] + B[m];
+            for (int m = 0; m < NW; m++) lanes[r][m] += A[m] + B[m];
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < ND; r++) {
+            uint32_t A[NW] = {}, B[NW] = {};
+            if (stage_read_ok(e0[r], lim, a.status)) lds_row<NW>(base + e0[r], A);
+            if (stage_read_ok(e1[r], lim, a.status)) lds_row<NW>(base + e1[r], B);
+#pragma unroll
+            for (int m = 0; m < NW; m++) lanes[r][m] += A[m] + B[m];
+          }
         }
       }
       if (p < cp) {
@@ -259,7 +332,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
         mbar_wait(&full[k % kStages], (k / kStages) & 1, nullptr);
     return;
   }
-  fold();
+  if constexpr (!WIDE) fold();
 
   // Each lane holds 2 consecutive samples per (trial, word).
   const bool vec = (a.out_pitch & 1) == 0;
@@ -272,21 +345,30 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
     for (int m = 0; m < NW; m++) {
       const int t = t0 + (int)(toff >> 1) + 64 * m;
       if (t >= a.n_out) continue;
-      if (a.out_u16) {
+      int32_t s0, s1;
+      if constexpr (WIDE) {
+        const uint32_t c = cnt[(r * NW + m) / 2] >> (8 * ((r * NW + m) & 1));
+        s0 = (int32_t)((lanes[r][m] & 0xFFFFu) + (c & 0xFFu) * kWideCount);
+        s1 = (int32_t)((lanes[r][m] >> 16) + ((c >> 16) & 0xFFu) * kWideCount);
+      } else {
+        s0 = acc[r][m][0];
+        s1 = acc[r][m][1];
+      }
+      if (!WIDE && a.out_u16) {
         uint16_t* o = static_cast<uint16_t*>(a.out) + row * a.out_pitch + t;
         if (t + 1 < a.n_out && vec) {
-          *reinterpret_cast<uint32_t*>(o) = (uint32_t)acc[r][m][0] | ((uint32_t)acc[r][m][1] << 16);
+          *reinterpret_cast<uint32_t*>(o) = (uint32_t)s0 | ((uint32_t)s1 << 16);
         } else {
-          o[0] = (uint16_t)acc[r][m][0];
-          if (t + 1 < a.n_out) o[1] = (uint16_t)acc[r][m][1];
+          o[0] = (uint16_t)s0;
+          if (t + 1 < a.n_out) o[1] = (uint16_t)s1;
         }
       } else {
         int32_t* o = static_cast<int32_t*>(a.out) + row * a.out_pitch + t;
         if (t + 1 < a.n_out && vec) {
-          *reinterpret_cast<int2*>(o) = make_int2(acc[r][m][0], acc[r][m][1]);
+          *reinterpret_cast<int2*>(o) = make_int2(s0, s1);
         } else {
-          o[0] = acc[r][m][0];
-          if (t + 1 < a.n_out) o[1] = acc[r][m][1];
+          o[0] = s0;
+          if (t + 1 < a.n_out) o[1] = s1;
         }
       }
     }
@@ -295,8 +377,8 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
 
 template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
-presum_pass_kernel(PresumPassArgs a, int wd, int cp_max, int wb) {
-  presum_pass_block<ND, NW>(a, blockIdx.x, blockIdx.y, blockIdx.z, wd, cp_max, wb);
+presum_pass_kernel(PresumPassArgs a, int wd, int wb) {
+  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, blockIdx.x, blockIdx.y, blockIdx.z, wd, wb);
 }
 
 // Batched form: one launch over a work list of tiles from several passes of
@@ -304,11 +386,10 @@ presum_pass_kernel(PresumPassArgs a, int wd, int cp_max, int wb) {
 // tile, group}; each pass's arguments (and its window bytes) live in `passes`.
 template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
-presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* __restrict__ work, int wd,
-                        int cp_max) {
+presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* __restrict__ work, int wd) {
   const int4 w = work[blockIdx.x];
   const PresumPassArgs& a = passes[w.x];
-  presum_pass_block<ND, NW>(a, w.y, w.z, w.w, wd, cp_max, a.window_bytes);
+  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, w.w, wd, a.window_bytes);
 }
 
 // Adds bytes o + j .. o + j + 15 of W (24 bytes, o in 0 .. 7), for j = 0 and
@@ -517,8 +598,8 @@ __global__ void __launch_bounds__(256) presum_series_direct_kernel(const uint8_t
   store_series(q, q_pitch, s, u0, v);
 }
 
-typedef void (*PresumKernel)(PresumPassArgs, int, int, int);
-typedef void (*PresumListKernel)(const PresumPassArgs*, const int4*, int, int);
+typedef void (*PresumKernel)(PresumPassArgs, int, int);
+typedef void (*PresumListKernel)(const PresumPassArgs*, const int4*, int);
 
 template <int ND, int NW>
 constexpr PresumKernel k() { return presum_pass_kernel<ND, NW>; }
@@ -531,7 +612,7 @@ const Variant kVariants[] = {
     SPS_PRESUM_VARIANT(1, 2), SPS_PRESUM_VARIANT(1, 4), SPS_PRESUM_VARIANT(1, 8), SPS_PRESUM_VARIANT(1, 16),
     SPS_PRESUM_VARIANT(2, 2), SPS_PRESUM_VARIANT(2, 4), SPS_PRESUM_VARIANT(2, 8), SPS_PRESUM_VARIANT(2, 16),
     SPS_PRESUM_VARIANT(4, 2), SPS_PRESUM_VARIANT(4, 4), SPS_PRESUM_VARIANT(4, 8),
-    SPS_PRESUM_VARIANT(8, 2), SPS_PRESUM_VARIANT(8, 4),
+    SPS_PRESUM_VARIANT(8, 2), SPS_PRESUM_VARIANT(8, 4), SPS_PRESUM_VARIANT(8, 7),
 };
 #undef SPS_PRESUM_VARIANT
 
@@ -562,7 +643,8 @@ bool presum_config_supported(const sps_dedisp_config& c, std::string* why) {
     *why = "presum must be 1 (pairs) or 2 (quads) for this kernel";
     return false;
   }
-  if (c.samples_per_thread % 2 || !find(c.dms_per_thread, c.samples_per_thread / 2)) {
+  if (c.samples_per_thread % 2 || !find(c.dms_per_thread, c.samples_per_thread / 2) ||
+      presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) {
     *why = "no compiled pre-summed variant for this (dms_per_thread, samples_per_thread)";
     return false;
   }
@@ -578,10 +660,12 @@ bool presum_config_supported(const sps_dedisp_config& c, std::string* why) {
   return true;
 }
 
-size_t presum_smem_bytes(const sps_dedisp_config& c, int32_t data_bytes) {
-  const size_t stage = (size_t)data_bytes + (size_t)presum_chunk(c) * presum_di_pad(c) * 2;
-  return kStages * stage + 16 * kStages;
+int presum_fold_units(const sps_dedisp_config& c) {
+  const int room = presum_wide(c.dms_per_thread, c.samples_per_thread / 2) ? 65536 - (int)kWideCount : 65535;
+  return room / (255 << c.presum);
 }
+
+size_t presum_smem_bytes(int32_t stage_bytes) { return kStages * (size_t)stage_bytes + 16 * kStages; }
 
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
                                 int32_t n_units, int32_t unit_channels, int32_t max_rel, const PresumSeries* series,
@@ -606,17 +690,15 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
 }
 
 sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& c, cudaStream_t st) {
-  std::string why;
-  if (!presum_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
   PresumKernel fn = find(c.dms_per_thread, c.samples_per_thread / 2);
+  if (!fn) return fail(SPS_ERR_INVALID_ARG, "no compiled pre-summed variant");
   const int Di = c.warps_dm * c.dms_per_thread;
   const int Tt = c.warps_time * 32 * c.samples_per_thread;
-  const size_t smem = presum_smem_bytes(c, a.data_bytes);
+  const size_t smem = presum_smem_bytes(a.stage_bytes);
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, a.n_groups);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
   SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, presum_chunk(c),
-                                                        presum_window_bytes(c, a.dmax_tile));
+  fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, presum_window_bytes(c, a.dmax_tile));
   SPS_CUDA(cudaGetLastError());
   return SPS_OK;
 }
@@ -637,15 +719,13 @@ void presum_pass_work(const PresumPassArgs& a, const sps_dedisp_config& c, int32
 }
 
 sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d_work, int64_t n_work,
-                                   const sps_dedisp_config& c, int32_t max_data_bytes, cudaStream_t st) {
-  std::string why;
-  if (!presum_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
+                                   const sps_dedisp_config& c, int32_t max_stage_bytes, cudaStream_t st) {
   if (n_work < 1 || n_work > 0x7fffffff) return fail(SPS_ERR_UNSUPPORTED, "work list size out of range");
   const Variant* v = find_variant(c.dms_per_thread, c.samples_per_thread / 2);
-  const size_t smem = presum_smem_bytes(c, max_data_bytes);
+  if (!v) return fail(SPS_ERR_INVALID_ARG, "no compiled pre-summed variant");
+  const size_t smem = presum_smem_bytes(max_stage_bytes);
   SPS_CUDA(cudaFuncSetAttribute(v->list, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  v->list<<<(unsigned)n_work, 32 * c.warps_dm * c.warps_time, smem, st>>>(d_passes, d_work, c.warps_dm,
-                                                                         presum_chunk(c));
+  v->list<<<(unsigned)n_work, 32 * c.warps_dm * c.warps_time, smem, st>>>(d_passes, d_work, c.warps_dm);
   SPS_CUDA(cudaGetLastError());
   return SPS_OK;
 }

@@ -122,8 +122,9 @@ std::vector<sps_kernel_config> default_configs() {
   return out;
 }
 
-// Largest packed window data of any (tile, group, chunk) of the pre-summed
-// kernel for a configuration (cached).
+// Bytes of a stage of the pre-summed kernel for a configuration: the largest
+// windows of any (tile, group) of its chunk of units, and their offset table
+// (cached).
 int32_t cached_presum_stage(const sps_plan* p, int which, const sps_dedisp_config& c) {
   const int32_t Di = c.warps_dm * c.dms_per_thread, cu = presum_chunk(c);
   const int32_t Tt = c.warps_time * 32 * c.samples_per_thread;
@@ -132,10 +133,11 @@ int32_t cached_presum_stage(const sps_plan* p, int which, const sps_dedisp_confi
   auto it = p->presum_stage_cache.find(key);
   if (it != p->presum_stage_cache.end()) return it->second;
   const int32_t K = 1 << c.presum;
-  const int32_t v = which == 0
+  const int32_t data = which == 0
                         ? presum_stage_data(p->delays, (int32_t)p->dms.size(), p->channels, p->channels, K, Di, cu, Tt)
                         : presum_stage_data(p->d1, (int32_t)p->coarse_dms.size(), p->channels,
                                             p->channels / p->n_subbands, K, Di, cu, Tt);
+  const int32_t v = (int32_t)std::min<int64_t>((int64_t)data + (int64_t)cu * presum_di_pad(c) * 2, INT32_MAX);
   p->presum_stage_cache[key] = v;
   return v;
 }
@@ -175,7 +177,7 @@ sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigC
     c.dmax_b = cached_spread(p, 0, di);
     const size_t need =
         cfg.brute.presum
-            ? presum_smem_bytes(cfg.brute, cached_presum_stage(p, 0, cfg.brute))
+            ? presum_smem_bytes(cached_presum_stage(p, 0, cfg.brute))
             : u8_smem_bytes(cfg.brute, c.dmax_b, p->channels, 1);
     if (need > (size_t)p->max_smem)
       return fail(SPS_ERR_INVALID_ARG, "brute config needs more shared memory than a block may use");
@@ -198,7 +200,7 @@ sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigC
     const int32_t di1 = cfg.step1.warps_dm * cfg.step1.dms_per_thread;
     const size_t need1 =
         cfg.step1.presum
-            ? presum_smem_bytes(cfg.step1, cached_presum_stage(p, 1, cfg.step1))
+            ? presum_smem_bytes(cached_presum_stage(p, 1, cfg.step1))
             : u8_smem_bytes(cfg.step1, c.dmax_1, p->channels / S, S);
     if (need1 > (size_t)p->max_smem)
       return fail(SPS_ERR_INVALID_ARG, "step1 config needs more shared memory than a block may use");
@@ -209,53 +211,95 @@ sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigC
   return SPS_OK;
 }
 
+// Whether `c` is the default pre-summed tile, and the wide tile in its place.
+bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* wide) {
+  *wide = {8, 14, 8, 1, 16, 2};
+  return c.presum == 2 && c.dms_per_thread == 4 && c.samples_per_thread == 16 && c.warps_dm == 8 &&
+         c.warps_time == 1 && c.chunk == 16 && channels <= kWideChannels;
+}
+
+// The tile the brute-force pass runs with.  The default pre-summed tile leaves
+// the choice to the library: the wide tile (64 trials x 448 samples per block, 8
+// trials x 7 words per thread, two blocks per SM) reads shared memory at 81 % of
+// its peak and half the series windows per output, so it takes over once its
+// larger blocks fill the GPU as well as the default's.  Cycles per unit of a
+// round of resident blocks, measured on the 1536-channel band (0.2 pc cm^-3 per
+// trial): wide 1020 with two blocks per SM and 775 with one, default 750 and
+// 585; 2048 trials of 12500 samples take 597 us against 800.
+sps_dedisp_config presum_tile(const sps_plan* p, const sps_dedisp_config& c) {
+  sps_dedisp_config wide;
+  if (!wide_form(c, p->channels, &wide)) return c;
+  auto cost = [&](const sps_dedisp_config& t, int64_t two, int64_t one) {
+    const int64_t di = t.warps_dm * t.dms_per_thread, tt = 32 * t.warps_time * t.samples_per_thread;
+    const int64_t blocks = ((int64_t)p->dms.size() + di - 1) / di * ((p->n_t + tt - 1) / tt);
+    const int64_t last = blocks % (2 * p->sms);
+    return blocks / (2 * p->sms) * two + (last > p->sms ? two : (last ? one : 0));
+  };
+  if (cost(wide, 1020, 775) >= cost(c, 750, 585)) return c;
+  sps_dedisp_config unit = wide;  // sized for single units: the largest unit's stage
+  unit.chunk = 4;
+  return cached_presum_stage(p, 0, unit) <= kWideStage ? wide : c;
+}
+
+int32_t presum_stage(const sps_plan* p, const sps_dedisp_config& c) {
+  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return kWideStage;
+  return cached_presum_stage(p, p->mode == SPS_MODE_BRUTE ? 0 : 1, c);
+}
+
 // Recompute everything that depends on the kernel configuration.
 sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   ConfigCheck chk;
   if (sps_status s = check_config(p, cfg, &chk)) return s;
   const int32_t n_dms = (int32_t)p->dms.size();
-  const int32_t dmax_b = chk.dmax_b, dmax_1 = chk.dmax_1, dmax_2 = chk.dmax_2;
+  const sps_dedisp_config tile = p->mode == SPS_MODE_BRUTE ? presum_tile(p, cfg.brute) : cfg.brute;
+  const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : cfg.step1;
+  const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0, dmax_1 = chk.dmax_1, dmax_2 = chk.dmax_2;
   const std::vector<int32_t>& tiles = chk.tiles;
-  const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? cfg.brute : cfg.step1;
   if (pass.presum) {
     PresumTables pt;
     sps_status s = p->mode == SPS_MODE_BRUTE
-                       ? build_presum_tables(p->delays, n_dms, p->channels, p->channels, (int32_t)p->n_t, pass, &pt)
+                       ? build_presum_tables(p->delays, n_dms, p->channels, p->channels, (int32_t)p->n_t, pass,
+                                             presum_stage(p, pass), &pt)
                        : build_presum_tables(p->d1, (int32_t)p->coarse_dms.size(), p->channels,
-                                             p->channels / p->n_subbands, (int32_t)p->n_1, pass, &pt);
+                                             p->channels / p->n_subbands, (int32_t)p->n_1, pass, presum_stage(p, pass), &pt);
     if (s) return s;
     PresumSeries* dser = nullptr;
     PresumUnit* dunit = nullptr;
+    int4* dchunks = nullptr;
     int4* dslot = nullptr;
     uint16_t* doffs = nullptr;
     s = upload(pt.series, &dser);
     if (s == SPS_OK) s = upload(pt.units, &dunit);
+    if (s == SPS_OK) s = upload(pt.chunk_rows, &dchunks);
     if (s == SPS_OK) s = upload(pt.copies, &dslot);
     if (s == SPS_OK) s = upload(pt.offs, &doffs);
     if (s != SPS_OK) {
       cudaFree(dser);
       cudaFree(dunit);
+      cudaFree(dchunks);
       cudaFree(dslot);
       return s;
     }
     cudaFree(p->d_presum_series);
     cudaFree(p->d_presum_units);
+    cudaFree(p->d_presum_chunks);
     cudaFree(p->d_presum_copies);
     cudaFree(p->d_presum_offs);
     p->d_presum_series = dser;
     p->d_presum_units = dunit;
     p->n_presum_units = (int32_t)pt.units.size();
     p->presum_max_rel = pt.max_rel;
+    p->d_presum_chunks = dchunks;
     p->d_presum_copies = dslot;
     p->d_presum_offs = doffs;
     p->n_presum_series = (int32_t)pt.series.size();
     p->presum_copies_max = pt.copies_max;
-    p->presum_data_bytes = pt.data_bytes;
+    p->presum_stage_bytes = pt.stage_bytes;
   } else {
     std::vector<int32_t> b0;
     std::vector<uint32_t> offs;
     if (p->mode == SPS_MODE_BRUTE)
-      build_u8_tables(p->delays, n_dms, p->channels, p->channels, cfg.brute, dmax_b, &b0, &offs);
+      build_u8_tables(p->delays, n_dms, p->channels, p->channels, tile, dmax_b, &b0, &offs);
     else
       build_u8_tables(p->d1, (int32_t)p->coarse_dms.size(), p->channels, p->channels / p->n_subbands, cfg.step1,
                       dmax_1, &b0, &offs);
@@ -282,6 +326,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
     p->step2_tiles_host = tiles;
   }
   p->cfg = cfg;
+  p->brute_tile = tile;
   p->config_gen++;
   p->dmax_brute = dmax_b;
   p->dmax_step1 = dmax_1;
@@ -406,9 +451,10 @@ sps_status plan_create(const sps_plan_desc* d, sps_plan** out) {
                                     d->mode == SPS_MODE_BRUTE
                                         ? count_presum_series(p->delays, n_dms, C, C, K)
                                         : count_presum_series(p->d1, d->n_coarse, C, C / d->n_subbands, K));
-  if (cudaDeviceGetAttribute(&p->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess) {
+  if (cudaDeviceGetAttribute(&p->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     delete p;
-    return fail(SPS_ERR_CUDA, "cudaDeviceGetAttribute(max shared memory)");
+    return fail(SPS_ERR_CUDA, "cudaDeviceGetAttribute(max shared memory, multiprocessors)");
   }
   if (p->n_in > INT32_MAX / 2) { delete p; return fail(SPS_ERR_UNSUPPORTED, "input rows too long"); }
   int64_t max_sum = (int64_t)255 * C * p->widths.back();

@@ -14,15 +14,18 @@
 //            the sample range its trials read for outputs t < n_out:
 //            [min d', max d' + n_out), d' = the reference delay rounded down
 //            to even (copy 1 at d - 1 holds the samples from d on);
-//   copies : per (DM tile, group, chunk of units), the windows of series
-//            copies the tile reads -- one per (tuple, parity of d) that occurs,
-//            each just long enough for its trials -- packed back to back in
-//            the shared-memory stage: {row, start, (stage byte / 16) |
-//            (bytes / 16) << 16, 0}, and last {count, total bytes};
-//   offs   : per (DM tile, group, unit, trial), the offset of the trial's first
-//            sample inside the packed stage, in 4-byte words as uint16 (a stage
-//            is well below 256 KiB), so that one vector load fetches a warp's
-//            offsets for a unit.
+//   chunks : per (DM tile, group), its units in order, as many per chunk as fit
+//            a shared-memory stage (windows differ in length and number over the
+//            band, so a chunk holds more units where they are small);
+//   copies : per chunk, the windows of series copies the tile reads -- one per
+//            (tuple, parity of d) that occurs, each just long enough for its
+//            trials -- packed back to back in the stage: {row, start, (stage
+//            byte / 16) | (bytes / 16) << 16, 0}, and last {count, total bytes,
+//            units, offset table / 8 entries};
+//   offs   : per chunk, at the start of its stage, per (unit, trial) the offset
+//            of the trial's first sample inside the stage, in 4-byte words as
+//            uint16 (a stage is well below 256 KiB), so that one vector load
+//            fetches a warp's offsets for a unit.
 // Tiles start at multiples of 64 samples, so nothing depends on the time tile.
 #include <algorithm>
 #include <array>
@@ -54,13 +57,18 @@ Rel rel_of(const std::vector<int32_t>& d, int32_t C, int32_t i, Unit un) {
   return r;
 }
 
-// Distinct tuples of one unit over rows [i0, i1], in sorted order.
+// Distinct tuples of one unit over rows [i0, i1], in sorted order.  (Neighbouring
+// trials mostly share theirs.)
 std::vector<Rel> distinct_rels(const std::vector<int32_t>& d, int32_t C, int32_t i0, int32_t i1, Unit un) {
   std::vector<Rel> v;
-  v.reserve((size_t)(i1 - i0 + 1));
-  for (int32_t i = i0; i <= i1; i++) v.push_back(rel_of(d, C, i, un));
-  std::sort(v.begin(), v.end());
-  v.erase(std::unique(v.begin(), v.end()), v.end());
+  Rel last{-1, -1, -1};
+  for (int32_t i = i0; i <= i1; i++) {
+    const Rel r = rel_of(d, C, i, un);
+    if (r == last && i > i0) continue;
+    last = r;
+    const auto at = std::lower_bound(v.begin(), v.end(), r);
+    if (at == v.end() || *at != r) v.insert(at, r);
+  }
   return v;
 }
 
@@ -79,14 +87,15 @@ std::vector<TileCopy> tile_copies(const std::vector<int32_t>& d, int32_t C, int3
                                   const std::vector<Rel>& rels) {
   std::vector<TileCopy> out;
   for (int32_t i = i0; i <= i1; i++) {
-    const int32_t k = index_of(rels, rel_of(d, C, i, un));
+    const int32_t k = rels.size() == 1 ? 0 : index_of(rels, rel_of(d, C, i, un));
     const int32_t de = ref_delay(d, C, i, un), j = de & 1, e = de & ~1;
-    auto it = std::find_if(out.begin(), out.end(), [&](const TileCopy& c) { return c.k == k && c.j == j; });
-    if (it == out.end()) {
+    size_t q = 0;
+    while (q < out.size() && (out[q].k != k || out[q].j != j)) q++;
+    if (q == out.size()) {
       out.push_back({k, j, e, e});
     } else {
-      it->lo = std::min(it->lo, e);
-      it->hi = std::max(it->hi, e);
+      out[q].lo = std::min(out[q].lo, e);
+      out[q].hi = std::max(out[q].hi, e);
     }
   }
   std::sort(out.begin(), out.end(), [](const TileCopy& a, const TileCopy& b) {
@@ -130,15 +139,14 @@ int32_t presum_stage_data(const std::vector<int32_t>& d, int32_t rows, int32_t C
 }
 
 sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C, int32_t per, int32_t n_out,
-                               const sps_dedisp_config& cfg, PresumTables* out) {
+                               const sps_dedisp_config& cfg, int32_t stage_bytes, PresumTables* out) {
   const int32_t K = 1 << cfg.presum;
   const int32_t G = C / per;
   const int32_t U = (per + K - 1) / K;
   const int32_t Di = cfg.warps_dm * cfg.dms_per_thread;
   const int32_t Tt = cfg.warps_time * 32 * cfg.samples_per_thread;
   const int32_t di_pad = presum_di_pad(cfg);
-  const int32_t cu = presum_chunk(cfg);
-  const int32_t n_chunks = (U + cu - 1) / cu;
+  const int32_t most = std::min(presum_fold_units(cfg), kPresumChunkUnits);
   const int32_t n_tiles = (rows + Di - 1) / Di;
 
   // series: per unit, every tuple over all trials
@@ -176,53 +184,74 @@ sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int3
       out->max_rel = std::max(out->max_rel, max_rel);
     }
 
-  // copy lists per (tile, group, chunk), packed in order; the offsets of each
-  // trial point at its (tuple, parity) copy
-  const size_t n_chunk_rows = (size_t)n_tiles * G * n_chunks;
-  std::vector<std::vector<int4>> lists(n_chunk_rows);
-  std::vector<int32_t> used(n_chunk_rows, 0);
-  out->offs.assign((size_t)n_tiles * G * U * di_pad, 0);
-  int32_t copies_max = 0, data_bytes = 0;
+  // chunks per (tile, group): units taken in order while their windows and
+  // offsets fit a stage; the offsets of each trial point at its (tuple, parity)
+  // copy in the stage, behind the chunk's offset table
+  out->chunk_rows.clear();
+  out->copies_max = 0;
+  std::vector<std::vector<int4>> lists;
+  std::vector<int4> heads;
   for (int32_t tile = 0; tile < n_tiles; tile++) {
     const int32_t i0 = tile * Di, i1 = std::min(i0 + Di, rows) - 1;
-    for (int32_t g = 0; g < G; g++)
+    for (int32_t g = 0; g < G; g++) {
+      const size_t first = lists.size();
+      std::vector<std::vector<Rel>> rels(U);
+      std::vector<std::vector<TileCopy>> copies(U);
+      std::vector<int32_t> bytes(U, 0);
       for (int32_t u = 0; u < U; u++) {
         const Unit un = unit_of(g, u, per, K);
-        const size_t row = ((size_t)tile * G + g) * n_chunks + u / cu;
-        const std::vector<Rel> rels = distinct_rels(d, C, i0, i1, un);
-        const std::vector<TileCopy> copies = tile_copies(d, C, i0, i1, un, rels);
-        std::vector<int32_t> dst(copies.size());
-        for (size_t q = 0; q < copies.size(); q++) {
-          const TileCopy& c = copies[q];
-          const int32_t series = sbase[(size_t)g * U + u] + index_of(all[(size_t)g * U + u], rels[c.k]);
-          dst[q] = used[row];
-          lists[row].push_back({2 * series + c.j, copy_start(c), (dst[q] >> 4) | ((copy_bytes(c, Tt) >> 4) << 16), 0});
-          used[row] += copy_bytes(c, Tt);
-        }
-        copies_max = std::max<int32_t>(copies_max, (int32_t)lists[row].size());
-        data_bytes = std::max(data_bytes, used[row]);
-        const size_t key = ((size_t)tile * G + g) * U + u;
-        for (int32_t r = 0; r < di_pad; r++) {
-          const int32_t i = std::min(i0 + std::min(r, Di - 1), rows - 1);
-          const int32_t k = index_of(rels, rel_of(d, C, i, un));
-          const int32_t de = ref_delay(d, C, i, un);
-          size_t q = 0;
-          while (copies[q].k != k || copies[q].j != (de & 1)) q++;
-          const int64_t word = ((int64_t)dst[q] + 2 * ((de & ~1) - copy_start(copies[q]))) / 4;
-          if (word > 0xFFFF) return fail(SPS_ERR_UNSUPPORTED, "pre-summed staging window beyond 256 KiB");
-          out->offs[key * di_pad + r] = (uint16_t)word;
-        }
+        rels[u] = distinct_rels(d, C, i0, i1, un);
+        copies[u] = tile_copies(d, C, i0, i1, un, rels[u]);
+        for (const TileCopy& c : copies[u]) bytes[u] += copy_bytes(c, Tt);
       }
+      for (int32_t u0 = 0; u0 < U;) {
+        int32_t n = 0, need = 0;
+        while (u0 + n < U && n < most && need + bytes[u0 + n] + 2 * di_pad <= stage_bytes) {
+          need += bytes[u0 + n] + 2 * di_pad;
+          n++;
+        }
+        if (n == 0) return fail(SPS_ERR_UNSUPPORTED, "a pre-summed unit's windows exceed a stage");
+        if (n > 4 && u0 + n < U) n &= ~1;  // units are added two at a time
+        int32_t at = n * 2 * di_pad;  // windows follow the offset table
+        lists.emplace_back();
+        const size_t table = out->offs.size();
+        out->offs.resize(table + (size_t)n * di_pad, 0);
+        for (int32_t u = u0; u < u0 + n; u++) {
+          const Unit un = unit_of(g, u, per, K);
+          std::vector<int32_t> dst(copies[u].size());
+          for (size_t q = 0; q < copies[u].size(); q++) {
+            const TileCopy& c = copies[u][q];
+            const int32_t series = sbase[(size_t)g * U + u] + index_of(all[(size_t)g * U + u], rels[u][c.k]);
+            dst[q] = at;
+            lists.back().push_back({2 * series + c.j, copy_start(c), (at >> 4) | ((copy_bytes(c, Tt) >> 4) << 16), 0});
+            at += copy_bytes(c, Tt);
+          }
+          for (int32_t r = 0; r < di_pad; r++) {
+            const int32_t i = std::min(i0 + std::min(r, Di - 1), rows - 1);
+            const int32_t k = index_of(rels[u], rel_of(d, C, i, un));
+            const int32_t de = ref_delay(d, C, i, un);
+            size_t q = 0;
+            while (copies[u][q].k != k || copies[u][q].j != (de & 1)) q++;
+            const int64_t word = ((int64_t)dst[q] + 2 * ((de & ~1) - copy_start(copies[u][q]))) / 4;
+            if (word > 0xFFFF) return fail(SPS_ERR_UNSUPPORTED, "pre-summed staging window beyond 256 KiB");
+            out->offs[table + (size_t)(u - u0) * di_pad + r] = (uint16_t)word;
+          }
+        }
+        heads.push_back({(int32_t)lists.back().size(), at - n * 2 * di_pad, n, (int32_t)(table / 8)});
+        out->copies_max = std::max<int32_t>(out->copies_max, (int32_t)lists.back().size());
+        u0 += n;
+      }
+      out->chunk_rows.push_back({(int32_t)first, (int32_t)(lists.size() - first), 0, 0});
+    }
   }
-  if (data_bytes >= (1 << 18) || copies_max >= (1 << 14))
+  if (stage_bytes >= (1 << 18) || out->copies_max >= (1 << 14))
     return fail(SPS_ERR_UNSUPPORTED, "pre-summed stage beyond 256 KiB or 16383 windows");
-  out->copies_max = copies_max;
-  out->data_bytes = data_bytes;
-  out->copies.assign(n_chunk_rows * (size_t)(copies_max + 1), int4{-1, 0, 0, 0});
-  for (size_t q = 0; q < n_chunk_rows; q++) {
-    int4* row = &out->copies[q * (copies_max + 1)];
-    for (size_t k = 0; k < lists[q].size(); k++) row[k] = lists[q][k];
-    row[copies_max] = int4{(int32_t)lists[q].size(), used[q], 0, 0};
+  out->stage_bytes = stage_bytes;
+  out->copies.assign(lists.size() * (size_t)(out->copies_max + 1), int4{-1, 0, 0, 0});
+  for (size_t q = 0; q < lists.size(); q++) {
+    int4* row = &out->copies[q * (out->copies_max + 1)];
+    std::copy(lists[q].begin(), lists[q].end(), row);
+    row[out->copies_max] = heads[q];
   }
   return SPS_OK;
 }
@@ -243,8 +272,6 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
   const int32_t Di = cfg.warps_dm * cfg.dms_per_thread;
   const int32_t Tt = cfg.warps_time * 32 * cfg.samples_per_thread;
   const int32_t di_pad = presum_di_pad(cfg);
-  const int32_t cu = presum_chunk(cfg);
-  const int32_t n_chunks = (U + cu - 1) / cu;
   const int32_t n_tiles = (rows + Di - 1) / Di;
   auto say = [&](const char* what, int32_t tile, int32_t g, int32_t u, int32_t r) {
     *why = std::string(what) + " (tile " + std::to_string(tile) + ", group " + std::to_string(g) + ", unit " +
@@ -252,18 +279,29 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
     return false;
   };
   for (int32_t tile = 0; tile < n_tiles; tile++)
-    for (int32_t g = 0; g < G; g++)
+    for (int32_t g = 0; g < G; g++) {
+      const int4 chunks = t.chunk_rows[(size_t)tile * G + g];
+      int32_t chunk = 0, chunk_u0 = 0;  // the unit's chunk and the chunk's first unit
       for (int32_t u = 0; u < U; u++) {
         const int32_t c0 = g * per + K * u, n = std::min(K, per - K * u), e = c0 + n - 1;
-        const size_t row = ((size_t)tile * G + g) * n_chunks + u / cu;
-        const int4* list = &t.copies[row * (t.copies_max + 1)];
-        const int32_t count = list[t.copies_max].x;
+        const int4* list = &t.copies[((size_t)chunks.x + chunk) * (t.copies_max + 1)];
+        if (u - chunk_u0 == list[t.copies_max].z) {
+          chunk_u0 = u;
+          chunk++;
+          list += t.copies_max + 1;
+        }
+        if (chunk >= chunks.y) return say("unit in no chunk", tile, g, u, 0);
+        const int32_t count = list[t.copies_max].x, table = list[t.copies_max].z * 2 * di_pad;
+        const uint16_t* offs = &t.offs[(size_t)list[t.copies_max].w * 8 + (size_t)(u - chunk_u0) * di_pad];
+        int32_t sum = 0;
+        for (int32_t q = 0; q < count; q++) sum += ((uint32_t)list[q].z >> 16) * 16;
+        if (sum != list[t.copies_max].y) return say("window bytes of a chunk", tile, g, u, 0);
         for (int32_t r = 0; r < Di; r++) {
           const int32_t i = tile * Di + r;
           if (i >= rows) break;
           const int32_t* di = &d[(size_t)i * C];
           const int32_t de = di[e], dprime = de & ~1, parity = de & 1;
-          const int64_t off = 4 * (int64_t)t.offs[(((size_t)tile * G + g) * U + u) * di_pad + r];  // stage bytes
+          const int64_t off = 4 * (int64_t)offs[r];  // stage bytes
           int32_t q = 0;
           for (; q < count; q++) {
             const int32_t dst = (list[q].z & 0xFFFF) * 16, bytes = ((uint32_t)list[q].z >> 16) * 16;
@@ -271,7 +309,7 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
           }
           if (q == count) return say("offset outside every window of the chunk", tile, g, u, r);
           const int32_t dst = (list[q].z & 0xFFFF) * 16, bytes = ((uint32_t)list[q].z >> 16) * 16;
-          if (dst + bytes > t.data_bytes) return say("window beyond the stage data", tile, g, u, r);
+          if (dst < table || dst + bytes > t.stage_bytes) return say("window beyond the stage data", tile, g, u, r);
           const int32_t srow = list[q].x, s = srow / 2;
           if (srow < 0 || s >= (int32_t)t.series.size()) return say("window row outside the series table", tile, g, u, r);
           if (srow % 2 != parity) return say("window of the wrong alignment copy", tile, g, u, r);
@@ -284,6 +322,8 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
             return say("a valid output reads outside the series' written range", tile, g, u, r);
         }
       }
+      if (chunk + 1 != chunks.y) return say("chunk without units", tile, g, U, 0);
+    }
   return true;
 }
 

@@ -66,11 +66,12 @@ struct U8PassArgs {
 struct PresumPassArgs {
   const uint16_t* q;       // [n_series][2][q_pitch]: unit-sum series, second copy shifted by one
   int32_t q_pitch;         // samples per series row (N_in rounded up to 16)
-  const int4* copies;      // [tiles][groups][chunks][copies_max + 1]: {row, start,
-                           // (stage byte / 16) | (bytes / 16) << 16, 0}; last {count, total bytes}
+  const int4* chunk_rows;  // [tiles][groups]: {first chunk, chunks, 0, 0}
+  const int4* copies;      // [chunks][copies_max + 1]: {row, start, (stage byte / 16) |
+                           // (bytes / 16) << 16, 0}; last {count, total bytes, units, table / 8}
   int32_t copies_max;
-  int32_t data_bytes;      // bytes of series windows per stage (the table follows)
-  const uint16_t* offs;    // [tiles][groups][units][di_pad]: staged offsets in 4-byte words
+  int32_t stage_bytes;     // a stage: a chunk's offset table, then its series windows
+  const uint16_t* offs;    // per chunk [units][di_pad]: staged offsets in 4-byte words
   int32_t di_pad;
   int32_t n_dm;            // delay-table rows
   int32_t n_groups;
@@ -85,6 +86,13 @@ struct PresumPassArgs {
   uint32_t* status;
   int32_t window_bytes;    // staged bytes of one series window (the batched form reads it here)
 };
+
+// The wide register tile of the pre-summed pass, 8 trials x 7 words per thread:
+// its 16-bit lanes fold into 8-bit counts of kWideCount.
+constexpr bool presum_wide(int nd, int nw) { return nd == 8 && nw == 7; }
+constexpr uint32_t kWideCount = 4096;
+constexpr int32_t kWideChannels = 4096;        // sums of more channels pass 255 counts
+constexpr int32_t kWideStage = 36 * 1024;      // three stages: two blocks per SM
 
 // One pre-summed series: channels c0 .. c0 + n - 1, channel c0 + j (j < n - 1)
 // taken rel[j] samples later than the last one.
@@ -106,10 +114,11 @@ struct PresumTables {
   std::vector<PresumSeries> series;
   std::vector<PresumUnit> units;
   int32_t max_rel = 0;
+  std::vector<int4> chunk_rows;
   std::vector<int4> copies;
   std::vector<uint16_t> offs;
   int32_t copies_max = 0;
-  int32_t data_bytes = 0;
+  int32_t stage_bytes = 0;
 };
 
 // Step two over uint16 subband series.
@@ -160,20 +169,22 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
                                 int32_t n_series, uint16_t* q, int32_t q_pitch, cudaStream_t st);
 sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& cfg, cudaStream_t st);
 // Batched pre-summed pass: one launch over the work list of several passes of
-// configuration `cfg` (d_passes / d_work in device memory; max_data_bytes =
-// the largest data_bytes of the passes).  presum_pass_work appends the work
+// configuration `cfg` (d_passes / d_work in device memory; max_stage_bytes =
+// the largest stage_bytes of the passes).  presum_pass_work appends the work
 // items of pass index `pass`; presum_pass_blocks counts them.
 sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d_work, int64_t n_work,
-                                   const sps_dedisp_config& cfg, int32_t max_data_bytes, cudaStream_t st);
+                                   const sps_dedisp_config& cfg, int32_t max_stage_bytes, cudaStream_t st);
 void presum_pass_work(const PresumPassArgs& a, const sps_dedisp_config& cfg, int32_t pass, std::vector<int4>* work);
 int64_t presum_pass_blocks(const PresumPassArgs& a, const sps_dedisp_config& cfg);
 sps_status launch_zap_copy(const uint8_t* x, int64_t pitch, int32_t in_len, const uint8_t* zap, int32_t channels,
                            uint8_t* out, int64_t out_pitch, cudaStream_t st);
 bool presum_config_supported(const sps_dedisp_config& cfg, std::string* why);
-size_t presum_smem_bytes(const sps_dedisp_config& cfg, int32_t data_bytes);
+size_t presum_smem_bytes(int32_t stage_bytes);
 int presum_window_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile);
 int presum_di_pad(const sps_dedisp_config& cfg);
-int presum_chunk(const sps_dedisp_config& cfg);  // units staged per chunk
+int presum_chunk(const sps_dedisp_config& cfg);  // units a stage is sized for
+int presum_fold_units(const sps_dedisp_config& cfg);  // units a 16-bit lane sums between folds
+constexpr int32_t kPresumChunkUnits = 16;             // most units per chunk
 // Host tables (presum_tables.cpp): series count over all rows, the largest
 // packed window data of any (tile, group, chunk), and the full tables of one
 // configuration.
@@ -181,7 +192,7 @@ int64_t count_presum_series(const std::vector<int32_t>& d, int32_t rows, int32_t
 int32_t presum_stage_data(const std::vector<int32_t>& d, int32_t rows, int32_t C, int32_t per, int32_t K, int32_t Di,
                           int32_t units_per_chunk, int32_t Tt);
 sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C, int32_t per, int32_t n_out,
-                               const sps_dedisp_config& cfg, PresumTables* out);
+                               const sps_dedisp_config& cfg, int32_t stage_bytes, PresumTables* out);
 bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C, int32_t per, int32_t read_n_out,
                           const sps_dedisp_config& cfg, const PresumTables& t, std::string* why);
 bool u8_config_supported(const sps_dedisp_config& cfg, std::string* why);
@@ -203,6 +214,7 @@ struct ConfigCheck {
 };
 sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigCheck* out);
 sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg);
+bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* wide);
 sps_status run_search(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws, size_t ws_bytes,
                       double* snr, int32_t* peak_t, int32_t* peak_val, int32_t* best, cudaStream_t st);
 sps_status dedisperse_into(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
@@ -263,19 +275,24 @@ struct sps_plan {
   sps::PresumUnit* d_presum_units = nullptr;
   int32_t n_presum_units = 0;
   int32_t presum_max_rel = 0;
+  int4* d_presum_chunks = nullptr;
   int4* d_presum_copies = nullptr;
   uint16_t* d_presum_offs = nullptr;
   int32_t n_presum_series = 0;   // of the current configuration's table
   int32_t presum_copies_max = 0;
-  int32_t presum_data_bytes = 0;
+  int32_t presum_stage_bytes = 0;
   int32_t q_pitch = 0;           // samples per series row
   int64_t max_presum_series = 0; // over presum 1 and 2 (sizes the workspace)
 
   int max_smem = 0;              // opt-in shared memory per block of the device
+  int sms = 0;                   // multiprocessors of the device
   mutable std::map<int64_t, int32_t> spread_cache;     // tile delay spread by (table, rows)
   mutable std::map<int64_t, int32_t> presum_stage_cache;  // stage data by (table, K, rows, units, samples)
 
   sps_kernel_config cfg{};
+  // the tile the brute-force pass runs with: cfg.brute, or the one the library
+  // picks for the default pre-summed tile (presum_tile in plan.cpp)
+  sps_dedisp_config brute_tile{};
   uint64_t config_gen = 0;       // bumped whenever the device tables are rebuilt
   // delay spread of one DM tile for the current configuration
   int32_t dmax_brute = 0, dmax_step1 = 0, dmax_step2 = 0;

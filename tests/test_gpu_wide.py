@@ -1,0 +1,35 @@
+"""The wide tile of the pre-summed pass (it takes the default tile's place on
+plans whose blocks fill the GPU): every row equal to the single-channel kernel's
+on the same plan, at the edges of its tile (64 trials x 448 samples, chunks cut
+by window size, an odd last unit) and of its 8-bit counts."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+# channels, samples, trials, DM step, saturated input
+CASES = [(41, 12501, 700, 0.05, False),    # 11 units, the last a single channel; rows of odd length
+         (389, 7013, 577, 0.31, False),    # one trial past a tile, 293 samples in the last
+         (384, 4480, 2048, 0.3, True),     # every lane at its bound, whole tiles only
+         (4096, 1793, 2500, 0.02, True),   # the most channels: 255 counts
+         (1536, 449, 11000, 0.02, False)]  # one sample in the last time tile
+
+
+@pytest.mark.parametrize("C,n_t,n_dms,step,full", CASES)
+def test_wide_tile_equals_single_channel_kernel(lib, C, n_t, n_dms, step, full):
+    import torch
+    plan = lib.Plan(C, 1250.0, 1550.0, 81.92e-6, n_t, step * np.arange(n_dms), [1])
+    assert plan.config.brute.presum == 2
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    x = torch.randint(255 if full else 0, 256, (C, plan.pitch), dtype=torch.uint8, device="cuda", generator=gen)
+    got = torch.full((n_dms, n_t), -1, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, got)
+    cfg = plan.config
+    cfg.brute = lib.DedispConfig(4, 16, 8, 1, 4, 0)
+    plan.config = cfg
+    want = torch.full((n_dms, n_t), -2, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, want)
+    assert plan.status() == 0
+    assert torch.equal(got, want)
+    if full:
+        assert int(got[0, 0]) == 255 * C
