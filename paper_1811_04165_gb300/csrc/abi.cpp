@@ -103,11 +103,15 @@ U8PassArgs u8_args(const sps_plan* p, const uint8_t* x, int64_t pitch, const uin
 // the pass that reads them.
 sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const uint8_t* x, int64_t pitch,
                           uint8_t* ws, int32_t rows, int32_t per, int32_t n_out, int64_t out_pitch, int32_t dmax,
-                          void* out, int32_t out_u16, cudaStream_t st, PresumPassArgs* args) {
+                          void* out, int32_t out_u16, int32_t splits, cudaStream_t st, PresumPassArgs* args) {
   uint16_t* q = reinterpret_cast<uint16_t*>(ws);
   const int32_t K = 1 << cfg.presum;
+  // split sums are added into zeroed rows
+  const bool split = splits > 1;
   sps_status s = launch_presum_series(x, pitch, (int32_t)p->n_in, p->d_presum_units, p->n_presum_units, K,
-                                      p->presum_max_rel, p->d_presum_series, p->n_presum_series, q, p->q_pitch, st);
+                                      p->presum_max_rel, p->d_presum_series, p->n_presum_series, q, p->q_pitch,
+                                      split ? static_cast<int32_t*>(out) : nullptr, split ? (int64_t)rows * out_pitch : 0,
+                                      st);
   if (s) return s;
   PresumPassArgs& a = *args;
   a = PresumPassArgs{};
@@ -119,6 +123,7 @@ sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const
   a.chunk_rows = p->d_presum_chunks;
   a.offs = p->d_presum_offs;
   a.di_pad = presum_di_pad(cfg);
+  a.splits = splits;
   a.n_dm = rows;
   a.n_groups = p->channels / per;
   a.group_units = (per + K - 1) / K;
@@ -140,7 +145,8 @@ sps_status run_u8_pass(const sps_plan* p, const sps_dedisp_config& cfg, const ui
                        void* out, int32_t out_u16, cudaStream_t st) {
   if (cfg.presum) {
     PresumPassArgs a{};
-    sps_status s = presum_prepass(p, cfg, x, pitch, ws, rows, per, n_out, out_pitch, dmax, out, out_u16, st, &a);
+    sps_status s = presum_prepass(p, cfg, x, pitch, ws, rows, per, n_out, out_pitch, dmax, out, out_u16,
+                                  out_u16 ? 1 : p->brute_splits, st, &a);
     if (s) return s;
     return launch_presum_pass(a, cfg, st);
   }
@@ -255,7 +261,7 @@ sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int
   uint8_t* w = static_cast<uint8_t*>(ws);
   if ((s = prepare_input(p, &x, &pitch, &w, st))) return s;
   return presum_prepass(p, p->brute_tile, x, pitch, w, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
-                        p->dmax_brute, D, 0, st, args);
+                        p->dmax_brute, D, 0, 1, st, args);
 }
 
 sps_status snr_into(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,
@@ -459,7 +465,12 @@ sps_status sps_presum_tables_verify(const int32_t* delays, int32_t rows, int32_t
   };
   if (sps_status s = check(*cfg, presum_chunk(*cfg), 0)) return s;
   sps_dedisp_config wide;
-  return per == channels && wide_form(*cfg, channels, &wide) ? check(wide, 1, kWideStage) : SPS_OK;
+  if (per != channels || !wide_form(*cfg, channels, &wide)) return SPS_OK;
+  for (int32_t warps : {8, 4}) {
+    wide.warps_dm = warps;
+    if (sps_status s = check(wide, 1, presum_wide_stage(wide))) return s;
+  }
+  return SPS_OK;
 }
 
 sps_status sps_plan_status(const sps_plan* p, uint32_t* host_status, int32_t clear) {

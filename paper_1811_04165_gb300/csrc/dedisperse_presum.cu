@@ -90,7 +90,7 @@ __device__ __forceinline__ void load_offs(const uint16_t* p, uint32_t (&o)[ND]) 
 // One block's tile: DM tile `tile`, time tile `ty`, group `g` of the pass `a`.
 // WIDE: 8-bit counts instead of int32 sums (see the top of the file).
 template <int ND, int NW, bool WIDE>
-__device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int tile, int ty, int g, int wd,
+__device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int tile, int ty, int g, int split, int wd,
                                                   int wb) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int wt = (int)(blockDim.x >> 5) / wd;
@@ -109,8 +109,11 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   const int dm_sub = warp % wd, t_sub = warp / wd;
   const int i0 = tile * Di;
   const int t0 = ty * Tt;
-  const int4 chunks = __ldg(&a.chunk_rows[(int64_t)tile * a.n_groups + g]);
-  const int n_chunks = chunks.y;
+  int4 chunks = __ldg(&a.chunk_rows[(int64_t)tile * a.n_groups + g]);
+  // the block's share of the chunks
+  const int c_lo = chunks.y * split / a.splits, c_hi = chunks.y * (split + 1) / a.splits;
+  chunks.x += c_lo;
+  const int n_chunks = c_hi - c_lo;
   const uint32_t toff = (uint32_t)(t_sub * 128 * NW + lane * 4);  // bytes
   const bool clip = t0 + wb / 2 + a.max_start > a.q_pitch;  // windows may be cut at the row end
   // bounds-checked build: the largest staged offset whose NW words fit the
@@ -364,7 +367,10 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
         }
       } else {
         int32_t* o = static_cast<int32_t*>(a.out) + row * a.out_pitch + t;
-        if (t + 1 < a.n_out && vec) {
+        if (a.splits > 1) {  // the splits' sums meet in the zeroed rows
+          atomicAdd(o, s0);
+          if (t + 1 < a.n_out) atomicAdd(o + 1, s1);
+        } else if (t + 1 < a.n_out && vec) {
           *reinterpret_cast<int2*>(o) = make_int2(s0, s1);
         } else {
           o[0] = s0;
@@ -378,7 +384,8 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
 template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 presum_pass_kernel(PresumPassArgs a, int wd, int wb) {
-  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, blockIdx.x, blockIdx.y, blockIdx.z, wd, wb);
+  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, blockIdx.x, blockIdx.y, blockIdx.z / a.splits, blockIdx.z % a.splits, wd,
+                                               wb);
 }
 
 // Batched form: one launch over a work list of tiles from several passes of
@@ -389,7 +396,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* __restrict__ work, int wd) {
   const int4 w = work[blockIdx.x];
   const PresumPassArgs& a = passes[w.x];
-  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, w.w, wd, a.window_bytes);
+  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, w.w, 0, wd, a.window_bytes);
 }
 
 // Adds bytes o + j .. o + j + 15 of W (24 bytes, o in 0 .. 7), for j = 0 and
@@ -484,6 +491,15 @@ __device__ __forceinline__ void load_row24(const uint8_t* row, int u, int in_len
   }
 }
 
+// The blocks' shares of `n` words of zeros (16-byte aligned).
+__device__ __forceinline__ void zero_share(int32_t* zero, int64_t n) {
+  if (n == 0) return;
+  const int64_t blocks = (int64_t)gridDim.x * gridDim.y;
+  const int64_t id = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+  for (int64_t k = id; k < n / 4; k += blocks * blockDim.x) reinterpret_cast<int4*>(zero)[k] = make_int4(0, 0, 0, 0);
+  if (id < n % 4) zero[n / 4 * 4 + id] = 0;
+}
+
 constexpr int kSeriesThreads = 128;
 constexpr int kSeriesBlock = kSeriesThreads * 16;  // samples per block
 
@@ -508,11 +524,13 @@ __device__ __forceinline__ void store_series(uint16_t* q, int64_t q_pitch, int s
 __global__ void __launch_bounds__(kSeriesThreads) presum_series_kernel(const uint8_t* x, int64_t pitch,
                                                                        int32_t in_len, const PresumUnit* units,
                                                                        const PresumSeries* series, uint16_t* q,
-                                                                       int32_t q_pitch, int32_t win_bytes) {
+                                                                       int32_t q_pitch, int32_t win_bytes,
+                                                                       int32_t* zero, int64_t n_zero) {
   extern __shared__ __align__(16) uint8_t win[];
   const int4 uh = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x));      // {c0, n, s_begin, s_end}
   const int4 ur = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x) + 1);  // {max_rel, lo, hi, 0}
   const int ub = blockIdx.y * kSeriesBlock;
+  zero_share(zero, n_zero);
   if (ub >= ur.z || ub + kSeriesBlock <= ur.y) return;  // no series of the unit needs these samples
   // asynchronous 16-byte copies (all in flight at once); bytes at and beyond
   // in_len are zero-filled and never read
@@ -573,7 +591,8 @@ __global__ void __launch_bounds__(kSeriesThreads) presum_series_kernel(const uin
 __global__ void __launch_bounds__(256) presum_series_direct_kernel(const uint8_t* x, int64_t pitch,
                                                                    int32_t in_len, const PresumSeries* series,
                                                                    int32_t n_series, uint16_t* q,
-                                                                   int32_t q_pitch) {
+                                                                   int32_t q_pitch, int32_t* zero, int64_t n_zero) {
+  zero_share(zero, n_zero);
   const int64_t per_row = q_pitch >> 4;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= per_row * n_series) return;
@@ -665,11 +684,15 @@ int presum_fold_units(const sps_dedisp_config& c) {
   return room / (255 << c.presum);
 }
 
+// Three stages of this let 16 warps' blocks share an SM.
+int32_t presum_wide_stage(const sps_dedisp_config& c) { return c.warps_dm * c.warps_time * 4608; }
+
 size_t presum_smem_bytes(int32_t stage_bytes) { return kStages * (size_t)stage_bytes + 16 * kStages; }
 
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
                                 int32_t n_units, int32_t unit_channels, int32_t max_rel, const PresumSeries* series,
-                                int32_t n_series, uint16_t* q, int32_t q_pitch, cudaStream_t st) {
+                                int32_t n_series, uint16_t* q, int32_t q_pitch, int32_t* zero, int64_t n_zero,
+                                cudaStream_t st) {
   if (n_series == 0) return SPS_OK;
   // staged window per channel row: the block's samples, the largest relative
   // delay, and the 16-byte reach of the last thread's loads
@@ -679,11 +702,11 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
     SPS_CUDA(cudaFuncSetAttribute(presum_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((unsigned)n_units, (unsigned)((q_pitch + kSeriesBlock - 1) / kSeriesBlock));
     presum_series_kernel<<<grid, kSeriesThreads, (size_t)smem, st>>>(x, pitch, in_len, units, series, q, q_pitch,
-                                                                    (int32_t)win);
+                                                                    (int32_t)win, zero, n_zero);
   } else {
     const int64_t threads = (int64_t)(q_pitch >> 4) * n_series;
     presum_series_direct_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(x, pitch, in_len, series,
-                                                                                   n_series, q, q_pitch);
+                                                                                   n_series, q, q_pitch, zero, n_zero);
   }
   SPS_CUDA(cudaGetLastError());
   return SPS_OK;
@@ -695,7 +718,7 @@ sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& 
   const int Di = c.warps_dm * c.dms_per_thread;
   const int Tt = c.warps_time * 32 * c.samples_per_thread;
   const size_t smem = presum_smem_bytes(a.stage_bytes);
-  dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, a.n_groups);
+  dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, a.n_groups * a.splits);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
   SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, presum_window_bytes(c, a.dmax_tile));

@@ -218,31 +218,62 @@ bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* 
          c.warps_time == 1 && c.chunk == 16 && channels <= kWideChannels;
 }
 
-// The tile the brute-force pass runs with.  The default pre-summed tile leaves
-// the choice to the library: the wide tile (64 trials x 448 samples per block, 8
-// trials x 7 words per thread, two blocks per SM) reads shared memory at 81 % of
-// its peak and half the series windows per output, so it takes over once its
-// larger blocks fill the GPU as well as the default's.  Cycles per unit of a
-// round of resident blocks, measured on the 1536-channel band (0.2 pc cm^-3 per
-// trial): wide 1020 with two blocks per SM and 775 with one, default 750 and
-// 585; 2048 trials of 12500 samples take 597 us against 800.
-sps_dedisp_config presum_tile(const sps_plan* p, const sps_dedisp_config& c) {
-  sps_dedisp_config wide;
-  if (!wide_form(c, p->channels, &wide)) return c;
-  auto cost = [&](const sps_dedisp_config& t, int64_t two, int64_t one) {
+// The tile and the channel splits the brute-force pass runs with, by a model of
+// its time.
+//   * The default pre-summed tile leaves the choice to the library.  The wide
+//     tiles (8 trials x 7 words per thread; 8 or 4 warps, each 8 trials x 448
+//     samples) read shared memory at 81 % of its peak and half the series windows
+//     per output; they are taken where single units fit their stages.  The one of
+//     4 warps serves plans of few trials, whose tiles it fills better.
+//   * A grid that leaves SMs idle, in its last round or altogether, is split
+//     along the channels: each split's blocks add their sums into zeroed rows.
+// Constants measured on the 1536-channel band, in ns: a unit takes a round of
+// resident blocks 500 (380 with at most half the SM's blocks), with the default
+// tile 370 (290); a block starts and ends in 2000; a split costs 0.24 per KB of
+// output (its additions reach the L2 at 4.3 TB/s).  64 trials x 12500 samples:
+// 140 us with the default tile, 160 wide, 59 wide in eight splits; 512 trials
+// (0.4 pc cm^-3 apart): 415, 266 and, in four splits, 237.
+void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_config* tile, int32_t* splits) {
+  *tile = c;
+  *splits = 1;
+  if (p->mode != SPS_MODE_BRUTE || !c.presum) return;
+  const int64_t rows = (int64_t)p->dms.size(), units = (p->channels + (1 << c.presum) - 1) >> c.presum;
+  const double out_kb = 4e-3 * rows * p->n_t;
+  double best = 1e30;
+  auto consider = [&](const sps_dedisp_config& t, int64_t per_sm, double full, double half) {
     const int64_t di = t.warps_dm * t.dms_per_thread, tt = 32 * t.warps_time * t.samples_per_thread;
-    const int64_t blocks = ((int64_t)p->dms.size() + di - 1) / di * ((p->n_t + tt - 1) / tt);
-    const int64_t last = blocks % (2 * p->sms);
-    return blocks / (2 * p->sms) * two + (last > p->sms ? two : (last ? one : 0));
+    const int64_t blocks = (rows + di - 1) / di * ((p->n_t + tt - 1) / tt), slots = per_sm * p->sms;
+    for (int32_t s : {1, 2, 3, 4, 6, 8, 12, 16}) {
+      if (s > 1 && s > units / 8) break;
+      const int64_t whole = blocks * s / slots, last = blocks * s % slots;
+      double ns = whole * (units * full / s + 2000);
+      if (last) ns += units * (last > slots / 2 ? full : half) / s + 2000;
+      if (s > 1) ns += 0.24 * (s + 1) * out_kb;
+      if (ns < best) {
+        best = ns;
+        *tile = t;
+        *splits = s;
+      }
+    }
   };
-  if (cost(wide, 1020, 775) >= cost(c, 750, 585)) return c;
-  sps_dedisp_config unit = wide;  // sized for single units: the largest unit's stage
-  unit.chunk = 4;
-  return cached_presum_stage(p, 0, unit) <= kWideStage ? wide : c;
+  sps_dedisp_config wide;
+  if (wide_form(c, p->channels, &wide)) {
+    for (int32_t warps : {8, 4}) {
+      wide.warps_dm = warps;
+      wide.chunk = 4;  // single units, for the stage check
+      if (cached_presum_stage(p, 0, wide) > presum_wide_stage(wide)) continue;
+      wide.chunk = c.chunk;
+      consider(wide, 16 / warps, 500, 380);
+    }
+    if (best < 1e30) return;
+  }
+  const size_t per_sm = p->smem_per_sm / (presum_smem_bytes(cached_presum_stage(p, 0, c)) + 1024);
+  const int64_t warps = c.warps_dm * c.warps_time;
+  consider(c, std::max<int64_t>(1, std::min<int64_t>(16 / warps, (int64_t)per_sm)), 370, 290);
 }
 
 int32_t presum_stage(const sps_plan* p, const sps_dedisp_config& c) {
-  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return kWideStage;
+  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return presum_wide_stage(c);
   return cached_presum_stage(p, p->mode == SPS_MODE_BRUTE ? 0 : 1, c);
 }
 
@@ -251,7 +282,9 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   ConfigCheck chk;
   if (sps_status s = check_config(p, cfg, &chk)) return s;
   const int32_t n_dms = (int32_t)p->dms.size();
-  const sps_dedisp_config tile = p->mode == SPS_MODE_BRUTE ? presum_tile(p, cfg.brute) : cfg.brute;
+  sps_dedisp_config tile;
+  int32_t splits = 1;
+  choose_tile(p, cfg.brute, &tile, &splits);
   const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : cfg.step1;
   const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0, dmax_1 = chk.dmax_1, dmax_2 = chk.dmax_2;
   const std::vector<int32_t>& tiles = chk.tiles;
@@ -327,6 +360,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   }
   p->cfg = cfg;
   p->brute_tile = tile;
+  p->brute_splits = splits;
   p->config_gen++;
   p->dmax_brute = dmax_b;
   p->dmax_step1 = dmax_1;
@@ -452,9 +486,10 @@ sps_status plan_create(const sps_plan_desc* d, sps_plan** out) {
                                         ? count_presum_series(p->delays, n_dms, C, C, K)
                                         : count_presum_series(p->d1, d->n_coarse, C, C / d->n_subbands, K));
   if (cudaDeviceGetAttribute(&p->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&p->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, p->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     delete p;
-    return fail(SPS_ERR_CUDA, "cudaDeviceGetAttribute(max shared memory, multiprocessors)");
+    return fail(SPS_ERR_CUDA, "cudaDeviceGetAttribute(shared memory, multiprocessors)");
   }
   if (p->n_in > INT32_MAX / 2) { delete p; return fail(SPS_ERR_UNSUPPORTED, "input rows too long"); }
   int64_t max_sum = (int64_t)255 * C * p->widths.back();

@@ -77,6 +77,7 @@ struct PresumPassArgs {
   int32_t n_groups;
   int32_t group_units;     // units per group
   int32_t fold_units;      // units a 16-bit lane sums exactly: 65535 / (255 K)
+  int32_t splits;          // blocks per output tile, each summing a share of its chunks (int32 rows, zeroed before)
   int32_t max_start;       // bound on any staged window's start (the pass's largest delay)
   int32_t n_out;
   int64_t out_pitch;
@@ -92,7 +93,6 @@ struct PresumPassArgs {
 constexpr bool presum_wide(int nd, int nw) { return nd == 8 && nw == 7; }
 constexpr uint32_t kWideCount = 4096;
 constexpr int32_t kWideChannels = 4096;        // sums of more channels pass 255 counts
-constexpr int32_t kWideStage = 36 * 1024;      // three stages: two blocks per SM
 
 // One pre-summed series: channels c0 .. c0 + n - 1, channel c0 + j (j < n - 1)
 // taken rel[j] samples later than the last one.
@@ -166,7 +166,8 @@ sps_status launch_expand(const uint8_t* x, int64_t pitch, int32_t in_len, int32_
                          int64_t pitch4, cudaStream_t st);
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
                                 int32_t n_units, int32_t unit_channels, int32_t max_rel, const PresumSeries* series,
-                                int32_t n_series, uint16_t* q, int32_t q_pitch, cudaStream_t st);
+                                int32_t n_series, uint16_t* q, int32_t q_pitch, int32_t* zero, int64_t n_zero,
+                                cudaStream_t st);
 sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& cfg, cudaStream_t st);
 // Batched pre-summed pass: one launch over the work list of several passes of
 // configuration `cfg` (d_passes / d_work in device memory; max_stage_bytes =
@@ -183,6 +184,7 @@ size_t presum_smem_bytes(int32_t stage_bytes);
 int presum_window_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile);
 int presum_di_pad(const sps_dedisp_config& cfg);
 int presum_chunk(const sps_dedisp_config& cfg);  // units a stage is sized for
+int32_t presum_wide_stage(const sps_dedisp_config& cfg);  // bytes of a wide tile's stage
 int presum_fold_units(const sps_dedisp_config& cfg);  // units a 16-bit lane sums between folds
 constexpr int32_t kPresumChunkUnits = 16;             // most units per chunk
 // Host tables (presum_tables.cpp): series count over all rows, the largest
@@ -285,6 +287,7 @@ struct sps_plan {
   int64_t max_presum_series = 0; // over presum 1 and 2 (sizes the workspace)
 
   int max_smem = 0;              // opt-in shared memory per block of the device
+  int smem_per_sm = 0;
   int sms = 0;                   // multiprocessors of the device
   mutable std::map<int64_t, int32_t> spread_cache;     // tile delay spread by (table, rows)
   mutable std::map<int64_t, int32_t> presum_stage_cache;  // stage data by (table, K, rows, units, samples)
@@ -293,6 +296,7 @@ struct sps_plan {
   // the tile the brute-force pass runs with: cfg.brute, or the one the library
   // picks for the default pre-summed tile (presum_tile in plan.cpp)
   sps_dedisp_config brute_tile{};
+  int32_t brute_splits = 1;      // shares of the channels that blocks of their own sum
   uint64_t config_gen = 0;       // bumped whenever the device tables are rebuilt
   // delay spread of one DM tile for the current configuration
   int32_t dmax_brute = 0, dmax_step1 = 0, dmax_step2 = 0;

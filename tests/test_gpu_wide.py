@@ -1,7 +1,8 @@
-"""The wide tile of the pre-summed pass (it takes the default tile's place on
-plans whose blocks fill the GPU): every row equal to the single-channel kernel's
-on the same plan, at the edges of its tile (64 trials x 448 samples, chunks cut
-by window size, an odd last unit) and of its 8-bit counts."""
+"""The wide tiles of the pre-summed pass, which take the default tile's place, and
+the channel splits of small grids: every row equal to the single-channel
+kernel's on the same plan, at the edges of the tiles (64 or 32 trials x 448
+samples, chunks cut by window size, an odd last unit), of the 8-bit counts and of
+the splits (added into rows that held other values)."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,11 @@ CASES = [(41, 12501, 700, 0.05, False),    # 11 units, the last a single channel
          (389, 7013, 577, 0.31, False),    # one trial past a tile, 293 samples in the last
          (384, 4480, 2048, 0.3, True),     # every lane at its bound, whole tiles only
          (4096, 1793, 2500, 0.02, True),   # the most channels: 255 counts
-         (1536, 449, 11000, 0.02, False)]  # one sample in the last time tile
+         (1536, 449, 11000, 0.02, False),  # one sample in the last time tile
+         (1536, 3001, 16, 0.2, True),      # the 32-trial tile in sixteen splits, rows of odd length
+         (389, 1003, 65, 0.2, False),      # splits with one trial in the last tile
+         (1537, 450, 200, 0.3, False),     # an odd last unit in the last split
+         (5000, 1201, 40, 0.05, True)]     # more channels than the counts hold: the default tile, split
 
 
 @pytest.mark.parametrize("C,n_t,n_dms,step,full", CASES)
