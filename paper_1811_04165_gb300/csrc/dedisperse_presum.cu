@@ -530,8 +530,11 @@ __global__ void __launch_bounds__(kSeriesThreads) presum_series_kernel(const uin
   const int4 uh = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x));      // {c0, n, s_begin, s_end}
   const int4 ur = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x) + 1);  // {max_rel, lo, hi, 0}
   const int ub = blockIdx.y * kSeriesBlock;
-  zero_share(zero, n_zero);
+  if (blockIdx.z == 0) zero_share(zero, n_zero);
   if (ub >= ur.z || ub + kSeriesBlock <= ur.y) return;  // no series of the unit needs these samples
+  // the block's share of the unit's series
+  const int s_lo = uh.z + (uh.w - uh.z) * (int)blockIdx.z / (int)gridDim.z;
+  const int s_hi = uh.z + (uh.w - uh.z) * ((int)blockIdx.z + 1) / (int)gridDim.z;
   // asynchronous 16-byte copies (all in flight at once); bytes at and beyond
   // in_len are zero-filled and never read
   for (int c = 0; c < uh.y; c++) {
@@ -551,13 +554,13 @@ __global__ void __launch_bounds__(kSeriesThreads) presum_series_kernel(const uin
   const int u0 = ub + l0, u1 = ub + l1;
   // each series' header {c0, n, rel0, rel1}, {rel2, lo, hi, 0} is fetched one series ahead
   int4 hn = make_int4(0, 0, 0, 0), rn = make_int4(0, 0, 0, 0);
-  if (uh.z < uh.w) {
-    hn = __ldg(reinterpret_cast<const int4*>(series + uh.z));
-    rn = __ldg(reinterpret_cast<const int4*>(series + uh.z) + 1);
+  if (s_lo < s_hi) {
+    hn = __ldg(reinterpret_cast<const int4*>(series + s_lo));
+    rn = __ldg(reinterpret_cast<const int4*>(series + s_lo) + 1);
   }
-  for (int s = uh.z; s < uh.w; s++) {
+  for (int s = s_lo; s < s_hi; s++) {
     const int4 h = hn, r = rn;
-    if (s + 1 < uh.w) {
+    if (s + 1 < s_hi) {
       hn = __ldg(reinterpret_cast<const int4*>(series + s + 1));
       rn = __ldg(reinterpret_cast<const int4*>(series + s + 1) + 1);
     }
@@ -700,7 +703,13 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
   const int64_t smem = win * unit_channels;
   if (smem <= 96 * 1024) {
     SPS_CUDA(cudaFuncSetAttribute(presum_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // Bands of few units have many series each: blocks take shares of a unit's
+    // series (each stages the rows anew) until the grid has 16 blocks per SM.
+    // 384 channels x 1024 trials (64 series per unit, 768 blocks): the call 203 ->
+    // 197 us; 200 channels x 512 trials: 112 -> 87; more blocks gain no more.
     dim3 grid((unsigned)n_units, (unsigned)((q_pitch + kSeriesBlock - 1) / kSeriesBlock));
+    const int64_t blocks = (int64_t)grid.x * grid.y;
+    grid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_series / (4 * n_units), (16 * 152 + blocks - 1) / blocks));
     presum_series_kernel<<<grid, kSeriesThreads, (size_t)smem, st>>>(x, pitch, in_len, units, series, q, q_pitch,
                                                                     (int32_t)win, zero, n_zero);
   } else {
