@@ -22,9 +22,9 @@
 // 64 quads); partial sums fold into int32 registers that often.  A group whose
 // size is not a multiple of K ends in a shorter unit.
 //
-// The wide tile (8 trials x 7 words per thread) keeps no int32 sums: a fold moves
-// the lanes' multiples of 4096 into 8-bit counts, four to a register, so a thread
-// holds 112 outputs in 84 registers where int32 sums take 192.  It is bound by
+// The wide tile (8 trials x 7 words per thread) keeps no int32 sums but 8-bit
+// counts (wide_tile.cuh), so a thread holds 112 outputs in 84 registers where
+// int32 sums take 192.  It is bound by
 // the shared-memory loads: with 64 trials x 448 samples per block the windows
 // staged per output (L2 -> shared, which alone took 0.6 ms of a 2048-trial pass
 // with 32 x 512 tiles) fall by 40 %, and loads run at 81 % of the LSU peak.  On
@@ -34,33 +34,13 @@
 
 #include "sps_internal.h"
 #include "tma.cuh"
+#include "wide_tile.cuh"
 
 namespace sps {
 namespace {
 
 constexpr int kMaxThreads = 512;
 constexpr int kStages = 3;  // shared-memory ring depth
-
-// NW words at shared address addr + 128 * m (immediate offsets).
-template <int NW, int M = 0>
-__device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
-  if constexpr (M < NW) {
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(w[M]) : "r"(addr), "n"(M * 128));
-    lds_row<NW, M + 1>(addr, w);
-  }
-}
-
-// The same into `w` only where `load` is set (uniform over the warp); otherwise
-// `w` keeps its words.
-template <int NW, int M = 0>
-__device__ __forceinline__ void lds_row_if(bool load, uint32_t addr, uint32_t (&w)[NW]) {
-  if constexpr (M < NW) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.shared.u32 %0, [%1+%3];\n\t}"
-                 : "+r"(w[M])
-                 : "r"(addr), "r"((uint32_t)load), "n"(M * 128));
-    lds_row_if<NW, M + 1>(load, addr, w);
-  }
-}
 
 // The staged offsets of one unit for a warp's ND trials (uint16 words, one
 // vector load), as byte offsets.
@@ -218,15 +198,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   }
   auto fold = [&]() {
     if constexpr (WIDE) {
-      // the lanes' multiples of kWideCount move to the counts
-#pragma unroll
-      for (int k = 0; k < ND * NW / 2; k++) {
-        uint32_t& x = lanes[2 * k / NW][2 * k % NW];
-        uint32_t& y = lanes[(2 * k + 1) / NW][(2 * k + 1) % NW];
-        cnt[k] += ((x >> 12) & 0x000F000Fu) + (((y >> 12) & 0x000F000Fu) << 8);
-        x &= 0x0FFF0FFFu;
-        y &= 0x0FFF0FFFu;
-      }
+      wide_fold<ND, NW>(lanes, cnt);
       return;
     } else {
 #pragma unroll
@@ -350,9 +322,9 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
       if (t >= a.n_out) continue;
       int32_t s0, s1;
       if constexpr (WIDE) {
-        const uint32_t c = cnt[(r * NW + m) / 2] >> (8 * ((r * NW + m) & 1));
-        s0 = (int32_t)((lanes[r][m] & 0xFFFFu) + (c & 0xFFu) * kWideCount);
-        s1 = (int32_t)((lanes[r][m] >> 16) + ((c >> 16) & 0xFFu) * kWideCount);
+        const int2 v = wide_sum<ND, NW>(lanes, cnt, r, m);
+        s0 = v.x;
+        s1 = v.y;
       } else {
         s0 = acc[r][m][0];
         s1 = acc[r][m][1];

@@ -20,11 +20,13 @@
 
 #include "sps_internal.h"
 #include "tma.cuh"
+#include "wide_tile.cuh"
 
 namespace sps {
 namespace {
 
 constexpr int kMaxThreads = 512;
+constexpr int kWideStages = 2;  // ring of the wide form (three and four stages measured no faster)
 
 template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
@@ -177,6 +179,184 @@ step2_kernel(Step2Args a, int wd, int cs_max, int wb) {
   }
 }
 
+// The wide tile (wide_tile.cuh): a warp takes 8 trials x 448 samples, a block wd
+// warps along DM by wt along time.  As above, with one barrier per chunk; the
+// staged offsets are 16-bit words [subband][trial], so that one vector load gives
+// a warp's eight; two subbands are added at a time; a trial that reads the words
+// of the trial before it keeps them (29 % of the reads at 0.2 pc cm^-3 per trial
+// and 32 subbands).  Bound by the shared loads (42 us of the LSU pipe at 64 x 32
+// trials of 12500 samples and 32 subbands, less the words kept) and by each
+// block's start and end (its offsets, the first copies, 115 KB of rows): 83 us
+// there, 97 with the tile above; eight subbands per chunk, 93 us with four.
+__global__ void __launch_bounds__(256, 2) step2_wide_kernel(Step2Args a, int wd, int cs_max, int wb) {
+  constexpr int ND = kWideTrials, NW = kWideWords;
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int Di = wd * ND;
+  const int wt = (int)(blockDim.x >> 5) / wd;
+  const int S = a.n_subbands;
+  const int copy_stride = cs_max * wb;  // one copy of a chunk's windows
+  const int stage_bytes = 2 * copy_stride;
+  uint16_t* tbl = reinterpret_cast<uint16_t*>(smem + kWideStages * stage_bytes);  // [S][Di]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kWideStages * stage_bytes + S * Di * 2);
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (int)(blockDim.x >> 5);
+  const int dm_sub = warp % wd, t_sub = warp / wd;
+  const int t0 = blockIdx.x * wt * kWideTime;
+  const int k = a.tiles[3 * blockIdx.y], ib = a.tiles[3 * blockIdx.y + 1], nd = a.tiles[3 * blockIdx.y + 2];
+  const int n_chunks = (S + cs_max - 1) / cs_max;
+  const uint32_t toff = (uint32_t)(t_sub * 128 * NW + lane * 4);  // bytes
+  const int64_t lim = (int64_t)stage_bytes - (int64_t)(toff + 128 * (NW - 1) + 4);
+  const int32_t* d2row0 = a.d2 + (int64_t)ib * S;
+  const uint16_t* ybase = a.y + (int64_t)k * S * a.y_pitch;
+
+  if (tid == 0) {
+    for (int q = 0; q < kWideStages; q++) mbar_init(&full[q], 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+
+  // warp 0: copy 0 of every window of chunk c into its stage, lane sl taking subband sl
+  auto issue = [&](int c) {
+    const int st = c % kWideStages, sb = c * cs_max, cs = min(cs_max, S - sb);
+    uint32_t bytes = 0;
+    int64_t start = 0;
+    if (lane < cs) {
+      start = (int64_t)((t0 + __ldg(&d2row0[sb + lane])) & ~7);
+      bytes = (uint32_t)min((int64_t)wb, 2 * (a.y_pitch - start));
+    }
+    const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) {
+      fence_proxy_async();
+      mbar_arrive_expect_tx(&full[st], total);
+    }
+    __syncwarp();
+    if (lane < cs)
+      bulk_g2s(smem + st * stage_bytes + lane * wb, ybase + (int64_t)(sb + lane) * a.y_pitch + start, bytes,
+               &full[st]);
+  };
+
+  uint32_t lanes[ND][NW], cnt[ND * NW / 2];
+#pragma unroll
+  for (int r = 0; r < ND; r++)
+#pragma unroll
+    for (int m = 0; m < NW; m++) lanes[r][m] = 0u;
+#pragma unroll
+  for (int q = 0; q < ND * NW / 2; q++) cnt[q] = 0u;
+
+  if (warp == 0)
+    for (int c = 0; c < min(kWideStages - 1, n_chunks); c++) issue(c);
+  // while chunk 0 lands: the staged offsets, as above, in words
+  for (int e = tid; e < Di * S; e += blockDim.x) {
+    const int r = e / S, s = e - r * S;
+    const int i = ib + min(r, nd - 1);
+    const int start = (t0 + __ldg(&d2row0[s])) & ~7;
+    const int rel = t0 + __ldg(&a.d2[(int64_t)i * S + s]) - start;  // samples
+    tbl[s * Di + r] = (uint16_t)(((rel & 1) * copy_stride + (s % cs_max) * wb + 2 * (rel & ~1)) >> 2);
+  }
+  int pending = 0;
+  const int wwords = wb >> 2;
+  for (int c = 0; c < n_chunks; c++) {
+    const int st = c % kWideStages, sb = c * cs_max, cs = min(cs_max, S - sb);
+    uint8_t* stage = smem + st * stage_bytes;
+    const bool ok = mbar_wait(&full[st], (c / kWideStages) & 1, a.status);
+    // copy 1 = copy 0 one sample later; a warp per subband window
+    const uint32_t* c0 = reinterpret_cast<const uint32_t*>(stage);
+    uint32_t* c1 = reinterpret_cast<uint32_t*>(stage + copy_stride);
+    if (ok)
+      for (int sl = warp; sl < cs; sl += nwarps)
+        for (int j = lane; j < wwords; j += 32) {
+          const int e = sl * wwords + j;
+          c1[e] = __byte_perm(c0[e], j + 1 < wwords ? c0[e + 1] : 0u, 0x5432);
+        }
+    // copy 1 is ready, and the chunk before is no longer read
+    if (__syncthreads_or(ok ? 0 : 1)) {
+      // the copies issued and not yet waited for may still be in flight: one
+      // more bounded wait for each before the block leaves
+      if (tid == 0)
+        for (int q = c; q < min(c + kWideStages - 1, n_chunks); q++)
+          mbar_wait(&full[q % kWideStages], (q / kWideStages) & 1, nullptr);
+      return;
+    }
+    if (warp == 0 && c + kWideStages - 1 < n_chunks) issue(c + kWideStages - 1);
+
+    const uint32_t base = smem_u32(stage) + toff;
+    const uint16_t* trow = tbl + sb * Di + dm_sub * ND;
+    auto offsets = [&](int sl, uint32_t (&o)[ND]) {
+      const uint4 v = *reinterpret_cast<const uint4*>(trow + sl * Di);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        o[2 * q] = (w[q] & 0xFFFFu) << 2;
+        o[2 * q + 1] = (w[q] >> 16) << 2;
+      }
+    };
+    int sl = 0;
+    for (; sl + 1 < cs; sl += 2) {
+      if (pending + 2 > a.flush_every) {
+        wide_fold<ND, NW>(lanes, cnt);
+        pending = 0;
+      }
+      pending += 2;
+      uint32_t e0[ND], e1[ND];
+      offsets(sl, e0);
+      offsets(sl + 1, e1);
+      uint32_t A[NW] = {}, B[NW] = {};
+#pragma unroll
+      for (int r = 0; r < ND; r++) {
+        if (kBoundsCheck) {
+          if (!stage_read_ok(e0[r], lim, a.status) || !stage_read_ok(e1[r], lim, a.status)) continue;
+          lds_row<NW>(base + e0[r], A);
+          lds_row<NW>(base + e1[r], B);
+        } else if (r == 0) {
+          lds_row<NW>(base + e0[0], A);
+          lds_row<NW>(base + e1[0], B);
+        } else {
+          lds_row_if<NW>(e0[r] != e0[r - 1], base + e0[r], A);
+          lds_row_if<NW>(e1[r] != e1[r - 1], base + e1[r], B);
+        }
+#pragma unroll
+        for (int m = 0; m < NW; m++) lanes[r][m] += A[m] + B[m];
+      }
+    }
+    if (sl < cs) {
+      if (pending + 1 > a.flush_every) {
+        wide_fold<ND, NW>(lanes, cnt);
+        pending = 0;
+      }
+      pending++;
+      uint32_t e0[ND];
+      offsets(sl, e0);
+#pragma unroll
+      for (int r = 0; r < ND; r++) {
+        uint32_t A[NW] = {};
+        if (stage_read_ok(e0[r], lim, a.status)) lds_row<NW>(base + e0[r], A);
+#pragma unroll
+        for (int m = 0; m < NW; m++) lanes[r][m] += A[m];
+      }
+    }
+  }
+
+  const bool vec = (a.n_t & 1) == 0;
+#pragma unroll
+  for (int r = 0; r < ND; r++) {
+    const int rr = dm_sub * ND + r;
+    if (rr >= nd) continue;
+    int32_t* orow = a.D + (int64_t)(ib + rr) * a.n_t;
+#pragma unroll
+    for (int m = 0; m < NW; m++) {
+      const int t = t0 + (int)(toff >> 1) + 64 * m;
+      if (t >= a.n_t) continue;
+      const int2 v = wide_sum<ND, NW>(lanes, cnt, r, m);
+      if (t + 1 < a.n_t && vec) {
+        *reinterpret_cast<int2*>(orow + t) = v;
+      } else {
+        orow[t] = v.x;
+        if (t + 1 < a.n_t) orow[t + 1] = v.y;
+      }
+    }
+  }
+}
+
 typedef void (*Step2Kernel)(Step2Args, int, int, int);
 
 template <int ND, int NW>
@@ -228,7 +408,23 @@ size_t step2_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int32_t n
   return 2 * stage + (Di * n_subbands * 4 + 15) / 16 * 16 + 16;
 }
 
+size_t step2_wide_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int32_t n_subbands) {
+  const size_t stage = 2 * (size_t)c.chunk * copy_bytes(c, dmax_tile);
+  return kWideStages * stage + (size_t)c.warps_dm * kWideTrials * n_subbands * 2 + 8 * kWideStages;
+}
+
 sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, cudaStream_t st) {
+  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) {
+    const int Tt = c.warps_time * kWideTime;
+    const size_t smem = step2_wide_smem_bytes(c, a.dmax_tile, a.n_subbands);
+    dim3 grid((a.n_t + Tt - 1) / Tt, a.n_tiles, 1);
+    if (grid.y > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many step-two tiles");
+    SPS_CUDA(cudaFuncSetAttribute(step2_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    step2_wide_kernel<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, c.chunk,
+                                                                         copy_bytes(c, a.dmax_tile));
+    SPS_CUDA(cudaGetLastError());
+    return SPS_OK;
+  }
   std::string why;
   if (!step2_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
   Step2Kernel fn = find(c.dms_per_thread, c.samples_per_thread / 2);

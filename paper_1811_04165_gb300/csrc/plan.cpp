@@ -153,6 +153,49 @@ int32_t cached_spread(const sps_plan* p, int which, int32_t tile) {
   return v;
 }
 
+// Step-two tiles: runs of trials that share a coarse DM, at most `di` long, and
+// the largest delay spread of one.
+void step2_tiles(const sps_plan* p, int32_t di, std::vector<int32_t>* tiles, int32_t* dmax) {
+  const int32_t n_dms = (int32_t)p->dms.size(), S = p->n_subbands;
+  tiles->clear();
+  *dmax = 0;
+  for (int32_t i = 0; i < n_dms;) {
+    const int32_t k = p->coarse_of[i];
+    int32_t j = i;
+    while (j < n_dms && p->coarse_of[j] == k && j - i < di) j++;
+    tiles->push_back(k);
+    tiles->push_back(i);
+    tiles->push_back(j - i);
+    for (int32_t s = 0; s < S; s++)
+      *dmax = std::max(*dmax, p->d2[(size_t)(j - 1) * S + s] - p->d2[(size_t)i * S + s]);
+    i = j;
+  }
+}
+
+// The tile step two runs with.  The default one leaves the choice to the library,
+// which takes the wide tile of eight warps (along DM up to the longest run of
+// trials of one coarse DM, the rest along time) where two subbands' sums fit its
+// lanes between folds, two blocks an SM, and the grid is at least two rounds of
+// them: 64 coarse x 32 fine trials of 12500 samples 97 -> 83 us, 64 x 24 (8
+// subbands) 41 -> 32; with one round (24 x 32) it takes 25 us against 23.
+sps_dedisp_config choose_step2(const sps_plan* p, const sps_dedisp_config& c) {
+  const int64_t unit = (int64_t)255 * (p->channels / p->n_subbands);
+  if (c.dms_per_thread != 4 || c.samples_per_thread != 16 || c.warps_dm != 8 || c.warps_time != 1 || c.chunk != 8 ||
+      p->channels > kWideChannels || 2 * unit > 65536 - (int64_t)kWideCount)
+    return c;
+  std::vector<int32_t> tiles;
+  int32_t dmax = 0, longest = 1;
+  step2_tiles(p, (int32_t)p->dms.size(), &tiles, &dmax);
+  for (size_t t = 2; t < tiles.size(); t += 3) longest = std::max(longest, tiles[t]);
+  sps_dedisp_config w{8, 14, std::min(4, (longest + 7) / 8), 1, 8, 0};
+  w.warps_time = 8 / w.warps_dm;
+  step2_tiles(p, 8 * w.warps_dm, &tiles, &dmax);
+  const int64_t tt = 32 * w.warps_time * w.samples_per_thread;
+  const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
+  const bool fits = 2 * (step2_wide_smem_bytes(w, dmax, p->n_subbands) + 1024) <= (size_t)p->smem_per_sm;
+  return fits && blocks >= 4 * p->sms ? w : c;
+}
+
 // Validate a configuration against the compiled variants and the device's
 // shared memory, without changing the plan; fills the per-config sizes.
 sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigCheck* out) {
@@ -186,17 +229,7 @@ sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigC
     // step-two tiles: runs of trials sharing one coarse DM, at most Di long
     const int32_t di = cfg.step2.warps_dm * cfg.step2.dms_per_thread;
     const int32_t S = p->n_subbands;
-    for (int32_t i = 0; i < n_dms;) {
-      const int32_t k = p->coarse_of[i];
-      int32_t j = i;
-      while (j < n_dms && p->coarse_of[j] == k && j - i < di) j++;
-      c.tiles.push_back(k);
-      c.tiles.push_back(i);
-      c.tiles.push_back(j - i);
-      for (int32_t s = 0; s < S; s++)
-        c.dmax_2 = std::max(c.dmax_2, p->d2[(size_t)(j - 1) * S + s] - p->d2[(size_t)i * S + s]);
-      i = j;
-    }
+    step2_tiles(p, di, &c.tiles, &c.dmax_2);
     const int32_t di1 = cfg.step1.warps_dm * cfg.step1.dms_per_thread;
     const size_t need1 =
         cfg.step1.presum
@@ -286,8 +319,10 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   int32_t splits = 1;
   choose_tile(p, cfg.brute, &tile, &splits);
   const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : cfg.step1;
-  const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0, dmax_1 = chk.dmax_1, dmax_2 = chk.dmax_2;
-  const std::vector<int32_t>& tiles = chk.tiles;
+  const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0;
+  const int32_t dmax_1 = chk.dmax_1;
+  int32_t dmax_2 = chk.dmax_2;
+  std::vector<int32_t>& tiles = chk.tiles;
   if (pass.presum) {
     PresumTables pt;
     sps_status s = p->mode == SPS_MODE_BRUTE
@@ -349,7 +384,10 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
     p->d_b0 = db0;
     p->d_offs = doffs;
   }
+  sps_dedisp_config tile2 = cfg.step2;
   if (p->mode == SPS_MODE_SUBBAND) {
+    tile2 = choose_step2(p, cfg.step2);
+    step2_tiles(p, tile2.warps_dm * tile2.dms_per_thread, &tiles, &dmax_2);
     int32_t* dt = nullptr;
     sps_status st = upload(tiles, &dt);
     if (st != SPS_OK) return st;
@@ -361,6 +399,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   p->cfg = cfg;
   p->brute_tile = tile;
   p->brute_splits = splits;
+  p->step2_tile = tile2;
   p->config_gen++;
   p->dmax_brute = dmax_b;
   p->dmax_step1 = dmax_1;

@@ -38,3 +38,31 @@ def test_wide_tile_equals_single_channel_kernel(lib, C, n_t, n_dms, step, full):
     assert torch.equal(got, want)
     if full:
         assert int(got[0, 0]) == 255 * C
+
+
+# subbands, channels per subband, coarse DMs, trials per coarse DM, samples, saturated
+STEP2 = [(5, 120, 64, 32, 9001, True),    # the most channels per subband, an odd chunk, rows of odd length
+         (17, 6, 128, 20, 4481, False),   # three warps along DM, the last with four trials
+         (32, 12, 96, 7, 14400, False)]   # one warp along DM, runs shorter than its eight trials
+
+
+@pytest.mark.parametrize("S,per,coarse,fine,n_t,full", STEP2)
+def test_wide_step_two_equals_narrow(lib, S, per, coarse, fine, n_t, full):
+    import torch
+    dms = 0.1 * np.arange(coarse * fine)
+    plan = lib.Plan(S * per, 1250.0, 1550.0, 81.92e-6, n_t, dms, [1], mode=lib.MODE_SUBBAND, n_subbands=S,
+                    coarse_dms=dms[::fine].copy())
+    gen = torch.Generator(device="cuda").manual_seed(S)
+    Y = torch.randint(255 * per if full else 0, 255 * per + 1, plan.y_shape, dtype=torch.int32, device="cuda",
+                      generator=gen).to(torch.int16).view(torch.uint16)
+    got = torch.full((plan.n_dms, n_t), -1, dtype=torch.int32, device="cuda")
+    lib.sps_subband_step2(plan, Y, got)
+    cfg = plan.config
+    cfg.step2 = lib.DedispConfig(4, 8, 4, 1, 4, 0)
+    plan.config = cfg
+    want = torch.full((plan.n_dms, n_t), -2, dtype=torch.int32, device="cuda")
+    lib.sps_subband_step2(plan, Y, want)
+    assert plan.status() == 0
+    assert torch.equal(got, want)
+    if full:
+        assert int(got[0, 0]) == 255 * per * S
