@@ -167,7 +167,7 @@ sps_status run_u8_pass(const sps_plan* p, const sps_dedisp_config& cfg, const ui
 
 sps_status run_step1(const sps_plan* p, const uint8_t* x, int64_t pitch, uint8_t* ws, uint16_t* Y,
                      cudaStream_t st) {
-  return run_u8_pass(p, p->cfg.step1, x, pitch, ws, (int32_t)p->coarse_dms.size(), p->channels / p->n_subbands,
+  return run_u8_pass(p, p->step1_tile, x, pitch, ws, (int32_t)p->coarse_dms.size(), p->channels / p->n_subbands,
                      (int32_t)p->n_1, p->y_pitch, p->dmax_step1, Y, 1, st);
 }
 

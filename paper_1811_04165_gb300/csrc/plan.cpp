@@ -172,28 +172,67 @@ void step2_tiles(const sps_plan* p, int32_t di, std::vector<int32_t>* tiles, int
   }
 }
 
+bool same_tile(const sps_dedisp_config& a, const sps_dedisp_config& b) {
+  return a.dms_per_thread == b.dms_per_thread && a.samples_per_thread == b.samples_per_thread &&
+         a.warps_dm == b.warps_dm && a.warps_time == b.warps_time && a.chunk == b.chunk && a.presum == b.presum;
+}
+
+// Microseconds of a pass whose blocks each start and end in 2, take `step` per
+// chunk and then `cycles` of their SM at 2.03 GHz, in rounds of the blocks that
+// fit the GPU at once.
+double pass_us(const sps_plan* p, int64_t blocks, int64_t per_sm, int64_t chunks, double step, double cycles) {
+  const int64_t slots = per_sm * p->sms;
+  auto round = [&](int64_t n) {
+    const int64_t on_sm = (n + p->sms - 1) / p->sms;
+    return 2.0 + step * chunks + on_sm * cycles / 2030.0;
+  };
+  return (blocks / slots) * round(slots) + (blocks % slots ? round(blocks % slots) : 0.0);
+}
+
 // The tile step two runs with.  The default one leaves the choice to the library,
 // which takes the wide tile of eight warps (along DM up to the longest run of
 // trials of one coarse DM, the rest along time) where two subbands' sums fit its
 // lanes between folds, two blocks an SM, and the grid is at least two rounds of
 // them: 64 coarse x 32 fine trials of 12500 samples 97 -> 83 us, 64 x 24 (8
-// subbands) 41 -> 32; with one round (24 x 32) it takes 25 us against 23.
+// subbands) 41 -> 32; with one round (24 x 32) it takes 25 us against 23.  Smaller
+// grids take the default tile or smaller ones by the model of pass_us: 13 coarse x
+// 8 fine trials of 1697 samples, 48 subbands 18.0 -> 7.2 us in tiles of 8 x 128.
 sps_dedisp_config choose_step2(const sps_plan* p, const sps_dedisp_config& c) {
   const int64_t unit = (int64_t)255 * (p->channels / p->n_subbands);
-  if (c.dms_per_thread != 4 || c.samples_per_thread != 16 || c.warps_dm != 8 || c.warps_time != 1 || c.chunk != 8 ||
-      p->channels > kWideChannels || 2 * unit > 65536 - (int64_t)kWideCount)
-    return c;
+  struct Tile { sps_dedisp_config c; double cycles; };
+  const Tile narrow[] = {{{4, 16, 8, 1, 8, 0}, 1.7}, {{2, 8, 8, 1, 16, 0}, 2.0}, {{1, 8, 8, 1, 32, 0}, 2.2},
+                         {{1, 4, 8, 1, 32, 0}, 2.5}};
+  if (!same_tile(c, narrow[0].c)) return c;
   std::vector<int32_t> tiles;
   int32_t dmax = 0, longest = 1;
   step2_tiles(p, (int32_t)p->dms.size(), &tiles, &dmax);
   for (size_t t = 2; t < tiles.size(); t += 3) longest = std::max(longest, tiles[t]);
-  sps_dedisp_config w{8, 14, std::min(4, (longest + 7) / 8), 1, 8, 0};
-  w.warps_time = 8 / w.warps_dm;
-  step2_tiles(p, 8 * w.warps_dm, &tiles, &dmax);
-  const int64_t tt = 32 * w.warps_time * w.samples_per_thread;
-  const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
-  const bool fits = 2 * (step2_wide_smem_bytes(w, dmax, p->n_subbands) + 1024) <= (size_t)p->smem_per_sm;
-  return fits && blocks >= 4 * p->sms ? w : c;
+  if (p->channels <= kWideChannels && 2 * unit <= 65536 - (int64_t)kWideCount) {
+    sps_dedisp_config w{8, 14, std::min(4, (longest + 7) / 8), 1, 8, 0};
+    w.warps_time = 8 / w.warps_dm;
+    step2_tiles(p, 8 * w.warps_dm, &tiles, &dmax);
+    const int64_t tt = 32 * w.warps_time * w.samples_per_thread;
+    const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
+    const bool fits = 2 * (step2_wide_smem_bytes(w, dmax, p->n_subbands) + 1024) <= (size_t)p->smem_per_sm;
+    if (fits && blocks >= 4 * p->sms) return w;
+  }
+  sps_dedisp_config best = c;
+  double least = 1e30;
+  for (const Tile& t : narrow) {
+    step2_tiles(p, t.c.warps_dm * t.c.dms_per_thread, &tiles, &dmax);
+    const size_t smem = step2_smem_bytes(t.c, dmax, p->n_subbands);
+    if (smem > (size_t)p->max_smem) continue;
+    const int64_t tt = 32 * t.c.warps_time * t.c.samples_per_thread;
+    const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
+    const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(2, p->smem_per_sm / (smem + 1024)));
+    const int64_t words = 8 * t.c.dms_per_thread * (t.c.samples_per_thread / 2) * p->n_subbands;
+    const double us = pass_us(p, blocks, per_sm, (p->n_subbands + t.c.chunk - 1) / t.c.chunk, 0.6, words * t.cycles);
+    if (us < least) {
+      least = us;
+      best = t.c;
+    }
+  }
+  return best;
 }
 
 // Validate a configuration against the compiled variants and the device's
@@ -251,6 +290,47 @@ bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* 
          c.warps_time == 1 && c.chunk == 16 && channels <= kWideChannels;
 }
 
+// The tile the single-channel pass runs with (brute force, or step one).  The
+// default one leaves the choice to the library: larger blocks read the staged
+// windows more often, smaller ones spread a small plan over the SMs.  Cycles per
+// warp word (32 lanes x 4 bytes) beside one per 64 staged bytes, as measured (1536 channels x 12500 samples x 768 trials 652 us with the
+// default tile, 578 with twice the trials and channels per stage; 64 channels x
+// 4096 samples x 32 trials 14.2 us with 8 blocks, 5.8 with 128 small ones; step one
+// of 768 channels, 8 subbands, 4 coarse DMs 19.2 -> 7.8 us).
+sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c) {
+  struct Tile { sps_dedisp_config c; double cycles; };
+  const Tile tiles[] = {{{4, 16, 8, 1, 16, 0}, 1.45}, {{4, 16, 16, 1, 32, 0}, 1.34}, {{2, 16, 8, 1, 32, 0}, 1.45},
+                        {{2, 8, 8, 1, 32, 0}, 1.5},   {{1, 8, 8, 1, 48, 0}, 1.7},    {{1, 4, 8, 1, 64, 0}, 2.0}};
+  if (!same_tile(c, tiles[0].c)) return c;
+  const bool brute = p->mode == SPS_MODE_BRUTE;
+  const int64_t rows = brute ? (int64_t)p->dms.size() : (int64_t)p->coarse_dms.size();
+  const int64_t n_out = brute ? p->n_t : p->n_1;
+  const int32_t G = brute ? 1 : p->n_subbands, per = p->channels / G;
+  sps_dedisp_config best = c;
+  double least = 1e30;
+  for (const Tile& t : tiles) {
+    const int32_t di = t.c.warps_dm * t.c.dms_per_thread, tt = 32 * t.c.warps_time * t.c.samples_per_thread;
+    const size_t smem = u8_smem_bytes(t.c, cached_spread(p, brute ? 0 : 1, di), per, G);
+    if (smem > (size_t)p->max_smem) continue;
+    const int64_t warps = t.c.warps_dm * t.c.warps_time;
+    const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(16 / warps, p->smem_per_sm / (smem + 1024)));
+    const int64_t tiles_n = (rows + di - 1) / di * ((n_out + tt - 1) / tt);
+    const int64_t gpb = u8_groups_per_block(G, tiles_n), blocks = tiles_n * ((G + gpb - 1) / gpb);
+    const int64_t words = warps * t.c.dms_per_thread * (t.c.samples_per_thread / 4) * per * gpb;
+    const double staged = 4.0 * per * gpb * u8_window_bytes(t.c, cached_spread(p, brute ? 0 : 1, di));
+    double us = pass_us(p, blocks, per_sm, gpb * ((per + t.c.chunk - 1) / t.c.chunk), 0.4,
+                        words * t.cycles + staged / 64);
+    // a block that has its SM to itself starts and ends with nothing beside it (step
+    // one of 1536 channels, 16 subbands, 40 coarse DMs: 53 us, 60 in such blocks)
+    if (warps == 16) us += 10.0 * ((blocks + p->sms - 1) / p->sms);
+    if (us < least) {
+      least = us;
+      best = t.c;
+    }
+  }
+  return best;
+}
+
 // The tile and the channel splits the brute-force pass runs with, by a model of
 // its time.
 //   * The default pre-summed tile leaves the choice to the library.  The wide
@@ -269,7 +349,11 @@ bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* 
 void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_config* tile, int32_t* splits) {
   *tile = c;
   *splits = 1;
-  if (p->mode != SPS_MODE_BRUTE || !c.presum) return;
+  if (p->mode != SPS_MODE_BRUTE) return;
+  if (!c.presum) {
+    *tile = choose_u8(p, c);
+    return;
+  }
   const int64_t rows = (int64_t)p->dms.size(), units = (p->channels + (1 << c.presum) - 1) >> c.presum;
   const double out_kb = 4e-3 * rows * p->n_t;
   double best = 1e30;
@@ -318,9 +402,11 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   sps_dedisp_config tile;
   int32_t splits = 1;
   choose_tile(p, cfg.brute, &tile, &splits);
-  const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : cfg.step1;
+  const sps_dedisp_config tile1 = p->mode == SPS_MODE_BRUTE || cfg.step1.presum ? cfg.step1 : choose_u8(p, cfg.step1);
+  const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : tile1;
   const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0;
-  const int32_t dmax_1 = chk.dmax_1;
+  const int32_t dmax_1 =
+      p->mode == SPS_MODE_SUBBAND ? cached_spread(p, 1, tile1.warps_dm * tile1.dms_per_thread) : 0;
   int32_t dmax_2 = chk.dmax_2;
   std::vector<int32_t>& tiles = chk.tiles;
   if (pass.presum) {
@@ -369,7 +455,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
     if (p->mode == SPS_MODE_BRUTE)
       build_u8_tables(p->delays, n_dms, p->channels, p->channels, tile, dmax_b, &b0, &offs);
     else
-      build_u8_tables(p->d1, (int32_t)p->coarse_dms.size(), p->channels, p->channels / p->n_subbands, cfg.step1,
+      build_u8_tables(p->d1, (int32_t)p->coarse_dms.size(), p->channels, p->channels / p->n_subbands, tile1,
                       dmax_1, &b0, &offs);
     int32_t* db0 = nullptr;
     uint32_t* doffs = nullptr;
@@ -399,6 +485,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   p->cfg = cfg;
   p->brute_tile = tile;
   p->brute_splits = splits;
+  p->step1_tile = tile1;
   p->step2_tile = tile2;
   p->config_gen++;
   p->dmax_brute = dmax_b;

@@ -201,6 +201,7 @@ bool u8_config_supported(const sps_dedisp_config& cfg, std::string* why);
 bool step2_config_supported(const sps_dedisp_config& cfg, std::string* why);
 bool snr_config_supported(const sps_snr_config& cfg, std::string* why);
 size_t u8_smem_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile, int32_t group_channels, int32_t n_groups);
+int u8_groups_per_block(int32_t n_groups, int64_t tiles);
 int u8_window_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile);
 int u8_di_pad(const sps_dedisp_config& cfg);
 size_t step2_wide_smem_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile, int32_t n_subbands);
@@ -297,7 +298,7 @@ struct sps_plan {
   // the tile the brute-force pass runs with: cfg.brute, or the one the library
   // picks for the default pre-summed tile (presum_tile in plan.cpp)
   sps_dedisp_config brute_tile{};
-  sps_dedisp_config step2_tile{};  // likewise step two's
+  sps_dedisp_config step1_tile{}, step2_tile{};  // likewise of the two steps
   int32_t brute_splits = 1;      // shares of the channels that blocks of their own sum
   uint64_t config_gen = 0;       // bumped whenever the device tables are rebuilt
   // delay spread of one DM tile for the current configuration
