@@ -74,7 +74,7 @@ size_t workspace_any_config(const sps_plan* p) {
 
 // Points the search at the masked copy of x when channels are zapped; moves
 // the workspace past it.
-sps_status prepare_input(const sps_plan* p, const uint8_t** x, int64_t* pitch, uint8_t** ws, cudaStream_t st) {
+sps_status prepare_input(const sps_plan* p, const uint8_t** x, int64_t* pitch, uint8_t** ws, Stream& st) {
   if (p->zap.empty()) return SPS_OK;
   if (sps_status s = launch_zap_copy(*x, *pitch, (int32_t)p->n_in, p->d_zap, p->channels, *ws, p->pitch4, st))
     return s;
@@ -103,7 +103,7 @@ U8PassArgs u8_args(const sps_plan* p, const uint8_t* x, int64_t pitch, const uin
 // the pass that reads them.
 sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const uint8_t* x, int64_t pitch,
                           uint8_t* ws, int32_t rows, int32_t per, int32_t n_out, int64_t out_pitch, int32_t dmax,
-                          void* out, int32_t out_u16, int32_t splits, cudaStream_t st, PresumPassArgs* args) {
+                          void* out, int32_t out_u16, int32_t splits, Stream& st, PresumPassArgs* args) {
   uint16_t* q = reinterpret_cast<uint16_t*>(ws);
   const int32_t K = 1 << cfg.presum;
   // split sums are added into zeroed rows
@@ -142,7 +142,7 @@ sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const
 // One uint8 pass (brute force or step one) with the configured kernel.
 sps_status run_u8_pass(const sps_plan* p, const sps_dedisp_config& cfg, const uint8_t* x, int64_t pitch,
                        uint8_t* ws, int32_t rows, int32_t per, int32_t n_out, int64_t out_pitch, int32_t dmax,
-                       void* out, int32_t out_u16, cudaStream_t st) {
+                       void* out, int32_t out_u16, Stream& st) {
   if (cfg.presum) {
     PresumPassArgs a{};
     sps_status s = presum_prepass(p, cfg, x, pitch, ws, rows, per, n_out, out_pitch, dmax, out, out_u16,
@@ -166,12 +166,12 @@ sps_status run_u8_pass(const sps_plan* p, const sps_dedisp_config& cfg, const ui
 }
 
 sps_status run_step1(const sps_plan* p, const uint8_t* x, int64_t pitch, uint8_t* ws, uint16_t* Y,
-                     cudaStream_t st) {
+                     Stream& st) {
   return run_u8_pass(p, p->step1_tile, x, pitch, ws, (int32_t)p->coarse_dms.size(), p->channels / p->n_subbands,
                      (int32_t)p->n_1, p->y_pitch, p->dmax_step1, Y, 1, st);
 }
 
-sps_status run_step2(const sps_plan* p, const uint16_t* Y, int32_t* D, cudaStream_t st) {
+sps_status run_step2(const sps_plan* p, const uint16_t* Y, int32_t* D, Stream& st) {
   Step2Args a{};
   a.y = Y;
   a.y_pitch = p->y_pitch;
@@ -197,7 +197,7 @@ sps_status check_workspace(const sps_plan* p, void* ws, size_t ws_bytes) {
 }
 
 sps_status run_dedisperse(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
-                          size_t ws_bytes, cudaStream_t st) {
+                          size_t ws_bytes, Stream& st) {
   sps_status s = check_x(p, x, pitch);
   if (s) return s;
   if (!D || !aligned16(D)) return fail(SPS_ERR_INVALID_ARG, "D must be non-null and 16-byte aligned");
@@ -213,7 +213,7 @@ sps_status run_dedisperse(const sps_plan* p, const uint8_t* x, int64_t pitch, in
 }
 
 sps_status run_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,
-                   int32_t* best, cudaStream_t st) {
+                   int32_t* best, Stream& st) {
   if (!D || !snr || !peak_t || !peak_val) return fail(SPS_ERR_INVALID_ARG, "null pointer");
   SnrArgs a{};
   a.D = D;
@@ -240,21 +240,24 @@ sps_status run_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* pe
 size_t plan_workspace_bytes(const sps_plan* p) { return workspace_needed(p); }
 
 sps_status run_search(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws, size_t ws_bytes,
-                      double* snr, int32_t* peak_t, int32_t* peak_val, int32_t* best, cudaStream_t st) {
+                      double* snr, int32_t* peak_t, int32_t* peak_val, int32_t* best, cudaStream_t stream) {
+  Stream st(stream);
   sps_status s = run_dedisperse(p, x, pitch, D, ws, ws_bytes, st);
   if (s) return s;
   return run_snr(p, D, snr, peak_t, peak_val, best, st);
 }
 
 sps_status dedisperse_into(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
-                           size_t ws_bytes, cudaStream_t st) {
+                           size_t ws_bytes, cudaStream_t stream) {
+  Stream st(stream);
   return run_dedisperse(p, x, pitch, D, ws, ws_bytes, st);
 }
 
 bool batched_pass_form(const sps_plan* p) { return p->mode == SPS_MODE_BRUTE && p->cfg.brute.presum > 0; }
 
 sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
-                         size_t ws_bytes, cudaStream_t st, PresumPassArgs* args) {
+                         size_t ws_bytes, cudaStream_t stream, PresumPassArgs* args) {
+  Stream st(stream);
   if (!batched_pass_form(p)) return fail(SPS_ERR_INVALID_ARG, "not a pre-summed brute-force plan");
   sps_status s = check_x(p, x, pitch);
   if (s) return s;
@@ -267,7 +270,8 @@ sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int
 }
 
 sps_status snr_into(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,
-                    int32_t* best, cudaStream_t st) {
+                    int32_t* best, cudaStream_t stream) {
+  Stream st(stream);
   return run_snr(p, D, snr, peak_t, peak_val, best, st);
 }
 
@@ -364,7 +368,8 @@ sps_status sps_dedisperse(const sps_plan* p, const uint8_t* x, int64_t pitch, in
   clear_error();
   NvtxRange nvtx("sps_dedisperse");
   if (sps_status s = check_plan(p)) return s;
-  return run_dedisperse(p, x, pitch, D, ws, ws_bytes, (cudaStream_t)stream);
+  Stream st((cudaStream_t)stream);
+  return run_dedisperse(p, x, pitch, D, ws, ws_bytes, st);
 }
 
 sps_status sps_subband_step1(const sps_plan* p, const uint8_t* x, int64_t pitch, uint16_t* Y, void* ws,
@@ -377,8 +382,9 @@ sps_status sps_subband_step1(const sps_plan* p, const uint8_t* x, int64_t pitch,
   if (!Y || !aligned16(Y)) return fail(SPS_ERR_INVALID_ARG, "Y must be non-null and 16-byte aligned");
   if (sps_status s = check_workspace(p, ws, ws_bytes)) return s;
   uint8_t* w = static_cast<uint8_t*>(ws);
-  if (sps_status s = prepare_input(p, &x, &pitch, &w, (cudaStream_t)stream)) return s;
-  return run_step1(p, x, pitch, w, Y, (cudaStream_t)stream);
+  Stream st((cudaStream_t)stream);
+  if (sps_status s = prepare_input(p, &x, &pitch, &w, st)) return s;
+  return run_step1(p, x, pitch, w, Y, st);
 }
 
 sps_status sps_subband_step2(const sps_plan* p, const uint16_t* Y, int32_t* D, void* stream) {
@@ -387,7 +393,8 @@ sps_status sps_subband_step2(const sps_plan* p, const uint16_t* Y, int32_t* D, v
   if (sps_status s = check_plan(p)) return s;
   if (p->mode != SPS_MODE_SUBBAND) return fail(SPS_ERR_INVALID_ARG, "plan is not in SUBBAND mode");
   if (!Y || !aligned16(Y) || !D || !aligned16(D)) return fail(SPS_ERR_INVALID_ARG, "Y and D must be 16-byte aligned");
-  return run_step2(p, Y, D, (cudaStream_t)stream);
+  Stream st((cudaStream_t)stream);
+  return run_step2(p, Y, D, st);
 }
 
 sps_status sps_integrate(const sps_plan* p, const int32_t* D, int32_t* B, void* stream) {
@@ -395,8 +402,9 @@ sps_status sps_integrate(const sps_plan* p, const int32_t* D, int32_t* B, void* 
   NvtxRange nvtx("sps_integrate");
   if (sps_status s = check_plan(p)) return s;
   if (!D || !B) return fail(SPS_ERR_INVALID_ARG, "null pointer");
+  Stream st((cudaStream_t)stream);
   return launch_integrate(D, (int32_t)p->dms.size(), p->n_t, p->d_widths, (int32_t)p->widths.size(),
-                          p->smoothing == SPS_SMOOTH_DECIMATE ? 1 : 0, B, p->d_status, (cudaStream_t)stream);
+                          p->smoothing == SPS_SMOOTH_DECIMATE ? 1 : 0, B, p->d_status, st);
 }
 
 sps_status sps_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,
@@ -404,7 +412,8 @@ sps_status sps_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* pe
   clear_error();
   NvtxRange nvtx("sps_snr");
   if (sps_status s = check_plan(p)) return s;
-  return run_snr(p, D, snr, peak_t, peak_val, best, (cudaStream_t)stream);
+  Stream st((cudaStream_t)stream);
+  return run_snr(p, D, snr, peak_t, peak_val, best, st);
 }
 
 sps_status sps_search(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
@@ -413,9 +422,10 @@ sps_status sps_search(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_
   clear_error();
   NvtxRange nvtx("sps_search");
   if (sps_status s = check_plan(p)) return s;
-  sps_status s = run_dedisperse(p, x, pitch, D, ws, ws_bytes, (cudaStream_t)stream);
+  Stream st((cudaStream_t)stream);
+  sps_status s = run_dedisperse(p, x, pitch, D, ws, ws_bytes, st);
   if (s) return s;
-  return run_snr(p, D, snr, peak_t, peak_val, best, (cudaStream_t)stream);
+  return run_snr(p, D, snr, peak_t, peak_val, best, st);
 }
 
 sps_status sps_search_host(const sps_plan* p, const uint8_t* x_host, int64_t pitch, uint8_t* x_dev, int32_t* D,
@@ -430,9 +440,10 @@ sps_status sps_search_host(const sps_plan* p, const uint8_t* x_host, int64_t pit
   cudaStream_t st = (cudaStream_t)stream;
   const size_t n_out = (size_t)p->dms.size() * p->widths.size();
   SPS_CUDA(cudaMemcpyAsync(x_dev, x_host, (size_t)p->channels * pitch, cudaMemcpyHostToDevice, st));
-  sps_status s = run_dedisperse(p, x_dev, pitch, D, ws, ws_bytes, st);
+  Stream chain(st);
+  sps_status s = run_dedisperse(p, x_dev, pitch, D, ws, ws_bytes, chain);
   if (s) return s;
-  s = run_snr(p, D, snr_dev, peak_t_dev, peak_val_dev, best_dev, st);
+  s = run_snr(p, D, snr_dev, peak_t_dev, peak_val_dev, best_dev, chain);
   if (s) return s;
   if (snr_host) SPS_CUDA(cudaMemcpyAsync(snr_host, snr_dev, n_out * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (peak_t_host)

@@ -223,9 +223,10 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
         presum_pass_work(passes[pass_of[b]], plans[b]->brute_tile, pass_of[b] - first, &work);
         max_stage = std::max(max_stage, passes[pass_of[b]].stage_bytes);
       }
+      Stream list_stream(sg);
       if (st == SPS_OK)
         st = launch_presum_pass_list(batch->d_passes + first, batch->d_work + w0, (int64_t)(work.size() - w0),
-                                     plans[beams[0]]->brute_tile, max_stage, sg);
+                                     plans[beams[0]]->brute_tile, max_stage, list_stream);
       batch->list_launches++;
       if (st == SPS_OK) cuda_ok(cudaEventRecord(group_done[gi], sg), "cudaEventRecord");
     }

@@ -212,6 +212,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
     }
   };
 
+  pdl_wait();  // the series are written
   // Chunks 0 and 1 go out first; after computing chunk ch, warp (ch mod
   // nwarps) stages chunk ch + 2 into the stage chunk ch - 1 used, once every
   // warp has released that stage.  No block-wide barrier: a warp waits only for
@@ -309,6 +310,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   }
   if constexpr (!WIDE) fold();
 
+  pdl_next();
   // Each lane holds 2 consecutive samples per (trial, word).
   const bool vec = (a.out_pitch & 1) == 0;
 #pragma unroll
@@ -502,6 +504,7 @@ __global__ void __launch_bounds__(kSeriesThreads) presum_series_kernel(const uin
   const int4 uh = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x));      // {c0, n, s_begin, s_end}
   const int4 ur = __ldg(reinterpret_cast<const int4*>(units + blockIdx.x) + 1);  // {max_rel, lo, hi, 0}
   const int ub = blockIdx.y * kSeriesBlock;
+  pdl_wait();
   if (blockIdx.z == 0) zero_share(zero, n_zero);
   if (ub >= ur.z || ub + kSeriesBlock <= ur.y) return;  // no series of the unit needs these samples
   // the block's share of the unit's series
@@ -567,6 +570,7 @@ __global__ void __launch_bounds__(256) presum_series_direct_kernel(const uint8_t
                                                                    int32_t in_len, const PresumSeries* series,
                                                                    int32_t n_series, uint16_t* q,
                                                                    int32_t q_pitch, int32_t* zero, int64_t n_zero) {
+  pdl_wait();
   zero_share(zero, n_zero);
   const int64_t per_row = q_pitch >> 4;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -667,7 +671,7 @@ size_t presum_smem_bytes(int32_t stage_bytes) { return kStages * (size_t)stage_b
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
                                 int32_t n_units, int32_t unit_channels, int32_t max_rel, const PresumSeries* series,
                                 int32_t n_series, uint16_t* q, int32_t q_pitch, int32_t* zero, int64_t n_zero,
-                                cudaStream_t st) {
+                                Stream& st) {
   if (n_series == 0) return SPS_OK;
   // staged window per channel row: the block's samples, the largest relative
   // delay, and the 16-byte reach of the last thread's loads
@@ -682,18 +686,17 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
     dim3 grid((unsigned)n_units, (unsigned)((q_pitch + kSeriesBlock - 1) / kSeriesBlock));
     const int64_t blocks = (int64_t)grid.x * grid.y;
     grid.z = (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_series / (4 * n_units), (16 * 152 + blocks - 1) / blocks));
-    presum_series_kernel<<<grid, kSeriesThreads, (size_t)smem, st>>>(x, pitch, in_len, units, series, q, q_pitch,
-                                                                    (int32_t)win, zero, n_zero);
+    SPS_CUDA(launch(st, presum_series_kernel, grid, kSeriesThreads, (size_t)smem, x, pitch, in_len, units, series, q,
+                    q_pitch, (int32_t)win, zero, n_zero));
   } else {
     const int64_t threads = (int64_t)(q_pitch >> 4) * n_series;
-    presum_series_direct_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(x, pitch, in_len, series,
-                                                                                   n_series, q, q_pitch, zero, n_zero);
+    SPS_CUDA(launch(st, presum_series_direct_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, x, pitch, in_len,
+                    series, n_series, q, q_pitch, zero, n_zero));
   }
-  SPS_CUDA(cudaGetLastError());
   return SPS_OK;
 }
 
-sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& c, cudaStream_t st) {
+sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& c, Stream& st) {
   PresumKernel fn = find(c.dms_per_thread, c.samples_per_thread / 2);
   if (!fn) return fail(SPS_ERR_INVALID_ARG, "no compiled pre-summed variant");
   const int Di = c.warps_dm * c.dms_per_thread;
@@ -702,8 +705,8 @@ sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& 
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, a.n_groups * a.splits);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
   SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, presum_window_bytes(c, a.dmax_tile));
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm,
+                  presum_window_bytes(c, a.dmax_tile)));
   return SPS_OK;
 }
 
@@ -723,14 +726,14 @@ void presum_pass_work(const PresumPassArgs& a, const sps_dedisp_config& c, int32
 }
 
 sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d_work, int64_t n_work,
-                                   const sps_dedisp_config& c, int32_t max_stage_bytes, cudaStream_t st) {
+                                   const sps_dedisp_config& c, int32_t max_stage_bytes, Stream& st) {
   if (n_work < 1 || n_work > 0x7fffffff) return fail(SPS_ERR_UNSUPPORTED, "work list size out of range");
   const Variant* v = find_variant(c.dms_per_thread, c.samples_per_thread / 2);
   if (!v) return fail(SPS_ERR_INVALID_ARG, "no compiled pre-summed variant");
   const size_t smem = presum_smem_bytes(max_stage_bytes);
   SPS_CUDA(cudaFuncSetAttribute(v->list, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  v->list<<<(unsigned)n_work, 32 * c.warps_dm * c.warps_time, smem, st>>>(d_passes, d_work, c.warps_dm);
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, v->list, dim3((unsigned)n_work), 32 * c.warps_dm * c.warps_time, smem, d_passes, d_work,
+                  c.warps_dm));
   return SPS_OK;
 }
 

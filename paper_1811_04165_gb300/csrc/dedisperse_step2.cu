@@ -104,6 +104,7 @@ step2_kernel(Step2Args a, int wd, int cs_max, int wb) {
       }
   };
 
+  pdl_wait();  // step one's rows are written
   if (warp == 0) issue(0);
   // while chunk 0 lands: the staged offset of every (trial, subband).  Window
   // start of subband s = the tile's first trial's delay rounded down to 8
@@ -159,6 +160,7 @@ step2_kernel(Step2Args a, int wd, int cs_max, int wb) {
 #pragma unroll
     for (int m = 0; m < NW; m++) acc[r][m][0] = (int32_t)((uint32_t)acc[r][m][0] - ((uint32_t)acc[r][m][1] << 16));
 
+  pdl_next();
   const bool vec = (a.n_t & 1) == 0;
 #pragma unroll
   for (int r = 0; r < ND; r++) {
@@ -243,6 +245,7 @@ __global__ void __launch_bounds__(256, 2) step2_wide_kernel(Step2Args a, int wd,
 #pragma unroll
   for (int q = 0; q < ND * NW / 2; q++) cnt[q] = 0u;
 
+  pdl_wait();  // step one's rows are written
   if (warp == 0)
     for (int c = 0; c < min(kWideStages - 1, n_chunks); c++) issue(c);
   // while chunk 0 lands: the staged offsets, as above, in words
@@ -336,6 +339,7 @@ __global__ void __launch_bounds__(256, 2) step2_wide_kernel(Step2Args a, int wd,
     }
   }
 
+  pdl_next();
   const bool vec = (a.n_t & 1) == 0;
 #pragma unroll
   for (int r = 0; r < ND; r++) {
@@ -413,16 +417,15 @@ size_t step2_wide_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int3
   return kWideStages * stage + (size_t)c.warps_dm * kWideTrials * n_subbands * 2 + 8 * kWideStages;
 }
 
-sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, cudaStream_t st) {
+sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, Stream& st) {
   if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) {
     const int Tt = c.warps_time * kWideTime;
     const size_t smem = step2_wide_smem_bytes(c, a.dmax_tile, a.n_subbands);
     dim3 grid((a.n_t + Tt - 1) / Tt, a.n_tiles, 1);
     if (grid.y > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many step-two tiles");
     SPS_CUDA(cudaFuncSetAttribute(step2_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    step2_wide_kernel<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, c.chunk,
-                                                                         copy_bytes(c, a.dmax_tile));
-    SPS_CUDA(cudaGetLastError());
+    SPS_CUDA(launch(st, step2_wide_kernel, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
+                    copy_bytes(c, a.dmax_tile)));
     return SPS_OK;
   }
   std::string why;
@@ -433,8 +436,8 @@ sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, cudaStre
   dim3 grid((a.n_t + Tt - 1) / Tt, a.n_tiles, 1);
   if (grid.y > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many step-two tiles");
   SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, c.chunk, copy_bytes(c, a.dmax_tile));
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
+                  copy_bytes(c, a.dmax_tile)));
   return SPS_OK;
 }
 

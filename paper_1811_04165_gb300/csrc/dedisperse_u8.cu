@@ -225,6 +225,7 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
         for (int q = 0; q < 4; q++) acc[r][m][q] = 0;
   };
 
+  pdl_wait();  // the shifted copies are written
   issue(0);
   if (n_chunks > 1) issue(1);
 
@@ -289,6 +290,7 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
       for (int k = ch; k < min(ch + 2, n_chunks); k++) mbar_wait(&bars[k & 1], (k >> 1) & 1, a.status);
     return;
   }
+  pdl_next();
   if constexpr (!WALK) finish_group(g0);
 }
 
@@ -316,6 +318,7 @@ __device__ __forceinline__ void load_raw20(const uint8_t* row, int64_t p, int32_
 // x4[j - 1][c][p] = x[c][p + j] for j = 1..3 (0 at and beyond in_len).
 __global__ void __launch_bounds__(256) expand_kernel(const uint8_t* x, int64_t pitch, int32_t in_len,
                                                      int32_t channels, uint8_t* x4, int64_t pitch4) {
+  pdl_wait();
   const int64_t spr = pitch4 >> 4;
   const int64_t seg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (seg >= spr * channels) return;
@@ -403,14 +406,14 @@ size_t u8_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int32_t grou
 }
 
 sps_status launch_expand(const uint8_t* x, int64_t pitch, int32_t in_len, int32_t channels, uint8_t* x4,
-                         int64_t pitch4, cudaStream_t st) {
+                         int64_t pitch4, Stream& st) {
   const int64_t segs = (pitch4 >> 4) * channels;
-  expand_kernel<<<(unsigned)((segs + 255) / 256), 256, 0, st>>>(x, pitch, in_len, channels, x4, pitch4);
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, expand_kernel, dim3((unsigned)((segs + 255) / 256)), 256, 0, x, pitch, in_len, channels, x4,
+                  pitch4));
   return SPS_OK;
 }
 
-sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& c, cudaStream_t st) {
+sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& c, Stream& st) {
   std::string why;
   if (!u8_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
   const int Di = c.warps_dm * c.dms_per_thread;
@@ -422,9 +425,8 @@ sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& c, cudaS
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, (a.n_groups + gpb - 1) / gpb);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
   SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<grid, 32 * c.warps_dm * c.warps_time, smem, st>>>(a, c.warps_dm, c.chunk, u8_window_bytes(c, a.dmax_tile),
-                                                          gpb);
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
+                  u8_window_bytes(c, a.dmax_tile), gpb));
   return SPS_OK;
 }
 

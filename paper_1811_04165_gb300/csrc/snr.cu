@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(kMaxThreads, FAST ? 2 : 1) snr_kernel(SnrArgs 
   const int i = blockIdx.x;
   const int n_t = a.n_t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  pdl_wait();  // the rows are written
   uint32_t seg = 0;
   if (!load_prefix(a.D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, a.status, &seg)) return;
   const uint32_t* P = buf + kPad - 1;
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(kMaxThreads, FAST ? 2 : 1) snr_kernel(SnrArgs 
     gmax[k] = best;
   }
   __syncthreads();
+  pdl_next();
   // first position of the maximum: the warp of each thread holding it searches
   // that thread's samples (u = owner + m * blockDim.x) together, 32 at a time
 #pragma unroll
@@ -368,6 +370,7 @@ detect_kernel(const double* snr, const int32_t* peak_t, const int32_t* peak_val,
   __shared__ long long cv[kDetectBlocks];  // block 0: the blocks' results
   __shared__ int ci[kDetectBlocks], cw[kDetectBlocks];
   cluster.barrier_arrive();  // matched before the remote writes into block 0
+  pdl_wait();                // the table is written
   const int rank = (int)cluster.block_rank();
   const int total = n_widths * n_dms;  // below 2^31 (checked by the launcher)
   const int stride = kDetectBlocks * (int)blockDim.x;
@@ -589,6 +592,7 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
       if (lane == 0) s1v[k] = (unsigned long long)(1u << k) * T - e;
     }
   }
+  pdl_next();
   // first position of each maximum: the warp of each thread holding it searches
   // that thread's groups, 8 groups (32 outputs) at a time, in order
 #pragma unroll
@@ -632,6 +636,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_pow2_kernel(SnrArgs a) {
   __shared__ uint64_t bar;
   const int row = blockIdx.x;
   const int n_t = a.n_t;
+  pdl_wait();  // the row is written
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     fence_mbar_init();
@@ -853,6 +858,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_stream_kernel(SnrArgs a) {
   uint32_t* ring = dyn + warp * (kRing + 3 * kChunk + NW * 32);
   uint32_t* stage = ring + kRing;
   int* mc = reinterpret_cast<int*>(stage + 3 * kChunk) + lane;
+  pdl_wait();  // the rows are written
   const int n_chunks = (n_t + kChunk - 1) / kChunk;
   const int cb = warp * n_chunks / nwarps, ce = (warp + 1) * n_chunks / nwarps;
 
@@ -910,6 +916,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_stream_kernel(SnrArgs a) {
     gmax[k] = m;
   }
   __syncthreads();
+  pdl_next();
   // the earliest chunk holding each width's maximum
 #pragma unroll
   for (int k = 0; k < NW; k++)
@@ -1063,7 +1070,17 @@ size_t stream_smem(int nw, int threads) {
   return (size_t)(threads / 32) * (kRing + 3 * kChunk + nw * 32) * sizeof(uint32_t);
 }
 
-sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, cudaStream_t st) {
+// The detection, when asked for.
+sps_status launch_detect(const SnrArgs& a, Stream& st) {
+  if (!a.best) return SPS_OK;
+  if ((int64_t)a.n_widths * a.n_dms >= (int64_t)1 << 31)
+    return fail(SPS_ERR_UNSUPPORTED, "S/N table too large for the detection's 32-bit indices");
+  SPS_CUDA(launch(st, detect_kernel, dim3(kDetectBlocks), kDetectThreads, 0, a.snr, a.peak_t, a.peak_val, a.n_dms,
+                  a.n_widths, a.best));
+  return SPS_OK;
+}
+
+sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
   std::string why;
   if (!snr_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
   if (pow2_form(a) && !row_fits(a.n_t, pow2_smem(a.n_t, a.pow2_widths) - prefix_smem(a.n_t) + 8192) &&
@@ -1072,32 +1089,16 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, cudaStream_t st
     const size_t smem = stream_smem(a.pow2_widths, c.threads);
     StreamKernel fn = stream_variant(a.pow2_widths);
     SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    fn<<<a.n_dms, c.threads, smem, st>>>(a);
-    SPS_CUDA(cudaGetLastError());
-    if (a.best && (int64_t)a.n_widths * a.n_dms >= (int64_t)1 << 31)
-      return fail(SPS_ERR_UNSUPPORTED, "S/N table too large for the detection's 32-bit indices");
-    if (a.best) {
-      detect_kernel<<<kDetectBlocks, kDetectThreads, 0, st>>>(a.snr, a.peak_t, a.peak_val, a.n_dms, a.n_widths,
-                                                              a.best);
-      SPS_CUDA(cudaGetLastError());
-    }
-    return SPS_OK;
+    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a));
+    return launch_detect(a, st);
   }
   if (pow2_form(a)) {
     const size_t smem = pow2_smem(a.n_t, a.pow2_widths);
     if (sps_status s = check_row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192)) return s;
     Pow2Kernel fn = pow2_variant(a.pow2_widths);
     SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    fn<<<a.n_dms, c.threads, smem, st>>>(a);
-    SPS_CUDA(cudaGetLastError());
-    if (a.best && (int64_t)a.n_widths * a.n_dms >= (int64_t)1 << 31)
-      return fail(SPS_ERR_UNSUPPORTED, "S/N table too large for the detection's 32-bit indices");
-    if (a.best) {
-      detect_kernel<<<kDetectBlocks, kDetectThreads, 0, st>>>(a.snr, a.peak_t, a.peak_val, a.n_dms, a.n_widths,
-                                                              a.best);
-      SPS_CUDA(cudaGetLastError());
-    }
-    return SPS_OK;
+    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a));
+    return launch_detect(a, st);
   }
   if (sps_status s = check_row_fits(a.n_t, sizeof(Moments) * (kMaxThreads / 32) * kWidthsPerPass + 512)) return s;
   // largest boxcar value: 255 * channels * widest width (< 2^31, checked by the plan);
@@ -1117,25 +1118,18 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, cudaStream_t st
     SnrKernel fn = a.decimate ? (fast ? snr_variant<true, true>(nwp) : snr_variant<true, false>(nwp))
                               : (fast ? snr_variant<false, true>(nwp) : snr_variant<false, false>(nwp));
     SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    fn<<<a.n_dms, c.threads, smem, st>>>(a, w0, flush, tma_ok(a.D, a.n_t) ? 1 : 0, narrow);
-    SPS_CUDA(cudaGetLastError());
+    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a, w0, flush, tma_ok(a.D, a.n_t) ? 1 : 0, narrow));
   }
-  if (a.best) {
-    detect_kernel<<<kDetectBlocks, kDetectThreads, 0, st>>>(a.snr, a.peak_t, a.peak_val, a.n_dms, a.n_widths,
-                                                            a.best);
-    SPS_CUDA(cudaGetLastError());
-  }
-  return SPS_OK;
+  return launch_detect(a, st);
 }
 
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
-                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, cudaStream_t st) {
+                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, Stream& st) {
   if (sps_status s = check_row_fits(n_t, 256)) return s;
   const size_t smem = prefix_smem(n_t);
   SPS_CUDA(cudaFuncSetAttribute(integrate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  integrate_kernel<<<n_dms, 256, smem, st>>>(D, n_dms, n_t, widths, n_widths, B, tma_ok(D, n_t) ? 1 : 0, decimate,
-                                             status);
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, integrate_kernel, dim3(n_dms), 256, smem, D, n_dms, n_t, widths, n_widths, B,
+                  tma_ok(D, n_t) ? 1 : 0, decimate, status));
   return SPS_OK;
 }
 

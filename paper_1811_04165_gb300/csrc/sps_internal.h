@@ -37,6 +37,41 @@ void clear_error();
     if (e_ != cudaSuccess) return ::sps::cuda_fail(e_, #call); \
   } while (0)
 
+// The stream of one call, and how its kernels follow one another: a kernel
+// after the call's first may be put on the GPU while the one before it runs its
+// last blocks (programmatic dependent launch); it waits in pdl_wait() (tma.cuh)
+// until that one has completed, before it touches global memory.  The call's
+// first kernel is an ordinary launch, so calls follow one another as streams do.
+// Off while the stream is being captured into a graph.
+struct Stream {
+  cudaStream_t st;
+  bool overlap = false;
+  bool first = true;
+  explicit Stream(cudaStream_t s) : st(s) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) == cudaSuccess)
+      overlap = c == cudaStreamCaptureStatusNone;
+    else
+      cudaGetLastError();
+  }
+};
+
+template <class... P, class... A>
+cudaError_t launch(Stream& s, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, A... args) {
+  cudaLaunchAttribute after{};
+  after.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  after.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s.st;
+  c.attrs = &after;
+  c.numAttrs = s.overlap && !s.first ? 1 : 0;
+  s.first = false;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Kernel-side description of one de-dispersion pass over uint8 channels
 // (brute force, or subband step one with one output row per (coarse, subband)).
 struct U8PassArgs {
@@ -157,28 +192,28 @@ struct SnrArgs {
 // snr.cu, zap.cu).  launch_snr also writes the detection when SnrArgs::best is
 // set.  They validate the configuration
 // against the kernel's compiled variants and return UNSUPPORTED otherwise.
-sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& cfg, cudaStream_t st);
-sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& cfg, cudaStream_t st);
-sps_status launch_snr(const SnrArgs& a, const sps_snr_config& cfg, cudaStream_t st);
+sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& cfg, Stream& st);
+sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& cfg, Stream& st);
+sps_status launch_snr(const SnrArgs& a, const sps_snr_config& cfg, Stream& st);
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
-                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, cudaStream_t st);
+                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, Stream& st);
 sps_status launch_expand(const uint8_t* x, int64_t pitch, int32_t in_len, int32_t channels, uint8_t* x4,
-                         int64_t pitch4, cudaStream_t st);
+                         int64_t pitch4, Stream& st);
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
                                 int32_t n_units, int32_t unit_channels, int32_t max_rel, const PresumSeries* series,
                                 int32_t n_series, uint16_t* q, int32_t q_pitch, int32_t* zero, int64_t n_zero,
-                                cudaStream_t st);
-sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& cfg, cudaStream_t st);
+                                Stream& st);
+sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& cfg, Stream& st);
 // Batched pre-summed pass: one launch over the work list of several passes of
 // configuration `cfg` (d_passes / d_work in device memory; max_stage_bytes =
 // the largest stage_bytes of the passes).  presum_pass_work appends the work
 // items of pass index `pass`; presum_pass_blocks counts them.
 sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d_work, int64_t n_work,
-                                   const sps_dedisp_config& cfg, int32_t max_stage_bytes, cudaStream_t st);
+                                   const sps_dedisp_config& cfg, int32_t max_stage_bytes, Stream& st);
 void presum_pass_work(const PresumPassArgs& a, const sps_dedisp_config& cfg, int32_t pass, std::vector<int4>* work);
 int64_t presum_pass_blocks(const PresumPassArgs& a, const sps_dedisp_config& cfg);
 sps_status launch_zap_copy(const uint8_t* x, int64_t pitch, int32_t in_len, const uint8_t* zap, int32_t channels,
-                           uint8_t* out, int64_t out_pitch, cudaStream_t st);
+                           uint8_t* out, int64_t out_pitch, Stream& st);
 bool presum_config_supported(const sps_dedisp_config& cfg, std::string* why);
 size_t presum_smem_bytes(int32_t stage_bytes);
 int presum_window_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile);

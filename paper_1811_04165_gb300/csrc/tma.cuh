@@ -32,6 +32,16 @@ __device__ __forceinline__ bool stage_read_ok(uint32_t off, int64_t limit, uint3
 // than any copy this library issues takes.
 constexpr uint32_t kMaxPolls = 1u << 22;
 
+// Waits until the kernel before this one in the call has completed and its
+// writes are visible (returns at once in an ordinary launch).  Every kernel that
+// may be launched beside its predecessor calls it before it touches memory that
+// an earlier kernel writes or reads.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the next kernel of the call be put on the GPU once every block has
+// started; it waits in pdl_wait() for this one to complete.
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

@@ -31,10 +31,10 @@ __global__ void __launch_bounds__(256) zap_copy_kernel(const uint8_t* x, int64_t
 }  // namespace
 
 sps_status launch_zap_copy(const uint8_t* x, int64_t pitch, int32_t in_len, const uint8_t* zap, int32_t channels,
-                           uint8_t* out, int64_t out_pitch, cudaStream_t st) {
+                           uint8_t* out, int64_t out_pitch, Stream& st) {
   const int64_t threads = (out_pitch >> 4) * channels;
-  zap_copy_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(x, pitch, in_len, zap, channels, out, out_pitch);
-  SPS_CUDA(cudaGetLastError());
+  SPS_CUDA(launch(st, zap_copy_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, x, pitch, in_len, zap,
+                  channels, out, out_pitch));
   return SPS_OK;
 }
 
