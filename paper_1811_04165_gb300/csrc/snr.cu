@@ -2,7 +2,7 @@
 // de-dispersed series, then S/N; the sliding-boxcar reading of "smoothing").
 //
 // One block per DM row.  The row arrives in shared memory by one bulk copy
-// (TMA) and is turned in place into prefix sums P[t] = sum_{u<t} D[u] (32-bit
+// (TMA; whatever its length and place, see stage_row) and is turned in place into prefix sums P[t] = sum_{u<t} D[u] (32-bit
 // wrap-around arithmetic: every boxcar B_w[t] = P[t + w] - P[t] is below 2^31,
 // so the wrapped difference is exact).  A single pass over t then serves all
 // widths of the pass at once, accumulating per width the exact integer moment
@@ -29,6 +29,7 @@ namespace {
 
 constexpr int kMaxThreads = 512;
 constexpr int kWidthsPerPass = 8;
+constexpr int kFactorsPerPass = 12;  // decimating
 constexpr int kPad = 4;  // P[k] lives at buf[kPad - 1 + k]; the row lands at buf[kPad]
 
 // Block-wide exclusive prefix sum (uint32, wrap-around) of one value per thread.
@@ -57,18 +58,64 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch) {
   return base + x - v;
 }
 
-// Load row i into buf[kPad .. kPad + n_t) and turn it into prefix sums in place:
-// afterwards buf[kPad - 1 + k] = sum_{u<k} D[u] for k = 0..n_t.  *seg = the sum
-// of the samples this thread scanned (the threads' segments tile the row).
-__device__ bool load_prefix(const int32_t* row, int n_t, uint32_t* buf, uint32_t* scratch, uint64_t* bar,
-                            bool use_tma, uint32_t* status, uint32_t* seg) {
+// Scans the row at buf[4 .. 4 + n_t) in place into P[k] = buf[3 + k] (k = 0 ..
+// n_t); returns the sum of the samples this thread scanned.  Each thread scans
+// a run of `per` samples (a multiple of 4 with per / 4 odd, so the 16-byte
+// accesses of a warp are conflict-free).
+__device__ uint32_t scan_row_v4(uint32_t* buf, int n_t, uint32_t* scratch) {
+  if (threadIdx.x == 0) buf[3] = 0u;
+  int per = ((n_t + blockDim.x - 1) / blockDim.x + 3) / 4 * 4;
+  if ((per / 4) % 2 == 0) per += 4;
+  const int b = min(n_t, (int)threadIdx.x * per), e = min(n_t, b + per);
+  const int ev = b + (e - b) / 4 * 4;  // vector part [b, ev)
+  uint32_t s = 0;
+  for (int t = b; t < ev; t += 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
+    s += v.x + v.y + v.z + v.w;
+  }
+  for (int t = ev; t < e; t++) s += buf[4 + t];
+  uint32_t run = block_exclusive_scan(s, scratch);
+  for (int t = b; t < ev; t += 4) {
+    uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
+    v.x += run;
+    v.y += v.x;
+    v.z += v.y;
+    v.w += v.z;
+    run = v.w;
+    *reinterpret_cast<uint4*>(buf + 4 + t) = v;
+  }
+  for (int t = ev; t < e; t++) {
+    run += buf[4 + t];
+    buf[4 + t] = run;
+  }
+  __syncthreads();
+  return s;
+}
+
+// Brings a row of n_t samples into buf[kPad + s + t], t < n_t, with s zeros before
+// it: s is what makes the row's 16-byte aligned part land on 16 bytes, so that one
+// bulk copy (TMA) takes it whatever the row's length and place; up to three samples
+// at either end are loaded by themselves.  Without `use_tma` (no room for s) s is 0
+// and the whole row is loaded that way.  *s_out = s; false when the copy did not
+// land in time.
+__device__ bool stage_row(const int32_t* row, int n_t, uint32_t* buf, uint64_t* bar, bool use_tma, uint32_t* status,
+                          int* s_out) {
+  const int s = use_tma ? (int)((uintptr_t)row >> 2) & 3 : 0;
+  *s_out = s;
   bool ok = true;
   if (use_tma) {
+    const int head = min(n_t, (4 - s) & 3), body = (n_t - head) & ~3, tail = n_t - head - body;
     if (threadIdx.x == 0) {
       mbar_init(bar, 1);
       fence_mbar_init();
-      mbar_arrive_expect_tx(bar, (uint32_t)n_t * 4u);
-      bulk_g2s(buf + kPad, row, (uint32_t)n_t * 4u, bar);
+      mbar_arrive_expect_tx(bar, (uint32_t)body * 4u);
+      if (body) bulk_g2s(buf + kPad + s + head, row + head, (uint32_t)body * 4u, bar);
+    }
+    if ((int)threadIdx.x < s) buf[kPad + threadIdx.x] = 0u;
+    if ((int)threadIdx.x < head) buf[kPad + s + threadIdx.x] = (uint32_t)__ldg(row + threadIdx.x);
+    if ((int)threadIdx.x < tail) {
+      const int t = head + body + (int)threadIdx.x;
+      buf[kPad + s + t] = (uint32_t)__ldg(row + t);
     }
     __syncthreads();
     ok = mbar_wait(bar, 0, status);
@@ -80,22 +127,20 @@ __device__ bool load_prefix(const int32_t* row, int n_t, uint32_t* buf, uint32_t
     }
   } else {
     for (int t = threadIdx.x; t < n_t; t += blockDim.x) buf[kPad + t] = (uint32_t)__ldg(row + t);
+    __syncthreads();
   }
-  if (threadIdx.x == 0) buf[kPad - 1] = 0u;
-  __syncthreads();
-  // odd segment lengths keep the strided shared accesses free of bank conflicts
-  const int per = ((n_t + blockDim.x - 1) / blockDim.x) | 1;
-  const int b = min(n_t, (int)threadIdx.x * per), e = min(n_t, b + per);
-  uint32_t s = 0;
-  for (int t = b; t < e; t++) s += buf[kPad + t];
-  *seg = s;
-  uint32_t run = block_exclusive_scan(s, scratch);
-  for (int t = b; t < e; t++) {
-    run += buf[kPad + t];
-    buf[kPad + t] = run;
-  }
-  __syncthreads();
-  return ok;
+  return true;
+}
+
+// The row staged and scanned: (*P)[k] = sum_{u<k} D[u] for k = 0..n_t.  *seg = the
+// sum of the samples this thread scanned (the threads' segments tile the row).
+__device__ bool load_prefix(const int32_t* row, int n_t, uint32_t* buf, uint32_t* scratch, uint64_t* bar,
+                            bool use_tma, uint32_t* status, uint32_t* seg, const uint32_t** P) {
+  int s = 0;
+  if (!stage_row(row, n_t, buf, bar, use_tma, status, &s)) return false;
+  *seg = scan_row_v4(buf, n_t + s, scratch);
+  *P = buf + kPad - 1 + s;
+  return true;
 }
 
 struct Moments {
@@ -173,8 +218,8 @@ __global__ void __launch_bounds__(kMaxThreads, FAST ? 2 : 1) snr_kernel(SnrArgs 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   pdl_wait();  // the rows are written
   uint32_t seg = 0;
-  if (!load_prefix(a.D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, a.status, &seg)) return;
-  const uint32_t* P = buf + kPad - 1;
+  const uint32_t* P;
+  if (!load_prefix(a.D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, a.status, &seg, &P)) return;
 
   int W[NWP];
   uint32_t mx[NWP];
@@ -327,8 +372,8 @@ integrate_kernel(const int32_t* D, int n_dms, int n_t, const int32_t* widths, in
   __shared__ uint64_t bar;
   const int i = blockIdx.x;
   uint32_t seg = 0;
-  if (!load_prefix(D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, status, &seg)) return;
-  const uint32_t* P = buf + kPad - 1;
+  const uint32_t* P;
+  if (!load_prefix(D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, status, &seg, &P)) return;
   for (int wi = 0; wi < n_widths; wi++) {
     const int w = __ldg(widths + wi);
     const int N = decimate ? n_t / w : n_t - w + 1;
@@ -360,6 +405,73 @@ __device__ __forceinline__ bool better(long long v, int i, int w, long long bv, 
 constexpr int kDetectBlocks = 8;
 constexpr int kDetectThreads = 1024;
 
+// The best entry of a block's threads, left in warp 0's lane 0.
+__device__ __forceinline__ void block_best(long long& bv, int& bi, int& bw, long long* sv, int* si, int* sw) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto warp_best = [&]() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long v = __shfl_down_sync(0xffffffffu, bv, o);
+      const int i = __shfl_down_sync(0xffffffffu, bi, o), w = __shfl_down_sync(0xffffffffu, bw, o);
+      if (better(v, i, w, bv, bi, bw)) { bv = v; bi = i; bw = w; }
+    }
+  };
+  warp_best();
+  if (lane == 0) { sv[warp] = bv; si[warp] = bi; sw[warp] = bw; }
+  __syncthreads();
+  if (warp == 0) {
+    bv = lane < nw ? sv[lane] : LLONG_MIN;
+    bi = lane < nw ? si[lane] : 0x7fffffff;
+    bw = lane < nw ? sw[lane] : 0x7fffffff;
+    warp_best();
+  }
+}
+
+// The best of the entries e0, e0 + stride, ... below `total` (below 2^31, checked
+// by the launcher).
+__device__ __forceinline__ void scan_table(const double* snr, int n_dms, int total, int e0, int stride, long long& bv,
+                                           int& bi, int& bw) {
+  const long long* key = reinterpret_cast<const long long*>(snr);
+  bv = LLONG_MIN;
+  bi = bw = 0x7fffffff;
+  constexpr int kIn = 4;  // table reads in flight per thread
+  for (; e0 < total; e0 += kIn * stride) {
+    long long v[kIn];
+#pragma unroll
+    for (int u = 0; u < kIn; u++) v[u] = e0 + u * stride < total ? key[e0 + u * stride] : LLONG_MIN;
+#pragma unroll
+    for (int u = 0; u < kIn; u++) {
+      const int e = e0 + u * stride;
+      if (e >= total) break;
+      const int w = e / n_dms, i = e - w * n_dms;
+      if (better(v[u], i, w, bv, bi, bw)) { bv = v[u]; bi = i; bw = w; }
+    }
+  }
+}
+
+// Small tables: one block (up to 4096 entries 0.8 us less than the cluster; at
+// 14336 entries 2 us more).
+constexpr int kDetectSmall = 4096;
+
+__global__ void __launch_bounds__(kDetectThreads, 1)
+detect_small_kernel(const double* snr, const int32_t* peak_t, const int32_t* peak_val, int n_dms, int n_widths,
+                    int32_t* best) {
+  __shared__ long long sv[32];
+  __shared__ int si[32], sw[32];
+  pdl_wait();  // the table is written
+  long long bv;
+  int bi, bw;
+  scan_table(snr, n_dms, n_widths * n_dms, (int)threadIdx.x, (int)blockDim.x, bv, bi, bw);
+  block_best(bv, bi, bw, sv, si, sw);
+  if (threadIdx.x == 0) {
+    const int64_t o = (int64_t)bw * n_dms + bi;
+    best[0] = bi;
+    best[1] = bw;
+    best[2] = peak_t[o];
+    best[3] = peak_val[o];
+  }
+}
+
 __global__ void __cluster_dims__(kDetectBlocks, 1, 1) __launch_bounds__(kDetectThreads, 1)
 detect_kernel(const double* snr, const int32_t* peak_t, const int32_t* peak_val, int n_dms, int n_widths,
               int32_t* best) {
@@ -372,46 +484,13 @@ detect_kernel(const double* snr, const int32_t* peak_t, const int32_t* peak_val,
   cluster.barrier_arrive();  // matched before the remote writes into block 0
   pdl_wait();                // the table is written
   const int rank = (int)cluster.block_rank();
-  const int total = n_widths * n_dms;  // below 2^31 (checked by the launcher)
-  const int stride = kDetectBlocks * (int)blockDim.x;
-  const long long* key = reinterpret_cast<const long long*>(snr);
-  long long bv = LLONG_MIN;
-  int bi = 0x7fffffff, bw = 0x7fffffff;
-  constexpr int kIn = 4;  // table reads in flight per thread
-  for (int e0 = rank * (int)blockDim.x + (int)threadIdx.x; e0 < total; e0 += kIn * stride) {
-    long long v[kIn];
-#pragma unroll
-    for (int u = 0; u < kIn; u++) v[u] = e0 + u * stride < total ? key[e0 + u * stride] : LLONG_MIN;
-#pragma unroll
-    for (int u = 0; u < kIn; u++) {
-      const int e = e0 + u * stride;
-      if (e >= total) break;
-      const int w = e / n_dms, i = e - w * n_dms;
-      if (better(v[u], i, w, bv, bi, bw)) { bv = v[u]; bi = i; bw = w; }
-    }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long v = __shfl_down_sync(0xffffffffu, bv, o);
-    const int i = __shfl_down_sync(0xffffffffu, bi, o), w = __shfl_down_sync(0xffffffffu, bw, o);
-    if (better(v, i, w, bv, bi, bw)) { bv = v; bi = i; bw = w; }
-  }
-  if (lane == 0) { sv[warp] = bv; si[warp] = bi; sw[warp] = bw; }
-  __syncthreads();
-  if (warp == 0) {
-    bv = lane < nw ? sv[lane] : LLONG_MIN;
-    bi = lane < nw ? si[lane] : 0x7fffffff;
-    bw = lane < nw ? sw[lane] : 0x7fffffff;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long v = __shfl_down_sync(0xffffffffu, bv, o);
-      const int i = __shfl_down_sync(0xffffffffu, bi, o), w = __shfl_down_sync(0xffffffffu, bw, o);
-      if (better(v, i, w, bv, bi, bw)) { bv = v; bi = i; bw = w; }
-    }
-  }
+  long long bv;
+  int bi, bw;
+  scan_table(snr, n_dms, n_widths * n_dms, rank * (int)blockDim.x + (int)threadIdx.x, kDetectBlocks * (int)blockDim.x,
+             bv, bi, bw);
+  block_best(bv, bi, bw, sv, si, sw);
   cluster.barrier_wait();  // every block of the cluster has started
-  if (warp == 0 && lane == 0) {
+  if (threadIdx.x == 0) {
     *cluster.map_shared_rank(&cv[rank], 0) = bv;
     *cluster.map_shared_rank(&ci[rank], 0) = bi;
     *cluster.map_shared_rank(&cw[rank], 0) = bw;
@@ -449,40 +528,6 @@ detect_kernel(const double* snr, const int32_t* peak_t, const int32_t* peak_val,
 //
 // The detection follows as its own one-cluster launch (detect_kernel).
 
-// Scans the row at buf[4 .. 4 + n_t) in place into P[k] = buf[3 + k] (k = 0 ..
-// n_t); returns the sum of the samples this thread scanned.  Each thread scans
-// a run of `per` samples (a multiple of 4 with per / 4 odd, so the 16-byte
-// accesses of a warp are conflict-free).
-__device__ uint32_t scan_row_v4(uint32_t* buf, int n_t, uint32_t* scratch) {
-  if (threadIdx.x == 0) buf[3] = 0u;
-  int per = ((n_t + blockDim.x - 1) / blockDim.x + 3) / 4 * 4;
-  if ((per / 4) % 2 == 0) per += 4;
-  const int b = min(n_t, (int)threadIdx.x * per), e = min(n_t, b + per);
-  const int ev = b + (e - b) / 4 * 4;  // vector part [b, ev)
-  uint32_t s = 0;
-  for (int t = b; t < ev; t += 4) {
-    const uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
-    s += v.x + v.y + v.z + v.w;
-  }
-  for (int t = ev; t < e; t++) s += buf[4 + t];
-  uint32_t run = block_exclusive_scan(s, scratch);
-  for (int t = b; t < ev; t += 4) {
-    uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
-    v.x += run;
-    v.y += v.x;
-    v.z += v.y;
-    v.w += v.z;
-    run = v.w;
-    *reinterpret_cast<uint4*>(buf + 4 + t) = v;
-  }
-  for (int t = ev; t < e; t++) {
-    run += buf[4 + t];
-    buf[4 + t] = run;
-  }
-  __syncthreads();
-  return s;
-}
-
 // S2 += B * B, a 32 x 32 -> 64-bit product added to a 64-bit sum (written in
 // C++: measured slightly faster on sm_103a than the explicit mad.wide.u32).
 __device__ __forceinline__ void add_square(unsigned long long& acc, uint32_t b) {
@@ -503,14 +548,16 @@ __device__ __forceinline__ uint32_t quad(const uint4& v, int i) {
 }
 
 // Moments, maxima and first peak positions of one scanned row for widths 1, 2,
-// ..., 2^(NW-1), written to the row's S/N, peak_t and peak_val entries.
+// ..., 2^(NW-1), written to the row's S/N, peak_t and peak_val entries.  The row
+// starts s zeros into the buffer (stage_row), so positions below count from those
+// and outputs start at s.
 template <int NW>
-__device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uint32_t segsum) {
+__device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uint32_t segsum, int s) {
   constexpr int WMAX = 1 << (NW - 1);
   __shared__ unsigned long long ps2[kMaxThreads / 32][NW], ptot[kMaxThreads / 32], s1v[NW];
   __shared__ uint32_t pmx[kMaxThreads / 32][NW];
   __shared__ int gmax[NW], first[NW];
-  const int n_t = a.n_t;
+  const int n_t = a.n_t + s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t* P = buf + 3;  // P[k], k = 0 .. n_t
   const int n_grp = (n_t + 3 + 3) / 4;  // groups of t = 4j - 3 .. 4j covering 0 .. n_t - 1
@@ -521,7 +568,7 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
   if (threadIdx.x < NW) first[threadIdx.x] = 0x7fffffff;
   for (int j = threadIdx.x; j < n_grp; j += blockDim.x) {
     const int t0 = 4 * j - 3;
-    if (t0 >= 0 && t0 + 3 + WMAX <= n_t) {
+    if (t0 >= s && t0 + 3 + WMAX <= n_t) {
       // every output of the group is valid for every width
       const uint4 A = *reinterpret_cast<const uint4*>(buf + 4 * j);      // P[t0 .. t0 + 3]
       const uint4 N = *reinterpret_cast<const uint4*>(buf + 4 * j + 4);  // P[t0 + 4 .. t0 + 7]
@@ -546,7 +593,7 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
 #pragma unroll 1
         for (int i = 0; i < 4; i++) {
           const int t = t0 + i;
-          if (t >= 0 && t + w <= n_t) {
+          if (t >= s && t + w <= n_t) {
             const uint32_t B = P[t + w] - P[t];
             add_square(s2[k], B);
             mx[k] = max(mx[k], B);
@@ -583,8 +630,8 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
     for (int q = 0; q < nw; q++) T += ptot[q];
     uint32_t e0 = 0u, e1 = 0u;
     const int j0 = lane + 1, j1 = lane + 33;
-    if (j0 < WMAX) e0 = P[j0] + (P[n_t] - P[n_t - j0]);
-    if (j1 < WMAX) e1 = P[j1] + (P[n_t] - P[n_t - j1]);
+    if (j0 < WMAX) e0 = P[s + j0] + (P[n_t] - P[n_t - j0]);
+    if (j1 < WMAX) e1 = P[s + j1] + (P[n_t] - P[n_t - j1]);
 #pragma unroll
     for (int k = 0; k < NW; k++) {
       const unsigned long long e = warp_sum64_redux((unsigned long long)(j0 < (1 << k) ? e0 : 0u) +
@@ -607,7 +654,7 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
         // lane -> group owner + (m0 + lane / 4) * blockDim, output lane % 4 of it
         const int j = owner + (m0 + (lane >> 2)) * (int)blockDim.x;
         const int t = 4 * j - 3 + (lane & 3);
-        const bool hit = j < n_grp && t >= 0 && t + w <= n_t && (int)(P[t + w] - P[t]) == gmax[k];
+        const bool hit = j < n_grp && t >= s && t + w <= n_t && (int)(P[t + w] - P[t]) == gmax[k];
         const unsigned h = __ballot_sync(0xffffffffu, hit);
         if (h) {
           const int l = __ffs(h) - 1;
@@ -623,8 +670,8 @@ __device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uin
     Moments r{s1v[k], ps2[0][k], 0ull, gmax[k], 0};
     for (int q = 1; q < nw; q++) r.s2lo += ps2[q][k];
     const int64_t o = (int64_t)k * a.n_dms + row;
-    a.snr[o] = snr_from_moments(n_t - (1 << k) + 1, r);
-    a.peak_t[o] = first[k];
+    a.snr[o] = snr_from_moments(a.n_t - (1 << k) + 1, r);
+    a.peak_t[o] = first[k] - s;
     a.peak_val[o] = gmax[k];
   }
 }
@@ -635,24 +682,11 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_pow2_kernel(SnrArgs a) {
   __shared__ uint32_t scratch[32];
   __shared__ uint64_t bar;
   const int row = blockIdx.x;
-  const int n_t = a.n_t;
   pdl_wait();  // the row is written
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    fence_mbar_init();
-    mbar_arrive_expect_tx(&bar, (uint32_t)n_t * 4u);
-    bulk_g2s(buf + 4, a.D + (int64_t)row * n_t, (uint32_t)n_t * 4u, &bar);
-  }
-  __syncthreads();
-  const bool ok = mbar_wait(&bar, 0, a.status);
-  if (__syncthreads_or(ok ? 0 : 1)) {
-    // a copy that did not land in time may still be in flight: one more
-    // bounded wait before the block's shared memory is released
-    if (threadIdx.x == 0) mbar_wait(&bar, 0, a.status);
-    return;
-  }
-  const uint32_t segsum = scan_row_v4(buf, n_t, scratch);
-  row_stats_v4<NW>(a, buf, row, segsum);
+  int s = 0;
+  if (!stage_row(a.D + (int64_t)row * a.n_t, a.n_t, buf, &bar, true, a.status, &s)) return;
+  const uint32_t segsum = scan_row_v4(buf, a.n_t + s, scratch);
+  row_stats_v4<NW>(a, buf, row, segsum, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1010,8 +1044,17 @@ SnrKernel snr_variant(int nwp) {
     case 5: return snr_kernel<5, DEC, FAST>;
     case 6: return snr_kernel<6, DEC, FAST>;
     case 7: return snr_kernel<7, DEC, FAST>;
-    default: return snr_kernel<8, DEC, FAST>;
+    case 8: return snr_kernel<8, DEC, FAST>;
   }
+  if constexpr (DEC) {
+    switch (nwp) {
+      case 9: return snr_kernel<9, DEC, FAST>;
+      case 10: return snr_kernel<10, DEC, FAST>;
+      case 11: return snr_kernel<11, DEC, FAST>;
+      default: return snr_kernel<12, DEC, FAST>;
+    }
+  }
+  return nullptr;
 }
 
 typedef void (*Pow2Kernel)(SnrArgs);
@@ -1029,10 +1072,11 @@ Pow2Kernel pow2_variant(int nw) {
 }
 
 // The vector kernel serves sliding boxcars of widths 1, 2, ..., 2^(NW-1)
-// (NW <= 7) on rows that a bulk copy can stage (16-byte aligned, a multiple
-// of 4 samples) whose sums of squares fit 64 bits; it has no decimating form.
+// (NW <= 7) whose sums of squares fit 64 bits; it has no decimating form.  Rows of
+// any length and place: 517 rows of 7013 samples took 21.0 us in the general
+// kernel, 15.0 here (like 7012).
 bool pow2_form(const SnrArgs& a) {
-  if (a.decimate || a.pow2_widths < 1 || a.pow2_widths > 7 || !tma_ok(a.D, a.n_t)) return false;
+  if (a.decimate || a.pow2_widths < 1 || a.pow2_widths > 7) return false;
   const long double bmax = (long double)std::max<int64_t>(1, a.max_boxcar);
   return (long double)a.n_t * bmax * bmax < 1.8e19L;
 }
@@ -1070,11 +1114,32 @@ size_t stream_smem(int nw, int threads) {
   return (size_t)(threads / 32) * (kRing + 3 * kChunk + nw * 32) * sizeof(uint32_t);
 }
 
+// Threads per row.  The default (256) leaves the choice to the library: where the
+// rows fill the GPU, short ones take fewer threads each, so that more rows share an
+// SM and a row's barriers join fewer warps (4096 rows of 1000 samples, widths 1 ..
+// 64: 46 us with 256 threads, 22 with 64; of 7000 samples 79 and, with 128, 68; of
+// 12500 samples 109 against 119 with 128); decimation does less work per sample
+// (4096 rows of 4096 samples 49 -> 24 us with 32).  Few rows keep 256 (32 rows of
+// 12500 samples: 11 us, 20 with 64).
+int snr_threads(const SnrArgs& a, int threads) {
+  if (threads != 256 || a.n_dms <= 152) return threads;
+  if (a.decimate) return a.n_dms > 608 && a.n_t <= 4500 ? 32 : (a.n_t <= 8000 ? 64 : 96);
+  if (a.n_dms <= 608) return a.n_t <= 3000 ? 128 : 256;
+  return a.n_t <= 4500 ? 64 : (a.n_t <= 10500 ? 128 : 256);
+}
+
 // The detection, when asked for.
 sps_status launch_detect(const SnrArgs& a, Stream& st) {
   if (!a.best) return SPS_OK;
   if ((int64_t)a.n_widths * a.n_dms >= (int64_t)1 << 31)
     return fail(SPS_ERR_UNSUPPORTED, "S/N table too large for the detection's 32-bit indices");
+  const int total = a.n_widths * a.n_dms;
+  if (total <= kDetectSmall) {
+    const unsigned threads = (unsigned)std::max(32, std::min(kDetectThreads, (total + 127) / 128 * 32));
+    SPS_CUDA(launch(st, detect_small_kernel, dim3(1), threads, 0, a.snr, a.peak_t, a.peak_val, a.n_dms, a.n_widths,
+                    a.best));
+    return SPS_OK;
+  }
   SPS_CUDA(launch(st, detect_kernel, dim3(kDetectBlocks), kDetectThreads, 0, a.snr, a.peak_t, a.peak_val, a.n_dms,
                   a.n_widths, a.best));
   return SPS_OK;
@@ -1083,42 +1148,53 @@ sps_status launch_detect(const SnrArgs& a, Stream& st) {
 sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
   std::string why;
   if (!snr_config_supported(c, &why)) return fail(SPS_ERR_INVALID_ARG, why);
-  if (pow2_form(a) && !row_fits(a.n_t, pow2_smem(a.n_t, a.pow2_widths) - prefix_smem(a.n_t) + 8192) &&
-      stream_form(a)) {
-    // rows too long to stage whole: the streaming form, any row length
-    const size_t smem = stream_smem(a.pow2_widths, c.threads);
-    StreamKernel fn = stream_variant(a.pow2_widths);
-    SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a));
-    return launch_detect(a, st);
-  }
+  // rows that do not all start on 16 bytes need room for up to three zeros each
+  const bool aligned = tma_ok(a.D, a.n_t);
+  const int room = aligned ? 0 : 3;
+  const unsigned threads = (unsigned)snr_threads(a, c.threads);
   if (pow2_form(a)) {
-    const size_t smem = pow2_smem(a.n_t, a.pow2_widths);
-    if (sps_status s = check_row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192)) return s;
-    Pow2Kernel fn = pow2_variant(a.pow2_widths);
-    SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a));
-    return launch_detect(a, st);
+    const size_t smem = pow2_smem(a.n_t + room, a.pow2_widths);
+    const bool fits = row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192);
+    if (aligned && !fits && stream_form(a)) {
+      // rows too long to stage whole: the streaming form, any row length
+      const size_t stream = stream_smem(a.pow2_widths, c.threads);
+      StreamKernel fn = stream_variant(a.pow2_widths);
+      SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stream));
+      SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, stream, a));
+      return launch_detect(a, st);
+    }
+    if (aligned && !fits) return check_row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192);
+    if (fits) {
+      Pow2Kernel fn = pow2_variant(a.pow2_widths);
+      SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      SPS_CUDA(launch(st, fn, dim3(a.n_dms), threads, smem, a));
+      return launch_detect(a, st);
+    }
   }
-  if (sps_status s = check_row_fits(a.n_t, sizeof(Moments) * (kMaxThreads / 32) * kWidthsPerPass + 512)) return s;
+  auto extra = [&](int per_pass) { return sizeof(Moments) * (kMaxThreads / 32) * per_pass + 512; };
+  if (sps_status s = check_row_fits(a.n_t, extra(kWidthsPerPass))) return s;
+  // decimating passes take up to 12 factors where their partials fit beside the row
+  // (a pass costs 11 us at 512 rows of 12500 samples whatever its factors)
+  const int most = a.decimate && row_fits(a.n_t + room, extra(kFactorsPerPass)) ? kFactorsPerPass : kWidthsPerPass;
   // largest boxcar value: 255 * channels * widest width (< 2^31, checked by the plan);
   // a thread's 64-bit S2 partial takes `flush` squares before it must be flushed
   const unsigned long long bmax = std::max<unsigned long long>(1ull, (unsigned long long)a.max_boxcar);
   const unsigned long long f2 = 0xFFFFFFFFFFFFFFFFull / (bmax * bmax);
   const int flush = (int)std::max<unsigned long long>(1ull, std::min<unsigned long long>(f2, 1ull << 30));
   // a warp's S2: 32 threads x ceil(n_t / threads) samples x bmax^2, in 64 bits?
-  const unsigned long long per_thread = (unsigned long long)((a.n_t + c.threads - 1) / c.threads);
+  const unsigned long long per_thread = (unsigned long long)((a.n_t + threads - 1) / threads);
   const long double warp_s2 = 32.0L * (long double)per_thread * (long double)bmax * (long double)bmax;
   const int narrow = warp_s2 < 1.8e19L ? 1 : 0;
   // no thread ever flushes: its sample count stays within `flush`
   const bool fast = narrow && per_thread <= (unsigned long long)flush;
-  const size_t smem = prefix_smem(a.n_t);
-  for (int w0 = 0; w0 < a.n_widths; w0 += kWidthsPerPass) {
-    const int nwp = std::min(kWidthsPerPass, a.n_widths - w0);
+  const int use_tma = aligned || row_fits(a.n_t + room, extra(most)) ? 1 : 0;
+  const size_t smem = prefix_smem(a.n_t + (use_tma ? room : 0));
+  for (int w0 = 0; w0 < a.n_widths; w0 += most) {
+    const int nwp = std::min(most, a.n_widths - w0);
     SnrKernel fn = a.decimate ? (fast ? snr_variant<true, true>(nwp) : snr_variant<true, false>(nwp))
                               : (fast ? snr_variant<false, true>(nwp) : snr_variant<false, false>(nwp));
     SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, smem, a, w0, flush, tma_ok(a.D, a.n_t) ? 1 : 0, narrow));
+    SPS_CUDA(launch(st, fn, dim3(a.n_dms), threads, smem, a, w0, flush, use_tma, narrow));
   }
   return launch_detect(a, st);
 }
@@ -1126,10 +1202,12 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
                             int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, Stream& st) {
   if (sps_status s = check_row_fits(n_t, 256)) return s;
-  const size_t smem = prefix_smem(n_t);
+  const int room = tma_ok(D, n_t) ? 0 : 3;
+  const int use_tma = row_fits(n_t + room, 256) ? 1 : 0;
+  const size_t smem = prefix_smem(n_t + (use_tma ? room : 0));
   SPS_CUDA(cudaFuncSetAttribute(integrate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, integrate_kernel, dim3(n_dms), 256, smem, D, n_dms, n_t, widths, n_widths, B,
-                  tma_ok(D, n_t) ? 1 : 0, decimate, status));
+                  use_tma, decimate, status));
   return SPS_OK;
 }
 
