@@ -80,29 +80,43 @@ class _Lazy:
 _L = _Lazy()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
+_T = None
+
+
+def _torch():
+    global _T
+    if _T is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        _T = torch
+    return _T
+
+
+def _stream(stream) -> int:
+    """The cudaStream_t of a torch stream or a raw handle; None: the current stream."""
+    if stream is None:
+        t = _torch()
+        if not t.cuda.is_initialized():
+            return t.cuda.current_stream().cuda_stream
+        # the raw handle, without building a Stream object per call (3.1 us)
+        return t._C._cuda_getCurrentRawStream(t._C._cuda_getDevice())
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
-def _dev(t, dtype, name, shape=None):
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+def _dev(x, dtype, name, shape=None) -> int:
+    if not isinstance(x, _torch().Tensor) or not x.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
-        raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
+    if x.dtype != dtype:
+        raise TypeError(f"{name} must be {dtype}, got {x.dtype}")
+    if not x.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    if shape is not None and x.shape != shape:
+        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(x.shape)}")
+    return x.data_ptr()
 
 
-def _xdev(plan, x, name="x"):
+def _xdev(plan, x, name="x") -> int:
     """A filterbank on the device: uint8 [channels][pitch], one row per channel
     (the library reads `channels` rows of the given pitch)."""
     t = _torch()
@@ -166,7 +180,7 @@ def sps_dedisperse(plan, x, D, workspace=None, stream=None):
     p = plan.handle
     if workspace is None:
         workspace = plan.workspace()
-    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else ctypes.c_void_p()
+    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else None
     wsb = workspace.numel() * workspace.element_size() if workspace is not None else 0
     check(_L.sps_dedisperse(p, _xdev(plan, x), ctypes.c_int64(x.shape[1]),
                             _dev(D, _torch().int32, "D", (plan.n_dms, plan.n_samples)), ws,
@@ -210,7 +224,7 @@ def sps_snr(plan, D, snr, peak_t, peak_val, best=None, stream=None):
     check(_L.sps_snr(plan.handle, _dev(D, t.int32, "D", (plan.n_dms, plan.n_samples)),
                      _dev(snr, t.float64, "snr", shp), _dev(peak_t, t.int32, "peak_t", shp),
                      _dev(peak_val, t.int32, "peak_val", shp),
-                     _dev(best, t.int32, "best", (4,)) if best is not None else ctypes.c_void_p(),
+                     _dev(best, t.int32, "best", (4,)) if best is not None else None,
                      _stream(stream)), "sps_snr")
 
 
@@ -219,13 +233,13 @@ def sps_search(plan, x, D, snr, peak_t, peak_val, best=None, workspace=None, str
     if workspace is None:
         workspace = plan.workspace()
     shp = (plan.n_widths, plan.n_dms)
-    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else ctypes.c_void_p()
+    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else None
     wsb = workspace.numel() * workspace.element_size() if workspace is not None else 0
     check(_L.sps_search(plan.handle, _xdev(plan, x), ctypes.c_int64(x.shape[1]),
                         _dev(D, t.int32, "D", (plan.n_dms, plan.n_samples)), ws, ctypes.c_size_t(wsb),
                         _dev(snr, t.float64, "snr", shp), _dev(peak_t, t.int32, "peak_t", shp),
                         _dev(peak_val, t.int32, "peak_val", shp),
-                        _dev(best, t.int32, "best", (4,)) if best is not None else ctypes.c_void_p(),
+                        _dev(best, t.int32, "best", (4,)) if best is not None else None,
                         _stream(stream)), "sps_search")
 
 
@@ -235,7 +249,7 @@ def sps_search_host(plan, x_host, x_dev, D, snr_dev, peak_t_dev, peak_val_dev, b
     if workspace is None:
         workspace = plan.workspace()
     shp = (plan.n_widths, plan.n_dms)
-    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else ctypes.c_void_p()
+    ws = _dev(workspace, workspace.dtype, "workspace") if workspace is not None else None
     wsb = workspace.numel() * workspace.element_size() if workspace is not None else 0
     if tuple(x_host.shape) != tuple(x_dev.shape):
         raise ValueError("x_host and x_dev must have the same shape")
@@ -247,11 +261,6 @@ def sps_search_host(plan, x_host, x_dev, D, snr_dev, peak_t_dev, peak_val_dev, b
         _dev(best_dev, t.int32, "best_dev", (4,)), _host(snr_host, t.float64, "snr_host", shp),
         _host(peak_t_host, t.int32, "peak_t_host", shp), _host(peak_val_host, t.int32, "peak_val_host", shp),
         _host(best_host, t.int32, "best_host", (4,)), _stream(stream)), "sps_search_host")
-
-
-def _torch():
-    import torch
-    return torch
 
 
 class Plan:
@@ -449,12 +458,12 @@ class Batch:
         bufs = (BeamBuffers * len(self.plans))()
         for b, (p, x, o) in enumerate(zip(self.plans, self.xs, self.outs)):
             shp = (p.n_widths, p.n_dms)
-            bufs[b] = BeamBuffers(_xdev(p, x).value, int(x.shape[1]),
-                                  _dev(o["D"], t.int32, "D", (p.n_dms, p.n_samples)).value,
-                                  _dev(o["snr"], t.float64, "snr", shp).value,
-                                  _dev(o["peak_t"], t.int32, "peak_t", shp).value,
-                                  _dev(o["peak_val"], t.int32, "peak_val", shp).value,
-                                  _dev(o["best"], t.int32, "best", (4,)).value)
+            bufs[b] = BeamBuffers(_xdev(p, x), int(x.shape[1]),
+                                  _dev(o["D"], t.int32, "D", (p.n_dms, p.n_samples)),
+                                  _dev(o["snr"], t.float64, "snr", shp),
+                                  _dev(o["peak_t"], t.int32, "peak_t", shp),
+                                  _dev(o["peak_val"], t.int32, "peak_val", shp),
+                                  _dev(o["best"], t.int32, "best", (4,)))
         self._bufs = bufs
         h = ctypes.c_void_p()
         check(_L.sps_batch_create(arr, bufs, len(self.plans), int(branches), self.workspace.data_ptr(),

@@ -232,6 +232,7 @@ sps_status run_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* pe
   for (size_t k = 0; k < p->widths.size() && pow2; k++) pow2 = p->widths[k] == (1 << k);
   if (pow2) a.pow2_widths = (int32_t)p->widths.size();
   a.best = best;
+  a.max_smem = p->max_smem;
   return launch_snr(a, p->cfg.snr, st);
 }
 
@@ -404,7 +405,7 @@ sps_status sps_integrate(const sps_plan* p, const int32_t* D, int32_t* B, void* 
   if (!D || !B) return fail(SPS_ERR_INVALID_ARG, "null pointer");
   Stream st((cudaStream_t)stream);
   return launch_integrate(D, (int32_t)p->dms.size(), p->n_t, p->d_widths, (int32_t)p->widths.size(),
-                          p->smoothing == SPS_SMOOTH_DECIMATE ? 1 : 0, B, p->d_status, st);
+                          p->smoothing == SPS_SMOOTH_DECIMATE ? 1 : 0, B, p->max_smem, p->d_status, st);
 }
 
 sps_status sps_snr(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,

@@ -678,7 +678,6 @@ sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len,
   const int64_t win = ((int64_t)kSeriesBlock + max_rel + 16 + 15) / 16 * 16;
   const int64_t smem = win * unit_channels;
   if (smem <= 96 * 1024) {
-    SPS_CUDA(cudaFuncSetAttribute(presum_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // Bands of few units have many series each: blocks take shares of a unit's
     // series (each stages the rows anew) until the grid has 16 blocks per SM.
     // 384 channels x 1024 trials (64 series per unit, 768 blocks): the call 203 ->
@@ -704,7 +703,6 @@ sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& 
   const size_t smem = presum_smem_bytes(a.stage_bytes);
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, a.n_groups * a.splits);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
-  SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm,
                   presum_window_bytes(c, a.dmax_tile)));
   return SPS_OK;
@@ -731,7 +729,6 @@ sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d
   const Variant* v = find_variant(c.dms_per_thread, c.samples_per_thread / 2);
   if (!v) return fail(SPS_ERR_INVALID_ARG, "no compiled pre-summed variant");
   const size_t smem = presum_smem_bytes(max_stage_bytes);
-  SPS_CUDA(cudaFuncSetAttribute(v->list, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, v->list, dim3((unsigned)n_work), 32 * c.warps_dm * c.warps_time, smem, d_passes, d_work,
                   c.warps_dm));
   return SPS_OK;

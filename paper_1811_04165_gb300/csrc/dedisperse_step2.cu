@@ -423,7 +423,6 @@ sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, Stream& 
     const size_t smem = step2_wide_smem_bytes(c, a.dmax_tile, a.n_subbands);
     dim3 grid((a.n_t + Tt - 1) / Tt, a.n_tiles, 1);
     if (grid.y > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many step-two tiles");
-    SPS_CUDA(cudaFuncSetAttribute(step2_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     SPS_CUDA(launch(st, step2_wide_kernel, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
                     copy_bytes(c, a.dmax_tile)));
     return SPS_OK;
@@ -435,7 +434,6 @@ sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& c, Stream& 
   const size_t smem = step2_smem_bytes(c, a.dmax_tile, a.n_subbands);
   dim3 grid((a.n_t + Tt - 1) / Tt, a.n_tiles, 1);
   if (grid.y > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many step-two tiles");
-  SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
                   copy_bytes(c, a.dmax_tile)));
   return SPS_OK;

@@ -424,7 +424,6 @@ sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& c, Strea
   U8Kernel fn = find(c.dms_per_thread, c.samples_per_thread / 4, gpb > 1);
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, (a.n_groups + gpb - 1) / gpb);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
-  SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,
                   u8_window_bytes(c, a.dmax_tile), gpb));
   return SPS_OK;

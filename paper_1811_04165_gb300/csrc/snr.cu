@@ -1005,21 +1005,11 @@ size_t prefix_smem(int n_t) { return ((size_t)n_t + kPad + 3) / 4 * 4 * sizeof(u
 
 bool tma_ok(const int32_t* D, int n_t) { return ((uintptr_t)D & 15) == 0 && (n_t & 3) == 0; }
 
-bool row_fits(int n_t, size_t extra) {
-  int dev = 0, max_smem = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-    return false;
-  return prefix_smem(n_t) + extra <= (size_t)max_smem;
-}
+bool row_fits(int max_smem, int n_t, size_t extra) { return prefix_smem(n_t) + extra <= (size_t)max_smem; }
 
-sps_status check_row_fits(int n_t, size_t extra) {
-  int dev = 0, max_smem = 0;
-  SPS_CUDA(cudaGetDevice(&dev));
-  SPS_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (prefix_smem(n_t) + extra > (size_t)max_smem)
-    return fail(SPS_ERR_UNSUPPORTED, "rows too long for the shared-memory prefix");
-  return SPS_OK;
+sps_status check_row_fits(int max_smem, int n_t, size_t extra) {
+  return row_fits(max_smem, n_t, extra) ? SPS_OK
+                                        : fail(SPS_ERR_UNSUPPORTED, "rows too long for the shared-memory prefix");
 }
 
 }  // namespace
@@ -1154,28 +1144,26 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
   const unsigned threads = (unsigned)snr_threads(a, c.threads);
   if (pow2_form(a)) {
     const size_t smem = pow2_smem(a.n_t + room, a.pow2_widths);
-    const bool fits = row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192);
+    const bool fits = row_fits(a.max_smem, a.n_t, smem - prefix_smem(a.n_t) + 8192);
     if (aligned && !fits && stream_form(a)) {
       // rows too long to stage whole: the streaming form, any row length
       const size_t stream = stream_smem(a.pow2_widths, c.threads);
       StreamKernel fn = stream_variant(a.pow2_widths);
-      SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stream));
       SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, stream, a));
       return launch_detect(a, st);
     }
-    if (aligned && !fits) return check_row_fits(a.n_t, smem - prefix_smem(a.n_t) + 8192);
+    if (aligned && !fits) return check_row_fits(a.max_smem, a.n_t, smem - prefix_smem(a.n_t) + 8192);
     if (fits) {
       Pow2Kernel fn = pow2_variant(a.pow2_widths);
-      SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       SPS_CUDA(launch(st, fn, dim3(a.n_dms), threads, smem, a));
       return launch_detect(a, st);
     }
   }
   auto extra = [&](int per_pass) { return sizeof(Moments) * (kMaxThreads / 32) * per_pass + 512; };
-  if (sps_status s = check_row_fits(a.n_t, extra(kWidthsPerPass))) return s;
+  if (sps_status s = check_row_fits(a.max_smem, a.n_t, extra(kWidthsPerPass))) return s;
   // decimating passes take up to 12 factors where their partials fit beside the row
   // (a pass costs 11 us at 512 rows of 12500 samples whatever its factors)
-  const int most = a.decimate && row_fits(a.n_t + room, extra(kFactorsPerPass)) ? kFactorsPerPass : kWidthsPerPass;
+  const int most = a.decimate && row_fits(a.max_smem, a.n_t + room, extra(kFactorsPerPass)) ? kFactorsPerPass : kWidthsPerPass;
   // largest boxcar value: 255 * channels * widest width (< 2^31, checked by the plan);
   // a thread's 64-bit S2 partial takes `flush` squares before it must be flushed
   const unsigned long long bmax = std::max<unsigned long long>(1ull, (unsigned long long)a.max_boxcar);
@@ -1187,25 +1175,24 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
   const int narrow = warp_s2 < 1.8e19L ? 1 : 0;
   // no thread ever flushes: its sample count stays within `flush`
   const bool fast = narrow && per_thread <= (unsigned long long)flush;
-  const int use_tma = aligned || row_fits(a.n_t + room, extra(most)) ? 1 : 0;
+  const int use_tma = aligned || row_fits(a.max_smem, a.n_t + room, extra(most)) ? 1 : 0;
   const size_t smem = prefix_smem(a.n_t + (use_tma ? room : 0));
   for (int w0 = 0; w0 < a.n_widths; w0 += most) {
     const int nwp = std::min(most, a.n_widths - w0);
     SnrKernel fn = a.decimate ? (fast ? snr_variant<true, true>(nwp) : snr_variant<true, false>(nwp))
                               : (fast ? snr_variant<false, true>(nwp) : snr_variant<false, false>(nwp));
-    SPS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     SPS_CUDA(launch(st, fn, dim3(a.n_dms), threads, smem, a, w0, flush, use_tma, narrow));
   }
   return launch_detect(a, st);
 }
 
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
-                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, Stream& st) {
-  if (sps_status s = check_row_fits(n_t, 256)) return s;
+                            int32_t n_widths, int32_t decimate, int32_t* B, int max_smem, uint32_t* status,
+                            Stream& st) {
+  if (sps_status s = check_row_fits(max_smem, n_t, 256)) return s;
   const int room = tma_ok(D, n_t) ? 0 : 3;
-  const int use_tma = row_fits(n_t + room, 256) ? 1 : 0;
+  const int use_tma = row_fits(max_smem, n_t + room, 256) ? 1 : 0;
   const size_t smem = prefix_smem(n_t + (use_tma ? room : 0));
-  SPS_CUDA(cudaFuncSetAttribute(integrate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   SPS_CUDA(launch(st, integrate_kernel, dim3(n_dms), 256, smem, D, n_dms, n_t, widths, n_widths, B,
                   use_tma, decimate, status));
   return SPS_OK;

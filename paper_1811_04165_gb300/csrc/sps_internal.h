@@ -69,6 +69,10 @@ cudaError_t launch(Stream& s, void (*kernel)(P...), dim3 grid, unsigned threads,
   c.attrs = &after;
   c.numAttrs = s.overlap && !s.first ? 1 : 0;
   s.first = false;
+  // beyond the default 48 KB (static shared memory included) a kernel has to be
+  // allowed its size; most small plans stay below and save the call
+  if (smem > 40 * 1024)
+    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
@@ -186,6 +190,7 @@ struct SnrArgs {
   int32_t decimate;        // 1: widths are downsampling factors
   int32_t pow2_widths;     // NW when the widths are exactly 1, 2, ..., 2^(NW-1); else 0
   int32_t* best;           // device int32[4] for the detection, or null
+  int max_smem;            // opt-in shared memory per block of the device
 };
 
 // Kernel launchers (dedisperse_u8.cu, dedisperse_presum.cu, dedisperse_step2.cu,
@@ -196,7 +201,8 @@ sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& cfg, Str
 sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& cfg, Stream& st);
 sps_status launch_snr(const SnrArgs& a, const sps_snr_config& cfg, Stream& st);
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
-                            int32_t n_widths, int32_t decimate, int32_t* B, uint32_t* status, Stream& st);
+                            int32_t n_widths, int32_t decimate, int32_t* B, int max_smem, uint32_t* status,
+                            Stream& st);
 sps_status launch_expand(const uint8_t* x, int64_t pitch, int32_t in_len, int32_t channels, uint8_t* x4,
                          int64_t pitch4, Stream& st);
 sps_status launch_presum_series(const uint8_t* x, int64_t pitch, int32_t in_len, const PresumUnit* units,
