@@ -150,9 +150,11 @@ sps_status run_u8_pass(const sps_plan* p, const sps_dedisp_config& cfg, const ui
     if (s) return s;
     return launch_presum_pass(a, cfg, st);
   }
-  sps_status s = launch_expand(x, pitch, (int32_t)p->n_in, p->channels, ws, p->pitch4, st);
-  if (s) return s;
-  U8PassArgs a = u8_args(p, x, pitch, ws);
+  if (!p->build_copies) {
+    sps_status s = launch_expand(x, pitch, (int32_t)p->n_in, p->channels, ws, p->pitch4, st);
+    if (s) return s;
+  }
+  U8PassArgs a = u8_args(p, x, pitch, p->build_copies ? nullptr : ws);
   a.di_pad = u8_di_pad(cfg);
   a.n_dm = rows;
   a.group_channels = per;

@@ -13,12 +13,14 @@
 //     samples and walks its channels `chunk` at a time.  For each channel the
 //     window [t0 + d(i0, c), t0 + Tt + d(i_last, c)) is staged once and read by
 //     all Di trials.
-//   * Four copies of each window are staged, copy j shifted by j bytes, so that
+//   * Four copies of each window are kept, copy j shifted by j bytes, so that
 //     every 4-sample read is one aligned, conflict-free 32-bit shared load
-//     whatever the delay's alignment.  A pre-pass (expand_kernel) writes the
-//     shifted copies 1..3 of the whole batch once; all four copies and the
-//     chunk's shared-memory offset table arrive by bulk asynchronous copies
-//     (TMA) into a two-stage ring guarded by mbarriers, so the warps only add.
+//     whatever the delay's alignment.  Copy 0 and the chunk's offset table arrive
+//     by bulk asynchronous copies (TMA) into a two-stage ring guarded by mbarriers.
+//     Copies 1..3 either arrive the same way, from shifted copies of the whole
+//     batch that a pre-pass (expand_kernel) writes, or are made from copy 0 in
+//     shared memory by the warps (BUILD: 16 % more shared accesses for a 32 x 512
+//     tile, no pre-pass); build_copies() in plan.cpp chooses.
 //   * SWAR: the words of 4 samples are summed whole (one three-input add per
 //     two channels), and their odd bytes, moved into 16-bit lanes by one byte
 //     permute, are summed apart with integer multiply-adds by 1 on the FMA
@@ -63,9 +65,10 @@ __device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
   }
 }
 
+// BUILD: copies 1..3 are made here, not staged.
 // WALK: the block walks gpb > 1 groups in turn (subband step one); without it
 // the block has one group, compiled as a plain loop over its chunks.
-template <int ND, int NW, bool WALK>
+template <int ND, int NW, bool WALK, bool BUILD>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -76,7 +79,6 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
   const int stage_bytes = 4 * copy_stride + cc_max * a.di_pad * 4;
   int32_t* b0s = reinterpret_cast<int32_t*>(smem + 2 * stage_bytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * stage_bytes + ((gpb * a.group_channels * 4 + 15) & ~15));
-  __shared__ int aborted;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int dm_sub = warp % wd, t_sub = warp / wd;
@@ -101,7 +103,6 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
 
   for (int c = tid; c < ng * G; c += blockDim.x) b0s[c] = a.b0[(int64_t)tile * a.channels + c_lo + c];
   if (tid == 0) {
-    aborted = 0;
     mbar_init(&bars[0], blockDim.x >> 5);
     mbar_init(&bars[1], blockDim.x >> 5);
     fence_mbar_init();
@@ -109,11 +110,12 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
   __syncthreads();
 
   // Every warp stages its share of chunk `ch` (channels warp, warp + nwarps,
-  // ...) into stage ch & 1: the four shifted copies of each channel window;
-  // warp 0 also copies the chunk's offset table.  Each warp's lane 0 arrives
-  // on the stage barrier with the bytes its warp issued.  Chunk ch is chunk
-  // ch % chunks_g of the block's group ch / chunks_g; cb is its first channel
-  // inside the block's channel range.
+  // ...) into stage ch & 1, one copy of a window per lane: with BUILD lane q takes
+  // copy 0 of channel warp + q nwarps, else lanes 4q .. 4q+3 the four copies of it;
+  // warp 0 also copies the chunk's offset table.  Each warp's lane 0 arrives on the
+  // stage barrier with the bytes its warp issued.  Chunk ch is chunk ch % chunks_g
+  // of the block's group ch / chunks_g; cb is its first channel inside the block's
+  // channel range.
   const int nwarps = (int)(blockDim.x >> 5);
   auto issue = [&](int ch) {
     const int st = ch & 1;
@@ -122,25 +124,23 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
     const int cb = gi * G + cg * cc_max, cc = min(cc_max, G - cg * cc_max);
     const int npair = (cc + 1) >> 1;
     const uint32_t tbl_bytes = (uint32_t)(npair * a.di_pad * 8);
-    // lanes 4q..4q+3 of a warp handle copies 0..3 of channels warp + (q + 8k) * nwarps
-    const int q = lane >> 2, j = lane & 3;
+    const int q = BUILD ? lane : lane >> 2, j = BUILD ? 0 : lane & 3;
+    constexpr int kPer = BUILD ? 32 : 8;  // channels per warp and round
     uint32_t mine = 0;
-    for (int l = warp + q * nwarps; l < cc; l += 8 * nwarps)
+    for (int l = warp + q * nwarps; l < cc; l += kPer * nwarps)
       mine += (uint32_t)min(wb, a.win_limit - (t0 + b0s[cb + l]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane == 0) {
       fence_proxy_async();
       mbar_arrive_expect_tx(&bars[st], mine + (warp == 0 ? tbl_bytes : 0u));
     }
     __syncwarp();
-    for (int l = warp + q * nwarps; l < cc; l += 8 * nwarps) {
+    for (int l = warp + q * nwarps; l < cc; l += kPer * nwarps) {
       const int c = c_lo + cb + l;
       const int start = t0 + b0s[cb + l];
-      const uint32_t bytes = (uint32_t)min(wb, a.win_limit - start);
-      const uint8_t* src = j == 0 ? a.x + (int64_t)c * a.pitch + start
-                                  : a.x4 + ((int64_t)(j - 1) * a.channels + c) * a.pitch4 + start;
-      bulk_g2s(sb + j * copy_stride + l * wb, src, bytes, &bars[st]);
+      const uint8_t* src = BUILD || j == 0 ? a.x + (int64_t)c * a.pitch + start
+                                           : a.x4 + ((int64_t)(j - 1) * a.channels + c) * a.pitch4 + start;
+      bulk_g2s(sb + j * copy_stride + l * wb, src, (uint32_t)min(wb, a.win_limit - start), &bars[st]);
     }
     if (warp == 0 && lane == 0) {
       const uint32_t* src =
@@ -225,19 +225,43 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
         for (int q = 0; q < 4; q++) acc[r][m][q] = 0;
   };
 
-  pdl_wait();  // the shifted copies are written
+  pdl_wait();  // the shifted copies, or a masked copy of the input, are written
   issue(0);
   if (n_chunks > 1) issue(1);
 
   int pending = 0;
   int ch = 0;
   int gi = 0, cg = 0;  // group and chunk inside it of chunk ch (WALK)
+  const int wwords = wb >> 2;
   for (; ch < n_chunks; ch++) {
     const int st = ch & 1;
     const int cc = min(cc_max, G - (WALK ? cg : ch) * cc_max);
     if (pending + cc > 256) { fold(); pending = 0; }
-    if (!mbar_wait(&bars[st], (ch >> 1) & 1, a.status)) aborted = 1;
-    if (!aborted) {
+    const bool ok = mbar_wait(&bars[st], (ch >> 1) & 1, a.status);
+    // copies 1 .. 3 = copy 0 one to three bytes later; a warp per channel window
+    if (BUILD && ok) {
+      const uint32_t* c0 = reinterpret_cast<const uint32_t*>(smem + st * stage_bytes);
+      uint32_t* c1 = reinterpret_cast<uint32_t*>(smem + st * stage_bytes + copy_stride);
+      const int cw = copy_stride >> 2;
+      for (int l = warp; l < cc; l += nwarps)
+        for (int j = lane; j < wwords; j += 32) {
+          const int e = l * wwords + j;
+          const uint32_t lo = c0[e], hi4 = j + 1 < wwords ? c0[e + 1] : 0u;
+          c1[e] = __byte_perm(lo, hi4, 0x4321);
+          c1[cw + e] = __byte_perm(lo, hi4, 0x5432);
+          c1[2 * cw + e] = __byte_perm(lo, hi4, 0x6543);
+        }
+    }
+    // the copies are ready, and the other stage's chunk is no longer read
+    if (__syncthreads_or(ok ? 0 : 1)) {
+      // the copies issued and not yet waited for may still be in flight: one
+      // more bounded wait for each before the block leaves
+      if (tid == 0)
+        for (int k = ch; k < min(ch == 0 ? 2 : ch + 1, n_chunks); k++) mbar_wait(&bars[k & 1], (k >> 1) & 1, nullptr);
+      return;
+    }
+    if (ch > 0 && ch + 1 < n_chunks) issue(ch + 1);
+    {
       const uint32_t base = smem_u32(smem) + (uint32_t)(st * stage_bytes) + toff;
       const uint2* tb = reinterpret_cast<const uint2*>(smem + st * stage_bytes + 4 * copy_stride) + dm_sub * ND;
       int cl = 0;
@@ -271,9 +295,6 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
       }
     }
     pending += cc;
-    __syncthreads();
-    if (aborted) break;
-    if (ch + 2 < n_chunks) issue(ch + 2);
     if constexpr (WALK) {
       if (++cg == chunks_g) {
         // the group's last chunk: its sums go out while the next chunks land
@@ -283,12 +304,6 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
         gi++;
       }
     }
-  }
-  if (aborted) {
-    // let copies already in flight land before the block's shared memory goes away
-    if (tid == 0)
-      for (int k = ch; k < min(ch + 2, n_chunks); k++) mbar_wait(&bars[k & 1], (k >> 1) & 1, a.status);
-    return;
   }
   pdl_next();
   if constexpr (!WALK) finish_group(g0);
@@ -340,23 +355,20 @@ __global__ void __launch_bounds__(256) expand_kernel(const uint8_t* x, int64_t p
 
 typedef void (*U8Kernel)(U8PassArgs, int, int, int, int);
 
-template <int ND, int NW>
-constexpr U8Kernel k() { return u8_pass_kernel<ND, NW, false>; }
-template <int ND, int NW>
-constexpr U8Kernel kw() { return u8_pass_kernel<ND, NW, true>; }
-
-struct Variant { int nd, nw; U8Kernel fn, walk; };
+struct Variant { int nd, nw; U8Kernel fn[2][2]; };  // [walk][build]
+#define SPS_U8_VARIANT(ND, NW)                                                      \
+  {ND, NW, {{u8_pass_kernel<ND, NW, false, false>, u8_pass_kernel<ND, NW, false, true>}, \
+            {u8_pass_kernel<ND, NW, true, false>, u8_pass_kernel<ND, NW, true, true>}}}
 const Variant kVariants[] = {
-    {1, 1, k<1, 1>(), kw<1, 1>()}, {1, 2, k<1, 2>(), kw<1, 2>()}, {1, 4, k<1, 4>(), kw<1, 4>()},
-    {1, 8, k<1, 8>(), kw<1, 8>()}, {2, 1, k<2, 1>(), kw<2, 1>()}, {2, 2, k<2, 2>(), kw<2, 2>()},
-    {2, 4, k<2, 4>(), kw<2, 4>()}, {2, 8, k<2, 8>(), kw<2, 8>()}, {4, 1, k<4, 1>(), kw<4, 1>()},
-    {4, 2, k<4, 2>(), kw<4, 2>()}, {4, 4, k<4, 4>(), kw<4, 4>()}, {8, 1, k<8, 1>(), kw<8, 1>()},
-    {8, 2, k<8, 2>(), kw<8, 2>()},
+    SPS_U8_VARIANT(1, 1), SPS_U8_VARIANT(1, 2), SPS_U8_VARIANT(1, 4), SPS_U8_VARIANT(1, 8), SPS_U8_VARIANT(2, 1),
+    SPS_U8_VARIANT(2, 2), SPS_U8_VARIANT(2, 4), SPS_U8_VARIANT(2, 8), SPS_U8_VARIANT(4, 1), SPS_U8_VARIANT(4, 2),
+    SPS_U8_VARIANT(4, 4), SPS_U8_VARIANT(8, 1), SPS_U8_VARIANT(8, 2),
 };
+#undef SPS_U8_VARIANT
 
-U8Kernel find(int nd, int nw, bool walk = false) {
+U8Kernel find(int nd, int nw, bool walk = false, bool build = false) {
   for (const Variant& v : kVariants)
-    if (v.nd == nd && v.nw == nw) return walk ? v.walk : v.fn;
+    if (v.nd == nd && v.nw == nw) return v.fn[walk][build];
   return nullptr;
 }
 
@@ -421,7 +433,7 @@ sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& c, Strea
   const size_t smem = u8_smem_bytes(c, a.dmax_tile, a.group_channels, a.n_groups);
   const int64_t tiles = (int64_t)((a.n_dm + Di - 1) / Di) * ((a.n_out + Tt - 1) / Tt);
   const int gpb = u8_groups_per_block(a.n_groups, tiles);
-  U8Kernel fn = find(c.dms_per_thread, c.samples_per_thread / 4, gpb > 1);
+  U8Kernel fn = find(c.dms_per_thread, c.samples_per_thread / 4, gpb > 1, a.x4 == nullptr);
   dim3 grid((a.n_dm + Di - 1) / Di, (a.n_out + Tt - 1) / Tt, (a.n_groups + gpb - 1) / gpb);
   if (grid.y > 65535 || grid.z > 65535) return fail(SPS_ERR_UNSUPPORTED, "too many time tiles or groups");
   SPS_CUDA(launch(st, fn, grid, 32 * c.warps_dm * c.warps_time, smem, a, c.warps_dm, c.chunk,

@@ -297,10 +297,11 @@ bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* 
 // default tile, 578 with twice the trials and channels per stage; 64 channels x
 // 4096 samples x 32 trials 14.2 us with 8 blocks, 5.8 with 128 small ones; step one
 // of 768 channels, 8 subbands, 4 coarse DMs 19.2 -> 7.8 us).
-sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c) {
+sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c, double* pass) {
   struct Tile { sps_dedisp_config c; double cycles; };
   const Tile tiles[] = {{{4, 16, 8, 1, 16, 0}, 1.45}, {{4, 16, 16, 1, 32, 0}, 1.34}, {{2, 16, 8, 1, 32, 0}, 1.45},
                         {{2, 8, 8, 1, 32, 0}, 1.5},   {{1, 8, 8, 1, 48, 0}, 1.7},    {{1, 4, 8, 1, 64, 0}, 2.0}};
+  *pass = 1e30;
   if (!same_tile(c, tiles[0].c)) return c;
   const bool brute = p->mode == SPS_MODE_BRUTE;
   const int64_t rows = brute ? (int64_t)p->dms.size() : (int64_t)p->coarse_dms.size();
@@ -328,7 +329,17 @@ sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c) {
       best = t.c;
     }
   }
+  *pass = least;
   return best;
+}
+
+// Whether the single-channel pass of `pass_us` makes the shifted copies of its
+// windows itself.  That costs it about a tenth more shared accesses, per DM tile;
+// writing and reading them in device memory costs a launch and four times the
+// input: step one of the beam 112 -> 107 us (two tiles of coarse DMs), 64 channels
+// x 4096 samples x 32 trials 5.5 -> 4.4, but 1536 x 12500 x 768 trials 577 -> 595.
+bool build_copies(const sps_plan* p, double pass_us) {
+  return 0.1 * pass_us < 2.5 + 4.0 * p->channels * (double)p->n_in / 6e6;
 }
 
 // The tile and the channel splits the brute-force pass runs with, by a model of
@@ -346,12 +357,13 @@ sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c) {
 // output (its additions reach the L2 at 4.3 TB/s).  64 trials x 12500 samples:
 // 140 us with the default tile, 160 wide, 59 wide in eight splits; 512 trials
 // (0.4 pc cm^-3 apart): 415, 266 and, in four splits, 237.
-void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_config* tile, int32_t* splits) {
+void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_config* tile, int32_t* splits,
+                 double* u8_us) {
   *tile = c;
   *splits = 1;
   if (p->mode != SPS_MODE_BRUTE) return;
   if (!c.presum) {
-    *tile = choose_u8(p, c);
+    *tile = choose_u8(p, c, u8_us);
     return;
   }
   const int64_t rows = (int64_t)p->dms.size(), units = (p->channels + (1 << c.presum) - 1) >> c.presum;
@@ -401,8 +413,9 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   const int32_t n_dms = (int32_t)p->dms.size();
   sps_dedisp_config tile;
   int32_t splits = 1;
-  choose_tile(p, cfg.brute, &tile, &splits);
-  const sps_dedisp_config tile1 = p->mode == SPS_MODE_BRUTE || cfg.step1.presum ? cfg.step1 : choose_u8(p, cfg.step1);
+  double u8_us = 1e30;  // modelled time of the single-channel pass
+  choose_tile(p, cfg.brute, &tile, &splits, &u8_us);
+  const sps_dedisp_config tile1 = p->mode == SPS_MODE_BRUTE || cfg.step1.presum ? cfg.step1 : choose_u8(p, cfg.step1, &u8_us);
   const sps_dedisp_config& pass = p->mode == SPS_MODE_BRUTE ? tile : tile1;
   const int32_t dmax_b = p->mode == SPS_MODE_BRUTE ? cached_spread(p, 0, tile.warps_dm * tile.dms_per_thread) : 0;
   const int32_t dmax_1 =
@@ -485,6 +498,7 @@ sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg) {
   p->cfg = cfg;
   p->brute_tile = tile;
   p->brute_splits = splits;
+  p->build_copies = build_copies(p, u8_us);
   p->step1_tile = tile1;
   p->step2_tile = tile2;
   p->config_gen++;

@@ -81,7 +81,7 @@ cudaError_t launch(Stream& s, void (*kernel)(P...), dim3 grid, unsigned threads,
 struct U8PassArgs {
   const uint8_t* x;        // [channels][pitch]: copy 0 of every window
   int64_t pitch;           // bytes per channel row
-  const uint8_t* x4;       // [3][channels][pitch4]: rows shifted by 1, 2, 3 bytes
+  const uint8_t* x4;       // [3][channels][pitch4]: rows shifted by 1, 2, 3 bytes, or null: made in the pass
   int64_t pitch4;          // bytes per shifted row (N_in rounded up to 16)
   int32_t win_limit;       // no staged window reads at or beyond this byte of a row
   const int32_t* b0;       // [n_tiles][channels]: first-trial delay rounded down to 16
@@ -340,6 +340,7 @@ struct sps_plan {
   // picks for the default pre-summed tile (presum_tile in plan.cpp)
   sps_dedisp_config brute_tile{};
   sps_dedisp_config step1_tile{}, step2_tile{};  // likewise of the two steps
+  bool build_copies = false;       // the single-channel pass makes its shifted copies itself
   int32_t brute_splits = 1;      // shares of the channels that blocks of their own sum
   uint64_t config_gen = 0;       // bumped whenever the device tables are rebuilt
   // delay spread of one DM tile for the current configuration

@@ -66,3 +66,50 @@ def test_wide_step_two_equals_narrow(lib, S, per, coarse, fine, n_t, full):
     assert torch.equal(got, want)
     if full:
         assert int(got[0, 0]) == 255 * per * S
+
+
+# channels, samples, trials, DM step, zapped channel or None: quads do not fit, so
+# the default is the single-channel kernel
+SINGLE = [(100, 5001, 200, 0.5, None), (61, 4097, 70, 1.0, 17), (64, 4096, 32, 2.0, 0)]
+
+
+@pytest.mark.parametrize("C,n_t,n_dms,step,zap", SINGLE)
+def test_copies_made_in_the_pass_brute(lib, C, n_t, n_dms, step, zap):
+    """Small plans make the shifted copies of their windows in the pass; an
+    explicit tile reads them from device memory."""
+    import torch
+    z = None if zap is None else [int(c == zap) for c in range(C)]
+    plan = lib.Plan(C, 1250.0, 1550.0, 81.92e-6, n_t, step * np.arange(n_dms), [1], zap=z)
+    assert plan.config.brute.presum == 0
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    x = torch.randint(0, 256, (C, plan.pitch), dtype=torch.uint8, device="cuda", generator=gen)
+    got = torch.full((n_dms, n_t), -1, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, got)
+    cfg = plan.config
+    cfg.brute = lib.DedispConfig(4, 8, 4, 1, 8, 0)
+    plan.config = cfg
+    want = torch.full((n_dms, n_t), -2, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, want)
+    assert plan.status() == 0
+    assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("S,per,coarse,fine,n_t", [(7, 21, 40, 4, 6001), (32, 48, 64, 2, 3000), (3, 257, 9, 2, 1111)])
+def test_copies_made_in_the_pass_step_one(lib, S, per, coarse, fine, n_t):
+    import torch
+    dms = 0.3 * np.arange(coarse * fine)
+    plan = lib.Plan(S * per, 1250.0, 1550.0, 81.92e-6, n_t, dms, [1], mode=lib.MODE_SUBBAND, n_subbands=S,
+                    coarse_dms=dms[::fine].copy())
+    gen = torch.Generator(device="cuda").manual_seed(S)
+    x = torch.randint(200, 256, (S * per, plan.pitch), dtype=torch.uint8, device="cuda", generator=gen)
+    ys = []
+    for tile in (None, (4, 8, 4, 1, 8, 0)):
+        if tile:
+            cfg = plan.config
+            cfg.step1 = lib.DedispConfig(*tile)
+            plan.config = cfg
+        Y = torch.zeros(plan.y_shape, dtype=torch.int16, device="cuda").view(torch.uint16)
+        lib.sps_subband_step1(plan, x, Y)
+        ys.append(Y.view(torch.int16)[:, :, :plan.step1_samples])
+    assert plan.status() == 0
+    assert torch.equal(ys[0], ys[1])
