@@ -117,12 +117,13 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
   // byte in the stage and its length; lane 0 also copies the chunk's offset
   // table and arrives on the stage's "full" barrier with the byte count (the
   // list's last entry, unless a window may be cut at the end of a row).  The
-  // issuing warp asks for its list a chunk early (`fetch`): the wide tile
-  // loads the head and its first entry per lane; the narrow ones, whose sums
-  // leave no registers to hold them over a chunk, bring the list into L1.
+  // issuing warp asks for its list a chunk early (`fetch`): it loads the head and
+  // its first entry per lane, or, where int32 sums leave no registers to hold
+  // them over a chunk (4 x 8 words: the pass 12 % slower), brings the list into L1.
   // A list entry is {row, start, (stage byte / 16) | (bytes / 16) << 16, 0};
   // the last is {count, total bytes, units, offset table / 8 entries}.
   struct Fetched { uint32_t nt; int row, start, at; };  // nt = count | total << 14
+  constexpr bool kHold = WIDE || ND * NW <= 16;
   auto load_list = [&](int ch) {
     const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
     Fetched f;
@@ -135,7 +136,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
     return f;
   };
   auto fetch = [&](int ch) {
-    if constexpr (WIDE) return load_list(ch);
+    if constexpr (kHold) return load_list(ch);
     const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
     // a 128-byte line holds eight entries
     const int at = min(8 * lane, copies_max);
@@ -146,7 +147,7 @@ __device__ __forceinline__ void presum_pass_block(const PresumPassArgs& a, int t
     const int st = ch % kStages;
     uint8_t* sb = smem + st * stage_bytes;
     const int4* list = a.copies + (int64_t)(chunks.x + ch) * (copies_max + 1);
-    const Fetched f = WIDE ? fetched : load_list(ch);
+    const Fetched f = kHold ? fetched : load_list(ch);
     const int4 head = __ldg(&list[copies_max]);
     const uint32_t tbl_bytes = (uint32_t)(head.z * a.di_pad * 2);
     const int n = (int)(f.nt & 0x3FFFu);
@@ -369,7 +370,9 @@ template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* __restrict__ work, int wd) {
   const int4 w = work[blockIdx.x];
-  const PresumPassArgs& a = passes[w.x];
+  // a copy: read through the pointer, every field is loaded anew after each of
+  // the pass's memory-ordering statements (eight mixed beams 2003 -> 1954 us)
+  const PresumPassArgs a = passes[w.x];
   presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, w.w, 0, wd, a.window_bytes);
 }
 
