@@ -99,7 +99,11 @@ typedef struct {
  * staged through shared memory `chunk` at a time.  `presum` (brute force and
  * step one) selects the kernel: 0 sums single channels; 1 and 2 sum series of
  * 2^presum adjacent channels pre-added once per batch (pairs, quads), each
- * series taken at the delay of its highest-frequency channel.  All are exact. */
+ * series taken at the delay of its highest-frequency channel.  All are exact.
+ * A new plan's tiles leave the tile, and a split of the channels over more
+ * blocks, to the library, which goes by the plan's size (so do the same values
+ * set explicitly); other values are run as given, pre-summed brute force split
+ * where its grid would leave SMs idle. */
 typedef struct {
   int32_t dms_per_thread;     /* register tile along DM                            */
   int32_t samples_per_thread; /* register tile along time (4*k for the uint8 path)  */
@@ -111,7 +115,9 @@ typedef struct {
 
 /* Launch parameters of the fused boxcar + S/N kernel. */
 typedef struct {
-  int32_t threads;            /* threads per block (one block per DM row)           */
+  int32_t threads;            /* threads per block (one block per DM row); 256, the
+                                 default, leaves the number to the library by the
+                                 rows' count and length                             */
 } sps_snr_config;
 
 typedef struct {
@@ -221,6 +227,7 @@ sps_status sps_integrate(const sps_plan* plan, const int32_t* D, int32_t* B, voi
  * snr: device double [n_widths][n_dms]; peak_t, peak_val: device int32, same
  * shape.  best (may be NULL): device int32[4] = {DM index, width index,
  * peak_t, peak_val} of the largest S/N (ties: smaller DM, then smaller width).
+ * Rows may start anywhere (D aligned to its type) and have any length.
  * Rows are staged whole in shared memory when they fit (about 56000 samples);
  * longer rows are streamed in chunks for widths 1, 2, 4, ..., 64 and refused
  * with UNSUPPORTED for other width sets and for decimating smoothing. */
