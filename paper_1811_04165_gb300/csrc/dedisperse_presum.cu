@@ -450,7 +450,7 @@ __device__ __forceinline__ void load_row24(const uint8_t* row, int u, int in_len
   if (u >= 0 && u + 24 <= in_len) {
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-      const uint2 t = __ldg(reinterpret_cast<const uint2*>(row + u + 8 * k));
+      const uint2 t = *reinterpret_cast<const uint2*>(row + u + 8 * k);
       W[2 * k] = t.x;
       W[2 * k + 1] = t.y;
     }
@@ -461,7 +461,7 @@ __device__ __forceinline__ void load_row24(const uint8_t* row, int u, int in_len
 #pragma unroll
       for (int i = 0; i < 4; i++) {
         const int p = u + 4 * k + i;
-        if (p >= 0 && p < in_len) w |= (uint32_t)__ldg(row + p) << (8 * i);
+        if (p >= 0 && p < in_len) w |= (uint32_t)row[p] << (8 * i);
       }
       W[k] = w;
     }

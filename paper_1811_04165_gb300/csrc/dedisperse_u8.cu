@@ -312,9 +312,9 @@ u8_pass_kernel(U8PassArgs a, int wd, int cc_max, int wb, int gpb) {
 // Bytes [p, p + 20) of a channel row, zero at and beyond `len`.
 __device__ __forceinline__ void load_raw20(const uint8_t* row, int64_t p, int32_t len, uint32_t r[5]) {
   if (p + 20 <= len) {
-    uint4 v = __ldg(reinterpret_cast<const uint4*>(row + p));
+    const uint4 v = *reinterpret_cast<const uint4*>(row + p);
     r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
-    r[4] = __ldg(reinterpret_cast<const uint32_t*>(row + p + 16));
+    r[4] = *reinterpret_cast<const uint32_t*>(row + p + 16);
   } else {
 #pragma unroll
     for (int k = 0; k < 5; k++) {
@@ -322,7 +322,7 @@ __device__ __forceinline__ void load_raw20(const uint8_t* row, int64_t p, int32_
 #pragma unroll
       for (int b = 0; b < 4; b++) {
         int64_t q = p + 4 * k + b;
-        uint32_t v = q < len ? (uint32_t)__ldg(row + q) : 0u;
+        uint32_t v = q < len ? (uint32_t)row[q] : 0u;
         w |= v << (8 * b);
       }
       r[k] = w;

@@ -112,10 +112,10 @@ __device__ bool stage_row(const int32_t* row, int n_t, uint32_t* buf, uint64_t* 
       if (body) bulk_g2s(buf + kPad + s + head, row + head, (uint32_t)body * 4u, bar);
     }
     if ((int)threadIdx.x < s) buf[kPad + threadIdx.x] = 0u;
-    if ((int)threadIdx.x < head) buf[kPad + s + threadIdx.x] = (uint32_t)__ldg(row + threadIdx.x);
+    if ((int)threadIdx.x < head) buf[kPad + s + threadIdx.x] = (uint32_t)row[threadIdx.x];
     if ((int)threadIdx.x < tail) {
       const int t = head + body + (int)threadIdx.x;
-      buf[kPad + s + t] = (uint32_t)__ldg(row + t);
+      buf[kPad + s + t] = (uint32_t)row[t];
     }
     __syncthreads();
     ok = mbar_wait(bar, 0, status);
@@ -126,7 +126,7 @@ __device__ bool stage_row(const int32_t* row, int n_t, uint32_t* buf, uint64_t* 
       return false;
     }
   } else {
-    for (int t = threadIdx.x; t < n_t; t += blockDim.x) buf[kPad + t] = (uint32_t)__ldg(row + t);
+    for (int t = threadIdx.x; t < n_t; t += blockDim.x) buf[kPad + t] = (uint32_t)row[t];
     __syncthreads();
   }
   return true;
@@ -720,13 +720,13 @@ constexpr int kRing = 2 * kChunk + 64;    // two chunk slots and the mirror of s
 
 // D[idx .. idx + 3] of the row, zeros past its end (n_t is a multiple of 4, so a
 // quadruple lies wholly inside or wholly outside the row).
-__device__ __forceinline__ uint4 load_quad(const int32_t* __restrict__ row, int idx, int n_t) {
-  return idx < n_t ? __ldg(reinterpret_cast<const uint4*>(row + idx)) : make_uint4(0u, 0u, 0u, 0u);
+__device__ __forceinline__ uint4 load_quad(const int32_t* row, int idx, int n_t) {
+  return idx < n_t ? *reinterpret_cast<const uint4*>(row + idx) : make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Asynchronous 16-byte copy of D[idx .. idx + 3] into shared memory, zeros
 // past the row's end (the source is then not read).
-__device__ __forceinline__ void copy_quad(uint32_t* dst, const int32_t* __restrict__ row, int idx, int n_t) {
+__device__ __forceinline__ void copy_quad(uint32_t* dst, const int32_t* row, int idx, int n_t) {
   const bool in = idx < n_t;
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(row + (in ? idx : 0)),
                "r"(in ? 16 : 0)
@@ -735,7 +735,7 @@ __device__ __forceinline__ void copy_quad(uint32_t* dst, const int32_t* __restri
 
 // Chunk j's quadruples of this lane into staging slot j % 3 (nothing past
 // chunk `last`); always one commit group, so that group counts stay uniform.
-__device__ __forceinline__ void stage_chunk(uint32_t* stage, const int32_t* __restrict__ row, int j, int last,
+__device__ __forceinline__ void stage_chunk(uint32_t* stage, const int32_t* row, int j, int last,
                                             int n_t) {
   const int lane = threadIdx.x & 31;
   if (j <= last) {
@@ -846,7 +846,7 @@ __device__ __forceinline__ void chunk_boxcars(const uint32_t* ptr, int base, int
 
 // First sample t of chunk c whose width-w boxcar equals m (the row's maximum),
 // found by one warp from D; the ring serves as its scratch.  Every lane returns it.
-__device__ int first_in_chunk(const int32_t* __restrict__ row, int n_t, uint32_t* ring, int c, int w, int m) {
+__device__ int first_in_chunk(const int32_t* row, int n_t, uint32_t* ring, int c, int w, int m) {
   const int lane = threadIdx.x & 31;
   const int base = kChunk * c;
   uint32_t run = 0u;
@@ -888,7 +888,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_stream_kernel(SnrArgs a) {
   __shared__ int wmx[kWarps][NW], gmax[NW], gchunk[NW], gfirst[NW];
   const int row = blockIdx.x, n_t = a.n_t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int32_t* __restrict__ Drow = a.D + (int64_t)row * n_t;
+  const int32_t* Drow = a.D + (int64_t)row * n_t;
   uint32_t* ring = dyn + warp * (kRing + 3 * kChunk + NW * 32);
   uint32_t* stage = ring + kRing;
   int* mc = reinterpret_cast<int*>(stage + 3 * kChunk) + lane;
@@ -970,8 +970,8 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_stream_kernel(SnrArgs a) {
 #pragma unroll
     for (int j = 0; j < 2; j++) {
       const int u = lane + 32 * j, v = n_t - 64 + lane + 32 * j;
-      lo[j] = u < n_t ? (uint32_t)__ldg(Drow + u) : 0u;
-      hi[j] = v >= 0 ? (uint32_t)__ldg(Drow + v) : 0u;
+      lo[j] = u < n_t ? (uint32_t)Drow[u] : 0u;
+      hi[j] = v >= 0 ? (uint32_t)Drow[v] : 0u;
     }
 #pragma unroll
     for (int k = 0; k < NW; k++) {

@@ -35,7 +35,10 @@ constexpr uint32_t kMaxPolls = 1u << 22;
 // Waits until the kernel before this one in the call has completed and its
 // writes are visible (returns at once in an ordinary launch).  Every kernel that
 // may be launched beside its predecessor calls it before it touches memory that
-// an earlier kernel writes or reads.
+// an earlier kernel writes or reads, and reads such memory by plain loads or
+// copies, which stay behind the wait: __ldg (and __restrict__, which lets the
+// compiler make one) may be moved above it and asks for memory that is constant
+// over the kernel's whole life, so it is for the plan's tables alone.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Lets the next kernel of the call be put on the GPU once every block has
