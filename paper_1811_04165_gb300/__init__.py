@@ -367,6 +367,14 @@ class Plan:
     def config(self, c: KernelConfig):
         check(_L.sps_plan_set_config(self.handle, ctypes.byref(c)), "sps_plan_set_config")
 
+    def tiles(self):
+        """The tiles the plan's kernels run with (sps_plan_get_tiles): a KernelConfig,
+        the channel splits, and whether the single-channel pass makes its copies."""
+        c, splits, made = KernelConfig(), ctypes.c_int32(), ctypes.c_int32()
+        check(_L.sps_plan_get_tiles(self.handle, ctypes.byref(c), ctypes.byref(splits), ctypes.byref(made)),
+              "sps_plan_get_tiles")
+        return c, int(splits.value), bool(made.value)
+
     def shape_key(self) -> dict:
         """What a tuned configuration depends on: the band, sampling, DM grid and
         widths, mode and subbands (the key of a saved configuration)."""

@@ -26,6 +26,7 @@ SIGNATURES = {
     "sps_plan_workspace_bytes": (_I32, [_P, _P]),
     "sps_plan_get_config": (_I32, [_P, _P]),
     "sps_plan_set_config": (_I32, [_P, _P]),
+    "sps_plan_get_tiles": (_I32, [_P, _P, _P, _P]),
     "sps_dedisperse": (_I32, [_P, _P, _I64, _P, _P, _SZ, _P]),
     "sps_dedisperse_noalloc": (_I32, [_P, _P, _I64, _P, _P]),
     "sps_subband_step1": (_I32, [_P, _P, _I64, _P, _P, _SZ, _P]),

@@ -366,6 +366,17 @@ sps_status sps_plan_set_config(sps_plan* p, const sps_kernel_config* cfg) {
   return apply_config(p, *cfg);
 }
 
+sps_status sps_plan_get_tiles(const sps_plan* p, sps_kernel_config* tiles, int32_t* channel_splits,
+                              int32_t* copies_in_pass) {
+  clear_error();
+  if (sps_status s = check_plan(p)) return s;
+  if (!tiles || !channel_splits || !copies_in_pass) return fail(SPS_ERR_INVALID_ARG, "null output");
+  *tiles = {p->brute_tile, p->step1_tile, p->step2_tile, p->cfg.snr};
+  *channel_splits = p->brute_splits;
+  *copies_in_pass = p->build_copies ? 1 : 0;
+  return SPS_OK;
+}
+
 sps_status sps_dedisperse(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
                           size_t ws_bytes, void* stream) {
   clear_error();

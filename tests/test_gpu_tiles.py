@@ -1,0 +1,87 @@
+"""Which tiles the library picks, so that a test of a tile's results is known to
+run that tile, and the forms that the tests of results alone do not reach."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+BAND = (1250.0, 1550.0, 81.92e-6)
+WIDE = (8, 14)
+
+
+def _plan(lib, C, n_t, n_dms, step):
+    return lib.Plan(C, *BAND, n_t, step * np.arange(n_dms), [1])
+
+
+def _subband(lib, S, per, coarse, fine, n_t, step=0.1):
+    dms = step * np.arange(coarse * fine)
+    return lib.Plan(S * per, *BAND, n_t, dms, [1], mode=lib.MODE_SUBBAND, n_subbands=S, coarse_dms=dms[::fine].copy())
+
+
+def _step2(lib, plan, Y):
+    import torch
+    D = torch.full((plan.n_dms, plan.n_samples), -1, dtype=torch.int32, device="cuda")
+    lib.sps_subband_step2(plan, Y, D)
+    return D
+
+
+def _narrow_step2(lib, plan, Y):
+    cfg = plan.config
+    cfg.step2 = lib.DedispConfig(4, 8, 4, 1, 4, 0)
+    plan.config = cfg
+    return _step2(lib, plan, Y)
+
+
+def _y(plan, per, seed):
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randint(0, 255 * per + 1, plan.y_shape, dtype=torch.int32, device="cuda",
+                         generator=gen).to(torch.int16).view(torch.uint16)
+
+
+# brute force on quads: (channels, samples, trials, step) -> wide tile, split
+@pytest.mark.parametrize("shape,wide,split", [((1536, 12500, 2048, 0.2), True, False), ((1536, 3001, 16, 0.2), True, True),
+                                              ((5000, 1201, 40, 0.05), False, True)])
+def test_brute_tiles(lib, shape, wide, split):
+    tiles, splits, made = _plan(lib, *shape).tiles()
+    assert tiles.brute.presum == 2 and not made
+    assert (tiles.brute.as_tuple()[:2] == WIDE) == wide
+    assert (splits > 1) == split
+
+
+def test_explicit_tiles_run_as_given(lib):
+    plan = _plan(lib, 96, 2000, 40, 0.2)
+    cfg = plan.config
+    cfg.brute = lib.DedispConfig(4, 8, 4, 2, 16, 2)
+    plan.config = cfg
+    assert plan.tiles()[0].brute.as_tuple() == (4, 8, 4, 2, 16, 2)
+    cfg.brute = lib.DedispConfig(4, 8, 4, 1, 8, 0)
+    plan.config = cfg
+    tiles, splits, made = plan.tiles()
+    assert tiles.brute.as_tuple() == (4, 8, 4, 1, 8, 0) and splits == 1 and not made
+
+
+@pytest.mark.parametrize("C,n_t,n_dms,step", [(100, 5001, 200, 0.5), (61, 4097, 70, 1.0), (64, 4096, 32, 2.0)])
+def test_small_single_channel_plans_make_their_copies(lib, C, n_t, n_dms, step):
+    plan = _plan(lib, C, n_t, n_dms, step)
+    tiles, splits, made = plan.tiles()
+    assert tiles.brute.presum == 0 and made
+
+
+# subbands, channels per subband, coarse DMs, trials per coarse DM, samples -> warps along DM
+@pytest.mark.parametrize("S,per,coarse,fine,n_t,warps", [(5, 120, 64, 32, 9001, 4), (17, 6, 128, 20, 4481, 3),
+                                                         (32, 12, 96, 31, 14400, 4)])
+def test_wide_step_two_runs_and_equals_narrow(lib, S, per, coarse, fine, n_t, warps):
+    import torch
+    plan = _subband(lib, S, per, coarse, fine, n_t)
+    tile = plan.tiles()[0].step2
+    assert tile.as_tuple()[:2] == WIDE and (tile.warps_dm, tile.warps_time) == (warps, 8 // warps)
+    Y = _y(plan, per, S)
+    got = _step2(lib, plan, Y)
+    assert torch.equal(got, _narrow_step2(lib, plan, Y))
+    assert plan.status() == 0
+
+
+def test_short_runs_take_narrow_step_two(lib):
+    """One or two warps along DM leave eight or four along time, whose stages do not fit two blocks an SM."""
+    assert _subband(lib, 32, 12, 192, 7, 14400).tiles()[0].step2.as_tuple()[:2] != WIDE
