@@ -185,7 +185,7 @@ sps_status run_step2(const sps_plan* p, const uint16_t* Y, int32_t* D, Stream& s
   a.n_t = p->n_t;
   a.dmax_tile = p->dmax_step2;
   a.flush_every = presum_wide(p->step2_tile.dms_per_thread, p->step2_tile.samples_per_thread / 2)
-                      ? (65536 - (int32_t)kWideCount) / (255 * (p->channels / p->n_subbands))
+                      ? step2_wide_flush(p->channels, p->n_subbands)
                       : p->step2_flush;
   a.D = D;
   a.status = p->d_status;

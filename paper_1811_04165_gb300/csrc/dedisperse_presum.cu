@@ -16,8 +16,8 @@
 // kStages mbarrier-tracked stages.  A 32-bit load holds two samples of a unit
 // sum in 16-bit lanes: one add accumulates 2 K channel-samples, with no
 // unpacking.  Samples outside a series' written range reach only output lanes
-// past the end of the row (a lane's carry runs towards later samples), which
-// are never stored.  Unit sums
+// past the end of the row, which are never stored (a lane's carry runs towards
+// later samples; the wide tile's counts cannot carry, see kWideFolds).  Unit sums
 // are <= 255 K, so 16-bit lanes are exact for 65535 / (255 K) units (128 pairs,
 // 64 quads); partial sums fold into int32 registers that often.  A group whose
 // size is not a multiple of K ends in a shorter unit.

@@ -412,6 +412,29 @@ size_t step2_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int32_t n
   return 2 * stage + (Di * n_subbands * 4 + 15) / 16 * 16 + 16;
 }
 
+int32_t step2_wide_flush(int32_t channels, int32_t n_subbands) {
+  return (65536 - (int32_t)kWideCount) / (255 * (channels / n_subbands));
+}
+
+// As step2_wide_kernel counts them: two subbands at a time inside a chunk, one at
+// an odd chunk's end.
+int32_t step2_wide_folds(const sps_dedisp_config& c, int32_t channels, int32_t n_subbands) {
+  const int32_t every = step2_wide_flush(channels, n_subbands);
+  int32_t folds = 0, pending = 0;
+  for (int32_t sb = 0; sb < n_subbands; sb += c.chunk) {
+    const int32_t cs = std::min(c.chunk, n_subbands - sb);
+    for (int32_t sl = 0; sl < cs; sl += 2) {
+      const int32_t n = std::min(2, cs - sl);
+      if (pending + n > every) {
+        folds++;
+        pending = 0;
+      }
+      pending += n;
+    }
+  }
+  return folds;
+}
+
 size_t step2_wide_smem_bytes(const sps_dedisp_config& c, int32_t dmax_tile, int32_t n_subbands) {
   const size_t stage = 2 * (size_t)c.chunk * copy_bytes(c, dmax_tile);
   return kWideStages * stage + (size_t)c.warps_dm * kWideTrials * n_subbands * 2 + 8 * kWideStages;

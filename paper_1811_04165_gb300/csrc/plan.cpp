@@ -191,9 +191,10 @@ double pass_us(const sps_plan* p, int64_t blocks, int64_t per_sm, int64_t chunks
 
 // The tile step two runs with.  The default one leaves the choice to the library,
 // which takes the wide tile of eight warps (along DM up to the longest run of
-// trials of one coarse DM, the rest along time) where two subbands' sums fit its
-// lanes between folds, two blocks an SM, and the grid is at least two rounds of
-// them: 64 coarse x 32 fine trials of 12500 samples 97 -> 83 us, 64 x 24 (8
+// trials of one coarse DM, the rest along time; runs of at most 16 trials leave
+// stages too long for two blocks) where two subbands' sums fit its lanes between
+// folds, the folds its counts (kWideFolds), two blocks an SM, and the grid is at
+// least two rounds of them: 64 coarse x 32 fine trials of 12500 samples 97 -> 83 us, 64 x 24 (8
 // subbands) 41 -> 32; with one round (24 x 32) it takes 25 us against 23.  Smaller
 // grids take the default tile or smaller ones by the model of pass_us: 13 coarse x
 // 8 fine trials of 1697 samples, 48 subbands 18.0 -> 7.2 us in tiles of 8 x 128.
@@ -214,7 +215,8 @@ sps_dedisp_config choose_step2(const sps_plan* p, const sps_dedisp_config& c) {
     const int64_t tt = 32 * w.warps_time * w.samples_per_thread;
     const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
     const bool fits = 2 * (step2_wide_smem_bytes(w, dmax, p->n_subbands) + 1024) <= (size_t)p->smem_per_sm;
-    if (fits && blocks >= 4 * p->sms) return w;
+    const bool counts = step2_wide_folds(w, p->channels, p->n_subbands) <= kWideFolds;
+    if (fits && counts && blocks >= 4 * p->sms) return w;
   }
   sps_dedisp_config best = c;
   double least = 1e30;

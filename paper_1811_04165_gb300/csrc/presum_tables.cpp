@@ -16,7 +16,9 @@
 //            to even (copy 1 at d - 1 holds the samples from d on);
 //   chunks : per (DM tile, group), its units in order, as many per chunk as fit
 //            a shared-memory stage (windows differ in length and number over the
-//            band, so a chunk holds more units where they are small);
+//            band, so a chunk holds more units where they are small); where the
+//            wide tile's folds would otherwise be too many, chunks end where its
+//            lanes are full;
 //   copies : per chunk, the windows of series copies the tile reads -- one per
 //            (tuple, parity of d) that occurs, each just long enough for its
 //            trials -- packed back to back in the stage: {row, start, (stage
@@ -148,6 +150,14 @@ sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int3
   const int32_t di_pad = presum_di_pad(cfg);
   const int32_t most = std::min(presum_fold_units(cfg), kPresumChunkUnits);
   const int32_t n_tiles = (rows + Di - 1) / Di;
+  // The wide tile folds at most kWideFolds times.  A fold comes when the next chunk
+  // does not fit the lanes and so moves at least fold - most + 1 units; where that
+  // leaves too many, chunks are cut so that each moves `fold` units.
+  const int32_t fold = presum_fold_units(cfg);
+  const bool wide = presum_wide(cfg.dms_per_thread, cfg.samples_per_thread / 2);
+  const bool cut = wide && (U - 1) / (fold - most + 1) > kWideFolds;
+  if (wide && (U - 1) / fold > kWideFolds)
+    return fail(SPS_ERR_UNSUPPORTED, "more folds than the wide tile's counts hold");
 
   // series: per unit, every tuple over all trials
   std::vector<int32_t> sbase((size_t)G * U);
@@ -206,12 +216,13 @@ sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int3
       }
       for (int32_t u0 = 0; u0 < U;) {
         int32_t n = 0, need = 0;
-        while (u0 + n < U && n < most && need + bytes[u0 + n] + 2 * di_pad <= stage_bytes) {
+        const int32_t end = cut ? std::min(U, (u0 / fold + 1) * fold) : U;
+        while (u0 + n < end && n < most && need + bytes[u0 + n] + 2 * di_pad <= stage_bytes) {
           need += bytes[u0 + n] + 2 * di_pad;
           n++;
         }
         if (n == 0) return fail(SPS_ERR_UNSUPPORTED, "a pre-summed unit's windows exceed a stage");
-        if (n > 4 && u0 + n < U) n &= ~1;  // units are added two at a time
+        if (n > 4 && u0 + n < end) n &= ~1;  // units are added two at a time
         int32_t at = n * 2 * di_pad;  // windows follow the offset table
         lists.emplace_back();
         const size_t table = out->offs.size();
@@ -281,6 +292,18 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
   for (int32_t tile = 0; tile < n_tiles; tile++)
     for (int32_t g = 0; g < G; g++) {
       const int4 chunks = t.chunk_rows[(size_t)tile * G + g];
+      // the folds of a block that sums all chunks (one with a share of them makes no more)
+      int32_t folds = 0, pending = 0;
+      for (int32_t q = 0; q < chunks.y; q++) {
+        const int32_t n = t.copies[((size_t)chunks.x + q) * (t.copies_max + 1) + t.copies_max].z;
+        if (pending + n > presum_fold_units(cfg)) {
+          folds++;
+          pending = 0;
+        }
+        pending += n;
+      }
+      if (presum_wide(cfg.dms_per_thread, cfg.samples_per_thread / 2) && folds > kWideFolds)
+        return say("more folds than the wide tile's counts hold", tile, g, folds, 0);
       int32_t chunk = 0, chunk_u0 = 0;  // the unit's chunk and the chunk's first unit
       for (int32_t u = 0; u < U; u++) {
         const int32_t c0 = g * per + K * u, n = std::min(K, per - K * u), e = c0 + n - 1;

@@ -115,7 +115,7 @@ struct PresumPassArgs {
   int32_t n_dm;            // delay-table rows
   int32_t n_groups;
   int32_t group_units;     // units per group
-  int32_t fold_units;      // units a 16-bit lane sums exactly: 65535 / (255 K)
+  int32_t fold_units;      // units a 16-bit lane sums exactly between folds (presum_fold_units)
   int32_t splits;          // blocks per output tile, each summing a share of its chunks (int32 rows, zeroed before)
   int32_t max_start;       // bound on any staged window's start (the pass's largest delay)
   int32_t n_out;
@@ -128,10 +128,14 @@ struct PresumPassArgs {
 };
 
 // The wide register tile of the pre-summed pass, 8 trials x 7 words per thread:
-// its 16-bit lanes fold into 8-bit counts of kWideCount.
+// its 16-bit lanes fold into 8-bit counts of kWideCount.  Sums of kWideChannels
+// channels stay within 255 counts, and kWideFolds folds, of at most 15 counts each,
+// keep any lane within them: lanes past the end of a row add up bytes that nothing
+// wrote, and a count that ran over would carry into a valid sum's.
 constexpr bool presum_wide(int nd, int nw) { return nd == 8 && nw == 7; }
 constexpr uint32_t kWideCount = 4096;
-constexpr int32_t kWideChannels = 4096;        // sums of more channels pass 255 counts
+constexpr int32_t kWideChannels = 4096;
+constexpr int32_t kWideFolds = 17;
 
 // One pre-summed series: channels c0 .. c0 + n - 1, channel c0 + j (j < n - 1)
 // taken rel[j] samples later than the last one.
@@ -245,6 +249,10 @@ size_t u8_smem_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile, int32_t gr
 int u8_groups_per_block(int32_t n_groups, int64_t tiles);
 int u8_window_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile);
 int u8_di_pad(const sps_dedisp_config& cfg);
+// The wide step two: subbands its lanes sum exactly between folds, and the folds
+// it makes over all of them.
+int32_t step2_wide_flush(int32_t channels, int32_t n_subbands);
+int32_t step2_wide_folds(const sps_dedisp_config& cfg, int32_t channels, int32_t n_subbands);
 size_t step2_wide_smem_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile, int32_t n_subbands);
 size_t step2_smem_bytes(const sps_dedisp_config& cfg, int32_t dmax_tile, int32_t n_subbands);
 

@@ -4,7 +4,8 @@
 // Keeping int32 sums beside the 16-bit lanes takes three registers per word; the
 // counts take half a register: a fold moves the lanes' multiples of kWideCount
 // (4096) into 8-bit fields, the four samples of two words to a register, and
-// leaves the remainders in the lanes.  Sums up to 255 * 4096 + 65535 are exact.
+// leaves the remainders in the lanes.  Sums up to 255 * 4096 + 65535 are exact, and
+// with at most kWideFolds folds no lane's count passes 255, whatever it adds up.
 #pragma once
 
 #include <cstdint>
