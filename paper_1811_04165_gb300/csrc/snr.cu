@@ -59,22 +59,23 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* scratch) {
 }
 
 // Scans the row at buf[4 .. 4 + n_t) in place into P[k] = buf[3 + k] (k = 0 ..
-// n_t); returns the sum of the samples this thread scanned.  Each thread scans
+// n_t); returns the sum of the samples this thread scanned (in 64 bits: 588
+// samples of 28 700 saturated channels pass 2^32).  Each thread scans
 // a run of `per` samples (a multiple of 4 with per / 4 odd, so the 16-byte
 // accesses of a warp are conflict-free).
-__device__ uint32_t scan_row_v4(uint32_t* buf, int n_t, uint32_t* scratch) {
+__device__ unsigned long long scan_row_v4(uint32_t* buf, int n_t, uint32_t* scratch) {
   if (threadIdx.x == 0) buf[3] = 0u;
   int per = ((n_t + blockDim.x - 1) / blockDim.x + 3) / 4 * 4;
   if ((per / 4) % 2 == 0) per += 4;
   const int b = min(n_t, (int)threadIdx.x * per), e = min(n_t, b + per);
   const int ev = b + (e - b) / 4 * 4;  // vector part [b, ev)
-  uint32_t s = 0;
-  for (int t = b; t < ev; t += 4) {
+  unsigned long long s = 0;
+  for (int t = b; t < ev; t += 4) {  // (samples are below 2^31, so pairs fit 32 bits)
     const uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
-    s += v.x + v.y + v.z + v.w;
+    s += (unsigned long long)(v.x + v.y) + (v.z + v.w);
   }
   for (int t = ev; t < e; t++) s += buf[4 + t];
-  uint32_t run = block_exclusive_scan(s, scratch);
+  uint32_t run = block_exclusive_scan((uint32_t)s, scratch);
   for (int t = b; t < ev; t += 4) {
     uint4 v = *reinterpret_cast<const uint4*>(buf + 4 + t);
     v.x += run;
@@ -135,7 +136,7 @@ __device__ bool stage_row(const int32_t* row, int n_t, uint32_t* buf, uint64_t* 
 // The row staged and scanned: (*P)[k] = sum_{u<k} D[u] for k = 0..n_t.  *seg = the
 // sum of the samples this thread scanned (the threads' segments tile the row).
 __device__ bool load_prefix(const int32_t* row, int n_t, uint32_t* buf, uint32_t* scratch, uint64_t* bar,
-                            bool use_tma, uint32_t* status, uint32_t* seg, const uint32_t** P) {
+                            bool use_tma, uint32_t* status, unsigned long long* seg, const uint32_t** P) {
   int s = 0;
   if (!stage_row(row, n_t, buf, bar, use_tma, status, &s)) return false;
   *seg = scan_row_v4(buf, n_t + s, scratch);
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(kMaxThreads, FAST ? 2 : 1) snr_kernel(SnrArgs 
   const int n_t = a.n_t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   pdl_wait();  // the rows are written
-  uint32_t seg = 0;
+  unsigned long long seg = 0;
   const uint32_t* P;
   if (!load_prefix(a.D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, a.status, &seg, &P)) return;
 
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(kMaxThreads, FAST ? 2 : 1) snr_kernel(SnrArgs 
     // S1 = P[N f]: T less the samples after the last whole window (fewer than f)
 #pragma unroll
     for (int k = 0; k < NWP; k++)
-      s1t[k] = (unsigned long long)seg -
+      s1t[k] = seg -
                (threadIdx.x == 0 ? (unsigned long long)(P[n_t] - P[n_t / W[k] * W[k]]) : 0ull);
   } else {
 #pragma unroll
@@ -371,7 +372,7 @@ integrate_kernel(const int32_t* D, int n_dms, int n_t, const int32_t* widths, in
   __shared__ uint32_t scratch[32];
   __shared__ uint64_t bar;
   const int i = blockIdx.x;
-  uint32_t seg = 0;
+  unsigned long long seg = 0;
   const uint32_t* P;
   if (!load_prefix(D + (int64_t)i * n_t, n_t, buf, scratch, &bar, use_tma != 0, status, &seg, &P)) return;
   for (int wi = 0; wi < n_widths; wi++) {
@@ -552,7 +553,7 @@ __device__ __forceinline__ uint32_t quad(const uint4& v, int i) {
 // starts s zeros into the buffer (stage_row), so positions below count from those
 // and outputs start at s.
 template <int NW>
-__device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, uint32_t segsum, int s) {
+__device__ void row_stats_v4(const SnrArgs& a, const uint32_t* buf, int row, unsigned long long segsum, int s) {
   constexpr int WMAX = 1 << (NW - 1);
   __shared__ unsigned long long ps2[kMaxThreads / 32][NW], ptot[kMaxThreads / 32], s1v[NW];
   __shared__ uint32_t pmx[kMaxThreads / 32][NW];
@@ -685,7 +686,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_pow2_kernel(SnrArgs a) {
   pdl_wait();  // the row is written
   int s = 0;
   if (!stage_row(a.D + (int64_t)row * a.n_t, a.n_t, buf, &bar, true, a.status, &s)) return;
-  const uint32_t segsum = scan_row_v4(buf, a.n_t + s, scratch);
+  const unsigned long long segsum = scan_row_v4(buf, a.n_t + s, scratch);
   row_stats_v4<NW>(a, buf, row, segsum, s);
 }
 
@@ -762,7 +763,8 @@ __device__ __forceinline__ void staged_quads(const uint32_t* stage, int j, uint4
 // D[base + 128 + 4l ..]; `run`: P at the chunk's first sample, advanced past the
 // chunk.  p0[i] = P[base + 4l + i], p1[i] = P[base + 128 + 4l + i]; returns the
 // chunk's sum (the same in every lane).
-__device__ __forceinline__ uint32_t scan_chunk(const uint4& a, const uint4& b, uint32_t& run, uint4& p0, uint4& p1) {
+__device__ __forceinline__ unsigned long long scan_chunk(const uint4& a, const uint4& b, uint32_t& run, uint4& p0,
+                                                         uint4& p1) {
   const int lane = threadIdx.x & 31;
   const uint32_t sa = a.x + a.y + a.z + a.w, sb = b.x + b.y + b.z + b.w;
   uint32_t xa = sa, xb = sb;
@@ -781,7 +783,7 @@ __device__ __forceinline__ uint32_t scan_chunk(const uint4& a, const uint4& b, u
   p1.z = p1.y + b.y;
   p1.w = p1.z + b.z;
   run += ta + tb;
-  return ta + tb;
+  return (unsigned long long)ta + tb;
 }
 
 // Stores a scanned chunk in ring slot `slot` (and slot 0's mirror).
@@ -919,7 +921,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) snr_stream_kernel(SnrArgs a) {
       // chunk c + 1 (the lookahead past the segment's end included) into the other slot
       wait_staged<1>();
       staged_quads(stage, c + 1, da, db);
-      const uint32_t ct = scan_chunk(da, db, run, p0, p1);
+      const unsigned long long ct = scan_chunk(da, db, run, p0, p1);
       if (c + 1 < ce) tot += ct;
       store_chunk(ring, (c + 1) & 1, p0, p1);
       stage_chunk(stage, Drow, c + 3, ce, n_t);  // into chunk c's staging slot, read before
