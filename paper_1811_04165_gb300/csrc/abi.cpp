@@ -1,7 +1,9 @@
 // extern "C" entry points of libsps.so: argument checks, then kernel launches.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <string>
+#include <unordered_map>
 
 #include "sps_internal.h"
 
@@ -22,6 +24,29 @@ sps_status cuda_fail(cudaError_t e, const char* what) {
 }
 
 void clear_error() { g_last_error.clear(); }
+
+cudaError_t allow_shared(const void* kernel) {
+  // a kernel's static shared memory is fixed when it is compiled
+  static std::mutex m;
+  static std::unordered_map<const void*, int> fixed;
+  int own = -1;
+  {
+    std::lock_guard<std::mutex> lock(m);
+    const auto it = fixed.find(kernel);
+    if (it != fixed.end()) own = it->second;
+  }
+  if (own < 0) {
+    cudaFuncAttributes a;
+    if (cudaError_t e = cudaFuncGetAttributes(&a, kernel)) return e;
+    own = (int)a.sharedSizeBytes;
+    std::lock_guard<std::mutex> lock(m);
+    fixed[kernel] = own;
+  }
+  int dev = 0, most = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  if (cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - own);
+}
 
 sps_status plan_create(const sps_plan_desc* d, sps_plan** out);
 

@@ -56,6 +56,12 @@ struct Stream {
   }
 };
 
+// Allows a kernel all the dynamic shared memory its block may use on the current
+// device.  The limit is shared by every host thread, so each call sets the same
+// one: a limit of a launch's own size could be lowered by another thread's before
+// that launch.
+cudaError_t allow_shared(const void* kernel);
+
 template <class... P, class... A>
 cudaError_t launch(Stream& s, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, A... args) {
   cudaLaunchAttribute after{};
@@ -71,9 +77,10 @@ cudaError_t launch(Stream& s, void (*kernel)(P...), dim3 grid, unsigned threads,
   s.first = false;
   // beyond the default 48 KB (static shared memory included) a kernel has to be
   // allowed its size; most small plans stay below and save the call
-  if (smem > 40 * 1024)
-    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
-  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  cudaError_t e = smem > 40 * 1024 ? allow_shared(reinterpret_cast<const void*>(kernel)) : cudaSuccess;
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later call
+  return e;
 }
 
 // Kernel-side description of one de-dispersion pass over uint8 channels
