@@ -172,6 +172,10 @@ void step2_tiles(const sps_plan* p, int32_t di, std::vector<int32_t>* tiles, int
   }
 }
 
+// Blocks along a grid's second dimension (time tiles of the uint8 passes, DM tiles
+// of step two).  A tile that would need more is not taken for another.
+constexpr int64_t kMaxGridY = 65535;
+
 bool same_tile(const sps_dedisp_config& a, const sps_dedisp_config& b) {
   return a.dms_per_thread == b.dms_per_thread && a.samples_per_thread == b.samples_per_thread &&
          a.warps_dm == b.warps_dm && a.warps_time == b.warps_time && a.chunk == b.chunk && a.presum == b.presum;
@@ -216,14 +220,14 @@ sps_dedisp_config choose_step2(const sps_plan* p, const sps_dedisp_config& c) {
     const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
     const bool fits = 2 * (step2_wide_smem_bytes(w, dmax, p->n_subbands) + 1024) <= (size_t)p->smem_per_sm;
     const bool counts = step2_wide_folds(w, p->channels, p->n_subbands) <= kWideFolds;
-    if (fits && counts && blocks >= 4 * p->sms) return w;
+    if (fits && counts && blocks >= 4 * p->sms && (int64_t)(tiles.size() / 3) <= kMaxGridY) return w;
   }
   sps_dedisp_config best = c;
   double least = 1e30;
   for (const Tile& t : narrow) {
     step2_tiles(p, t.c.warps_dm * t.c.dms_per_thread, &tiles, &dmax);
     const size_t smem = step2_smem_bytes(t.c, dmax, p->n_subbands);
-    if (smem > (size_t)p->max_smem) continue;
+    if (smem > (size_t)p->max_smem || (int64_t)(tiles.size() / 3) > kMaxGridY) continue;
     const int64_t tt = 32 * t.c.warps_time * t.c.samples_per_thread;
     const int64_t blocks = (int64_t)(tiles.size() / 3) * ((p->n_t + tt - 1) / tt);
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(2, p->smem_per_sm / (smem + 1024)));
@@ -314,7 +318,7 @@ sps_dedisp_config choose_u8(const sps_plan* p, const sps_dedisp_config& c, doubl
   for (const Tile& t : tiles) {
     const int32_t di = t.c.warps_dm * t.c.dms_per_thread, tt = 32 * t.c.warps_time * t.c.samples_per_thread;
     const size_t smem = u8_smem_bytes(t.c, cached_spread(p, brute ? 0 : 1, di), per, G);
-    if (smem > (size_t)p->max_smem) continue;
+    if (smem > (size_t)p->max_smem || (n_out + tt - 1) / tt > kMaxGridY) continue;
     const int64_t warps = t.c.warps_dm * t.c.warps_time;
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(16 / warps, p->smem_per_sm / (smem + 1024)));
     const int64_t tiles_n = (rows + di - 1) / di * ((n_out + tt - 1) / tt);
@@ -389,9 +393,11 @@ void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_confi
   };
   sps_dedisp_config wide;
   if (wide_form(c, p->channels, &wide)) {
+    const int64_t tt = 32 * wide.samples_per_thread;
     for (int32_t warps : {8, 4}) {
       wide.warps_dm = warps;
       wide.chunk = 4;  // single units, for the stage check
+      if ((p->n_t + tt - 1) / tt > kMaxGridY) continue;
       if (cached_presum_stage(p, 0, wide) > presum_wide_stage(wide)) continue;
       wide.chunk = c.chunk;
       consider(wide, 16 / warps, 500, 380);
