@@ -161,12 +161,12 @@ sps_status sps_plan_workspace_bytes(const sps_plan* plan, size_t* bytes);
 sps_status sps_plan_get_config(const sps_plan* plan, sps_kernel_config* out);
 /* Validates every field against the device's limits before accepting it. */
 sps_status sps_plan_set_config(sps_plan* plan, const sps_kernel_config* cfg);
-/* The de-dispersion tiles the plan's kernels run with: the configuration, with
+/* The tiles the plan's kernels run with: the configuration, with
  * the library's choice where that is left to it.  channel_splits: the shares of
  * the channels that blocks of their own sum (pre-summed brute force, else 1);
  * copies_in_pass: 1 when the single-channel pass makes the shifted copies of its
  * windows itself, else 0.  Such tiles need not be among those that
- * sps_plan_set_config accepts; `snr` is the configuration's. */
+ * sps_plan_set_config accepts; snr.threads is that of rows staged whole. */
 sps_status sps_plan_get_tiles(const sps_plan* plan, sps_kernel_config* tiles, int32_t* channel_splits,
                               int32_t* copies_in_pass);
 

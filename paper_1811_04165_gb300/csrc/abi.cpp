@@ -396,7 +396,9 @@ sps_status sps_plan_get_tiles(const sps_plan* p, sps_kernel_config* tiles, int32
   clear_error();
   if (sps_status s = check_plan(p)) return s;
   if (!tiles || !channel_splits || !copies_in_pass) return fail(SPS_ERR_INVALID_ARG, "null output");
-  *tiles = {p->brute_tile, p->step1_tile, p->step2_tile, p->cfg.snr};
+  const bool decimate = p->smoothing == SPS_SMOOTH_DECIMATE;
+  *tiles = {p->brute_tile, p->step1_tile, p->step2_tile,
+            {snr_threads((int32_t)p->dms.size(), p->n_t, decimate, p->cfg.snr.threads)}};
   *channel_splits = p->brute_splits;
   *copies_in_pass = p->build_copies ? 1 : 0;
   return SPS_OK;

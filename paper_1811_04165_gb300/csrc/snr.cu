@@ -1110,15 +1110,21 @@ size_t stream_smem(int nw, int threads) {
 // rows fill the GPU, short ones take fewer threads each, so that more rows share an
 // SM and a row's barriers join fewer warps (4096 rows of 1000 samples, widths 1 ..
 // 64: 46 us with 256 threads, 22 with 64; of 7000 samples 79 and, with 128, 68; of
-// 12500 samples 109 against 119 with 128); decimation does less work per sample
-// (4096 rows of 4096 samples 49 -> 24 us with 32).  Few rows keep 256 (32 rows of
-// 12500 samples: 11 us, 20 with 64).
-int snr_threads(const SnrArgs& a, int threads) {
-  if (threads != 256 || a.n_dms <= 152) return threads;
-  if (a.decimate) return a.n_dms > 608 && a.n_t <= 4500 ? 32 : (a.n_t <= 8000 ? 64 : 96);
-  if (a.n_dms <= 608) return a.n_t <= 3000 ? 128 : 256;
-  return a.n_t <= 4500 ? 64 : (a.n_t <= 10500 ? 128 : 256);
+// 12500 samples 109 against 119 with 128; with up to eight rows an SM, 64 threads
+// are too few sooner: 620 rows of 4500 samples 18.7 us, 14.8 with 128, 17.4 with
+// 256); decimation does less work per sample (4096 rows of 4096 samples 49 -> 24 us
+// with 32).  Rows of which an SM holds only a few keep 256, since nothing else hides
+// a row's barriers and scan there (decimation of 4096 rows of 18000 samples 91 us
+// with 96 threads, 92 with 224; of 20000 127 and 121 with 288; of 55000 379 and
+// 315); so do few rows (32 rows of 12500 samples: 11 us, 20 with 64).
+int snr_threads(int32_t n_dms, int32_t n_t, bool decimate, int threads) {
+  if (threads != 256 || n_dms <= 152) return threads;
+  if (decimate && n_t > 18500) return 256;
+  if (decimate) return n_dms > 608 && n_t <= 4500 ? 32 : (n_t <= 8000 ? 64 : 96);
+  if (n_dms <= 608) return n_t <= 3000 ? 128 : 256;
+  return n_t <= (n_dms <= 1216 ? 2000 : 4500) ? 64 : (n_t <= 10500 ? 128 : 256);
 }
+
 
 // The detection, when asked for.
 sps_status launch_detect(const SnrArgs& a, Stream& st) {
@@ -1143,7 +1149,7 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
   // rows that do not all start on 16 bytes need room for up to three zeros each
   const bool aligned = tma_ok(a.D, a.n_t);
   const int room = aligned ? 0 : 3;
-  const unsigned threads = (unsigned)snr_threads(a, c.threads);
+  const unsigned threads = (unsigned)snr_threads(a.n_dms, a.n_t, a.decimate != 0, c.threads);
   if (pow2_form(a)) {
     const size_t smem = pow2_smem(a.n_t + room, a.pow2_widths);
     const bool fits = row_fits(a.max_smem, a.n_t, smem - prefix_smem(a.n_t) + 8192);

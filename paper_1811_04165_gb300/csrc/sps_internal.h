@@ -211,6 +211,8 @@ struct SnrArgs {
 sps_status launch_u8_pass(const U8PassArgs& a, const sps_dedisp_config& cfg, Stream& st);
 sps_status launch_step2(const Step2Args& a, const sps_dedisp_config& cfg, Stream& st);
 sps_status launch_snr(const SnrArgs& a, const sps_snr_config& cfg, Stream& st);
+// Threads per row that the library takes where a configuration has `threads`.
+int snr_threads(int32_t n_dms, int32_t n_t, bool decimate, int threads);
 sps_status launch_integrate(const int32_t* D, int32_t n_dms, int32_t n_t, const int32_t* widths,
                             int32_t n_widths, int32_t decimate, int32_t* B, int max_smem, uint32_t* status,
                             Stream& st);

@@ -85,3 +85,13 @@ def test_wide_step_two_runs_and_equals_narrow(lib, S, per, coarse, fine, n_t, wa
 def test_short_runs_take_narrow_step_two(lib):
     """One or two warps along DM leave eight or four along time, whose stages do not fit two blocks an SM."""
     assert _subband(lib, 32, 12, 192, 7, 14400).tiles()[0].step2.as_tuple()[:2] != WIDE
+
+
+@pytest.mark.parametrize("n_dms,n_t,decimate,threads", [(200, 55000, 1, 256), (4096, 20000, 1, 256), (4096, 12500, 1, 96),
+                                                        (620, 4500, 0, 128), (620, 2000, 0, 64), (2000, 4500, 0, 64),
+                                                        (100, 3000, 0, 256)])
+def test_snr_threads(lib, n_dms, n_t, decimate, threads):
+    """Rows of which an SM holds few keep their threads: decimation of 4096 rows of 55000 samples takes 379 us with
+    96, 315 with 224; 620 rows of 4500 samples 18.7 us with 64, 14.8 with 128."""
+    plan = lib.Plan(16, *BAND, n_t, 1e-3 * np.arange(n_dms), [1, 10], smoothing=decimate)
+    assert plan.tiles()[0].snr.threads == threads
