@@ -284,7 +284,7 @@ sps_status dedisperse_into(const sps_plan* p, const uint8_t* x, int64_t pitch, i
 bool batched_pass_form(const sps_plan* p) { return p->mode == SPS_MODE_BRUTE && p->cfg.brute.presum > 0; }
 
 sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
-                         size_t ws_bytes, cudaStream_t stream, PresumPassArgs* args) {
+                         size_t ws_bytes, int32_t splits, cudaStream_t stream, PresumPassArgs* args) {
   Stream st(stream);
   if (!batched_pass_form(p)) return fail(SPS_ERR_INVALID_ARG, "not a pre-summed brute-force plan");
   sps_status s = check_x(p, x, pitch);
@@ -294,7 +294,7 @@ sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int
   uint8_t* w = static_cast<uint8_t*>(ws);
   if ((s = prepare_input(p, &x, &pitch, &w, st))) return s;
   return presum_prepass(p, p->brute_tile, x, pitch, w, (int32_t)p->dms.size(), p->channels, p->n_t, p->n_t,
-                        p->dmax_brute, D, 0, 1, st, args);
+                        p->dmax_brute, D, 0, splits, st, args);
 }
 
 sps_status snr_into(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,

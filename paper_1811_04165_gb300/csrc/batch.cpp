@@ -5,9 +5,9 @@
 // brute-force kernel is the pre-summed one are searched in three phases: their
 // pre-passes (series into each beam's own workspace region) on the branches;
 // then, per kernel configuration, ONE launch of the pass over a device work
-// list of (beam, DM tile, time tile) descriptors covering all those beams, so
-// the beams' tiles fill the GPU together with no per-beam tail wave; then their
-// S/N kernels on the branches again.  Other beams (single-channel kernel,
+// list of (beam, DM tile, time tile, channel split) descriptors covering all
+// those beams, so the beams' tiles fill the GPU together with no per-beam tail
+// wave; then their S/N kernels on the branches again.  Other beams (single-channel kernel,
 // subband mode) run their whole search on a branch, each branch owning a
 // region of the caller's workspace.  Beams are assigned largest first to the
 // branch with the least work so far (work = DM trials x samples x channels).
@@ -108,6 +108,59 @@ sps_status plan_layout(const sps_plan* const* plans, int32_t n, int32_t branches
   return SPS_OK;
 }
 
+// The channel splits of the batched beams, none more than the beam's own.  Splits
+// fill the SMs that a beam's blocks leave idle; in a batch the other beams' blocks
+// do so too.
+//   * Beams of one band and tile: the splits that a pass of all their blocks takes.
+//   * Mixed beams: their rounds of blocks blur, and what is left idle is about half
+//     of the longest block at the end; a beam is split by the factor that makes
+//     that and the splits' additions (0.24 ns per KB of output and split) least, in
+//     the measure of its block's length.
+// One beam of 1536 channels x 12500 samples x 96 trials 84 us (209 unsplit), eight
+// of them 466 (526); eight mixed beams of 32 .. 112 trials x 7000 samples 222 -> 166.
+std::vector<int32_t> batch_splits(const sps_plan* const* plans, const std::vector<char>& batched) {
+  const int32_t n = (int32_t)batched.size();
+  std::vector<int32_t> splits(n, 1);
+  int32_t first = -1;
+  bool alike = true;
+  int64_t blocks = 0;
+  double kb = 0.0, longest = 0.0;
+  for (int32_t b = 0; b < n; b++) {
+    if (!batched[b]) continue;
+    const sps_plan* p = plans[b];
+    if (first < 0) first = b;
+    alike = alike && p->channels == plans[first]->channels && p->brute_tile.warps_dm == plans[first]->brute_tile.warps_dm &&
+            p->brute_tile.dms_per_thread == plans[first]->brute_tile.dms_per_thread;
+    blocks += pass_blocks(p, p->brute_tile);
+    kb += pass_out_kb(p);
+    longest = std::max(longest, pass_block_ns(p, p->brute_tile));
+  }
+  auto factor = [&](int32_t b, int32_t f) {
+    return std::min(plans[b]->brute_splits,
+                    std::max(1, (int32_t)(f * pass_block_ns(plans[b], plans[b]->brute_tile) / longest + 0.5)));
+  };
+  int32_t best = 1;
+  double least = 1e30;
+  for (int32_t f : {1, 2, 3, 4, 6, 8}) {
+    double tail = 0.0, added = 0.0;
+    for (int32_t b = 0; b < n; b++) {
+      if (!batched[b]) continue;
+      const int32_t s = factor(b, f);
+      tail = std::max(tail, 0.5 * pass_block_ns(plans[b], plans[b]->brute_tile) / s);
+      if (s > 1) added += 0.24 * (s + 1) * pass_out_kb(plans[b]);
+    }
+    if (tail + added < least) {
+      least = tail + added;
+      best = f;
+    }
+  }
+  for (int32_t b = 0; b < n; b++)
+    if (batched[b])
+      splits[b] = alike ? std::min(plans[b]->brute_splits, best_splits(plans[b], plans[b]->brute_tile, blocks, kb, &least))
+                        : factor(b, best);
+  return splits;
+}
+
 }  // namespace
 }  // namespace sps
 
@@ -149,6 +202,8 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
   for (auto& g : groups)
     for (int32_t b : g.second) pass_of[b] = n_passes++;
 
+  const std::vector<int32_t> splits = batch_splits(plans, L.batched);
+
   int cur = 0;
   SPS_CUDA(cudaGetDevice(&cur));
   if (cur != device) SPS_CUDA(cudaSetDevice(device));
@@ -171,15 +226,8 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
   };
   if (n_passes) {
     int64_t n_work = 0;
-    for (int32_t b = 0; b < n_beams; b++) {
-      if (!L.batched[b]) continue;
-      const sps_dedisp_config& c = plans[b]->brute_tile;
-      PresumPassArgs shape{};
-      shape.n_dm = (int32_t)plans[b]->dms.size();
-      shape.n_out = plans[b]->n_t;
-      shape.n_groups = 1;
-      n_work += presum_pass_blocks(shape, c);
-    }
+    for (int32_t b = 0; b < n_beams; b++)
+      if (L.batched[b]) n_work += pass_blocks(plans[b], plans[b]->brute_tile) * splits[b];
     if (cuda_ok(cudaMalloc(&batch->d_passes, sizeof(PresumPassArgs) * n_passes), "cudaMalloc"))
       cuda_ok(cudaMalloc(&batch->d_work, sizeof(int4) * n_work), "cudaMalloc");
   }
@@ -205,7 +253,7 @@ sps_status sps_batch_create(const sps_plan* const* plans, const sps_beam_buffers
       if (!L.batched[b]) {
         st = run_search(plans[b], u.x, u.x_pitch, u.D, w, L.ws_bytes[b], u.snr, u.peak_t, u.peak_val, u.best, sk);
       } else {
-        st = brute_prepass(plans[b], u.x, u.x_pitch, u.D, w, L.ws_bytes[b], sk, &passes[pass_of[b]]);
+        st = brute_prepass(plans[b], u.x, u.x_pitch, u.D, w, L.ws_bytes[b], splits[b], sk, &passes[pass_of[b]]);
         if (st == SPS_OK) cuda_ok(cudaEventRecord(pre_done[b], sk), "cudaEventRecord");
       }
     }

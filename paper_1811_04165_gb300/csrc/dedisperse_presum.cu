@@ -364,8 +364,8 @@ presum_pass_kernel(PresumPassArgs a, int wd, int wb) {
 }
 
 // Batched form: one launch over a work list of tiles from several passes of
-// the same configuration (several beams).  work[b] = {pass, DM tile, time
-// tile, group}; each pass's arguments (and its window bytes) live in `passes`.
+// the same configuration (several beams, brute force: one group).  work[b] =
+// {pass, DM tile, time tile, channel split}; each pass's arguments (and its window bytes) live in `passes`.
 template <int ND, int NW>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* __restrict__ work, int wd) {
@@ -373,7 +373,7 @@ presum_pass_list_kernel(const PresumPassArgs* __restrict__ passes, const int4* _
   // a copy: read through the pointer, every field is loaded anew after each of
   // the pass's memory-ordering statements (eight mixed beams 2003 -> 1954 us)
   const PresumPassArgs a = passes[w.x];
-  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, w.w, 0, wd, a.window_bytes);
+  presum_pass_block<ND, NW, presum_wide(ND, NW)>(a, w.y, w.z, 0, w.w, wd, a.window_bytes);
 }
 
 // Adds bytes o + j .. o + j + 15 of W (24 bytes, o in 0 .. 7), for j = 0 and
@@ -714,16 +714,16 @@ sps_status launch_presum_pass(const PresumPassArgs& a, const sps_dedisp_config& 
 int64_t presum_pass_blocks(const PresumPassArgs& a, const sps_dedisp_config& c) {
   const int Di = c.warps_dm * c.dms_per_thread;
   const int Tt = c.warps_time * 32 * c.samples_per_thread;
-  return (int64_t)((a.n_dm + Di - 1) / Di) * ((a.n_out + Tt - 1) / Tt) * a.n_groups;
+  return (int64_t)((a.n_dm + Di - 1) / Di) * ((a.n_out + Tt - 1) / Tt) * a.splits;
 }
 
 void presum_pass_work(const PresumPassArgs& a, const sps_dedisp_config& c, int32_t pass, std::vector<int4>* work) {
   const int Di = c.warps_dm * c.dms_per_thread;
   const int Tt = c.warps_time * 32 * c.samples_per_thread;
   const int tiles = (a.n_dm + Di - 1) / Di, ty = (a.n_out + Tt - 1) / Tt;
-  for (int g = 0; g < a.n_groups; g++)
-    for (int y = 0; y < ty; y++)
-      for (int t = 0; t < tiles; t++) work->push_back(make_int4(pass, t, y, g));
+  for (int y = 0; y < ty; y++)
+    for (int t = 0; t < tiles; t++)
+      for (int q = 0; q < a.splits; q++) work->push_back(make_int4(pass, t, y, q));
 }
 
 sps_status launch_presum_pass_list(const PresumPassArgs* d_passes, const int4* d_work, int64_t n_work,

@@ -348,6 +348,47 @@ bool build_copies(const sps_plan* p, double pass_us) {
   return 0.1 * pass_us < 2.5 + 4.0 * p->channels * (double)p->n_in / 6e6;
 }
 
+// Blocks of a pre-summed tile that one SM holds, and the ns a unit takes a round of
+// them (`half`: with at most half of them), as choose_tile says.
+struct PassRate { int64_t per_sm; double full, half; };
+
+PassRate pass_rate(const sps_plan* p, const sps_dedisp_config& c) {
+  const int64_t warps = c.warps_dm * c.warps_time;
+  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return {16 / warps, 500, 380};
+  const int64_t fit = p->smem_per_sm / (presum_smem_bytes(cached_presum_stage(p, 0, c)) + 1024);
+  return {std::max<int64_t>(1, std::min<int64_t>(16 / warps, fit)), 370, 290};
+}
+
+int64_t pass_blocks(const sps_plan* p, const sps_dedisp_config& c) {
+  const int64_t di = c.warps_dm * c.dms_per_thread, tt = 32 * c.warps_time * c.samples_per_thread;
+  return ((int64_t)p->dms.size() + di - 1) / di * ((p->n_t + tt - 1) / tt);
+}
+
+double pass_out_kb(const sps_plan* p) { return 4e-3 * (double)p->dms.size() * p->n_t; }
+
+double pass_block_ns(const sps_plan* p, const sps_dedisp_config& c) {
+  return ((p->channels + (1 << c.presum) - 1) >> c.presum) * pass_rate(p, c).full;
+}
+
+int32_t best_splits(const sps_plan* p, const sps_dedisp_config& c, int64_t blocks, double out_kb, double* least) {
+  const PassRate r = pass_rate(p, c);
+  const int64_t units = (p->channels + (1 << c.presum) - 1) >> c.presum, slots = r.per_sm * p->sms;
+  int32_t best = 1;
+  *least = 1e30;
+  for (int32_t s : {1, 2, 3, 4, 6, 8, 12, 16}) {
+    if (s > 1 && s > units / 8) break;
+    const int64_t whole = blocks * s / slots, last = blocks * s % slots;
+    double ns = whole * (units * r.full / s + 2000);
+    if (last) ns += units * (last > slots / 2 ? r.full : r.half) / s + 2000;
+    if (s > 1) ns += 0.24 * (s + 1) * out_kb;
+    if (ns < *least) {
+      *least = ns;
+      best = s;
+    }
+  }
+  return best;
+}
+
 // The tile and the channel splits the brute-force pass runs with, by a model of
 // its time.
 //   * The default pre-summed tile leaves the choice to the library.  The wide
@@ -372,23 +413,14 @@ void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_confi
     *tile = choose_u8(p, c, u8_us);
     return;
   }
-  const int64_t rows = (int64_t)p->dms.size(), units = (p->channels + (1 << c.presum) - 1) >> c.presum;
-  const double out_kb = 4e-3 * rows * p->n_t;
   double best = 1e30;
-  auto consider = [&](const sps_dedisp_config& t, int64_t per_sm, double full, double half) {
-    const int64_t di = t.warps_dm * t.dms_per_thread, tt = 32 * t.warps_time * t.samples_per_thread;
-    const int64_t blocks = (rows + di - 1) / di * ((p->n_t + tt - 1) / tt), slots = per_sm * p->sms;
-    for (int32_t s : {1, 2, 3, 4, 6, 8, 12, 16}) {
-      if (s > 1 && s > units / 8) break;
-      const int64_t whole = blocks * s / slots, last = blocks * s % slots;
-      double ns = whole * (units * full / s + 2000);
-      if (last) ns += units * (last > slots / 2 ? full : half) / s + 2000;
-      if (s > 1) ns += 0.24 * (s + 1) * out_kb;
-      if (ns < best) {
-        best = ns;
-        *tile = t;
-        *splits = s;
-      }
+  auto consider = [&](const sps_dedisp_config& t) {
+    double ns;
+    const int32_t s = best_splits(p, t, pass_blocks(p, t), pass_out_kb(p), &ns);
+    if (ns < best) {
+      best = ns;
+      *tile = t;
+      *splits = s;
     }
   };
   sps_dedisp_config wide;
@@ -400,13 +432,11 @@ void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_confi
       if ((p->n_t + tt - 1) / tt > kMaxGridY) continue;
       if (cached_presum_stage(p, 0, wide) > presum_wide_stage(wide)) continue;
       wide.chunk = c.chunk;
-      consider(wide, 16 / warps, 500, 380);
+      consider(wide);
     }
     if (best < 1e30) return;
   }
-  const size_t per_sm = p->smem_per_sm / (presum_smem_bytes(cached_presum_stage(p, 0, c)) + 1024);
-  const int64_t warps = c.warps_dm * c.warps_time;
-  consider(c, std::max<int64_t>(1, std::min<int64_t>(16 / warps, (int64_t)per_sm)), 370, 290);
+  consider(c);
 }
 
 int32_t presum_stage(const sps_plan* p, const sps_dedisp_config& c) {

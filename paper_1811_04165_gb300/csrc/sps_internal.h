@@ -276,6 +276,12 @@ struct ConfigCheck {
 };
 sps_status check_config(const sps_plan* p, const sps_kernel_config& cfg, ConfigCheck* out);
 sps_status apply_config(sps_plan* p, const sps_kernel_config& cfg);
+// The splits along the channels, and their modelled ns, of a pre-summed pass of the
+// plan's band with `c` over `blocks` output tiles of `out_kb` KB.
+int32_t best_splits(const sps_plan* p, const sps_dedisp_config& c, int64_t blocks, double out_kb, double* least);
+int64_t pass_blocks(const sps_plan* p, const sps_dedisp_config& c);  // output tiles of the brute-force pass
+double pass_out_kb(const sps_plan* p);
+double pass_block_ns(const sps_plan* p, const sps_dedisp_config& c);  // of an unsplit block on a full GPU
 bool wide_form(const sps_dedisp_config& c, int32_t channels, sps_dedisp_config* wide);
 sps_status run_search(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws, size_t ws_bytes,
                       double* snr, int32_t* peak_t, int32_t* peak_val, int32_t* best, cudaStream_t st);
@@ -283,11 +289,12 @@ sps_status dedisperse_into(const sps_plan* p, const uint8_t* x, int64_t pitch, i
                            size_t ws_bytes, cudaStream_t st);
 // The batched brute-force form (batch.cpp): plans whose brute-force kernel is
 // the pre-summed one run their pre-pass here (checks, zapping, the series into
-// the workspace) and return the arguments of their pass, which a batched list
-// launch then runs; snr_into is the S/N step of sps_search on its own.
+// the workspace, D zeroed where `splits` blocks share an output tile's channels)
+// and return the arguments of their pass, which a batched list launch then runs;
+// snr_into is the S/N step of sps_search on its own.
 bool batched_pass_form(const sps_plan* p);
 sps_status brute_prepass(const sps_plan* p, const uint8_t* x, int64_t pitch, int32_t* D, void* ws,
-                         size_t ws_bytes, cudaStream_t st, PresumPassArgs* args);
+                         size_t ws_bytes, int32_t splits, cudaStream_t st, PresumPassArgs* args);
 sps_status snr_into(const sps_plan* p, const int32_t* D, double* snr, int32_t* peak_t, int32_t* peak_val,
                     int32_t* best, cudaStream_t st);
 
