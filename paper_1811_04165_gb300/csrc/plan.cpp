@@ -394,16 +394,20 @@ int32_t best_splits(const sps_plan* p, const sps_dedisp_config& c, int64_t block
 //   * The default pre-summed tile leaves the choice to the library.  The wide
 //     tiles (8 trials x 7 words per thread; 8 or 4 warps, each 8 trials x 448
 //     samples) read shared memory at 81 % of its peak and half the series windows
-//     per output; they are taken where single units fit their stages.  The one of
-//     4 warps serves plans of few trials, whose tiles it fills better.
+//     per output; they are considered where single units fit their stages.  The
+//     one of 4 warps, and the default one itself (4 x 8 words, 32 trials x 512
+//     samples), serve plans whose trials or rounds they fill better: 384 channels x
+//     12500 samples x 700 trials, 0.1 apart, would be one round of wide blocks and
+//     four more (117 us with the pre-pass, 99 with the default tile).
 //   * A grid that leaves SMs idle, in its last round or altogether, is split
 //     along the channels: each split's blocks add their sums into zeroed rows.
 // Constants measured on the 1536-channel band, in ns: a unit takes a round of
 // resident blocks 500 (380 with at most half the SM's blocks), with the default
 // tile 370 (290); a block starts and ends in 2000; a split costs 0.24 per KB of
 // output (its additions reach the L2 at 4.3 TB/s).  64 trials x 12500 samples:
-// 140 us with the default tile, 160 wide, 59 wide in eight splits; 512 trials
-// (0.4 pc cm^-3 apart): 415, 266 and, in four splits, 237.
+// 131 us with the default tile, 52 wide in eight splits, 47 with the default tile
+// in six; 512 trials (0.4 pc cm^-3 apart): 415 with the default tile, 266 wide and,
+// in four splits, 237.
 void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_config* tile, int32_t* splits,
                  double* u8_us) {
   *tile = c;
@@ -434,7 +438,6 @@ void choose_tile(const sps_plan* p, const sps_dedisp_config& c, sps_dedisp_confi
       wide.chunk = c.chunk;
       consider(wide);
     }
-    if (best < 1e30) return;
   }
   consider(c);
 }

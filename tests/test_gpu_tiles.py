@@ -39,14 +39,31 @@ def _y(plan, per, seed):
                          generator=gen).to(torch.int16).view(torch.uint16)
 
 
-# brute force on quads: (channels, samples, trials, step) -> wide tile, split
-@pytest.mark.parametrize("shape,wide,split", [((1536, 12500, 2048, 0.2), True, False), ((1536, 3001, 16, 0.2), True, True),
-                                              ((5000, 1201, 40, 0.05), False, True)])
-def test_brute_tiles(lib, shape, wide, split):
-    tiles, splits, made = _plan(lib, *shape).tiles()
+# brute force on quads: (channels, samples, trials, step) -> warps of the wide tile (0: the configured one), split
+@pytest.mark.parametrize("shape,warps,split", [((1536, 3584, 2304, 0.2), 8, False), ((1536, 7013, 64, 0.2), 8, True),
+                                               ((384, 3001, 300, 0.3), 8, True), ((389, 7013, 577, 0.31), 4, True),
+                                               ((1536, 3001, 16, 0.2), 0, True), ((384, 12500, 700, 0.1), 0, False),
+                                               ((5000, 1201, 40, 0.05), 0, True)])
+def test_brute_tiles(lib, shape, warps, split):
+    """Each form of the pass is known to run, and equals the single-channel kernel.  (384 channels x 700 trials: one
+    wide round and four blocks more, 117 us, where the configured tile takes 99.)"""
+    import torch
+    plan = _plan(lib, *shape)
+    tiles, splits, made = plan.tiles()
     assert tiles.brute.presum == 2 and not made
-    assert (tiles.brute.as_tuple()[:2] == WIDE) == wide
+    assert (tiles.brute.warps_dm if tiles.brute.as_tuple()[:2] == WIDE else 0) == warps
     assert (splits > 1) == split
+    gen = torch.Generator(device="cuda").manual_seed(shape[0])
+    x = torch.randint(0, 256, (plan.channels, plan.pitch), dtype=torch.uint8, device="cuda", generator=gen)
+    got = torch.full((plan.n_dms, plan.n_samples), -1, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, got)
+    cfg = plan.config
+    cfg.brute = lib.DedispConfig(4, 16, 8, 1, 4, 0)
+    plan.config = cfg
+    want = torch.full((plan.n_dms, plan.n_samples), -2, dtype=torch.int32, device="cuda")
+    lib.sps_dedisperse(plan, x, want)
+    assert plan.status() == 0
+    assert torch.equal(got, want)
 
 
 def test_explicit_tiles_run_as_given(lib):
