@@ -100,6 +100,8 @@ typedef struct {
  * step one) selects the kernel: 0 sums single channels; 1 and 2 sum series of
  * 2^presum adjacent channels pre-added once per batch (pairs, quads), each
  * series taken at the delay of its highest-frequency channel.  All are exact.
+ * Pre-summed passes size a stage for `chunk` channels where the delays spread
+ * most, and elsewhere stage as many as fit (up to 16 series, or `chunk`).
  * A new plan's tiles leave the tile, and a split of the channels over more
  * blocks, to the library, which goes by the plan's size (so do the same values
  * set explicitly); other values are run as given, pre-summed brute force split

@@ -148,7 +148,7 @@ sps_status build_presum_tables(const std::vector<int32_t>& d, int32_t rows, int3
   const int32_t Di = cfg.warps_dm * cfg.dms_per_thread;
   const int32_t Tt = cfg.warps_time * 32 * cfg.samples_per_thread;
   const int32_t di_pad = presum_di_pad(cfg);
-  const int32_t most = std::min(presum_fold_units(cfg), kPresumChunkUnits);
+  const int32_t most = std::min(presum_fold_units(cfg), std::max(kPresumChunkUnits, presum_chunk(cfg)));
   const int32_t n_tiles = (rows + Di - 1) / Di;
   // The wide tile folds at most kWideFolds times.  A fold comes when the next chunk
   // does not fit the lanes and so moves at least fold - most + 1 units; where that
@@ -302,7 +302,12 @@ bool verify_presum_tables(const std::vector<int32_t>& d, int32_t rows, int32_t C
         }
         pending += n;
       }
-      if (presum_wide(cfg.dms_per_thread, cfg.samples_per_thread / 2) && folds > kWideFolds)
+      // a tile's first chunk holds the units its stage is sized for (an even number from six on)
+      const bool wide = presum_wide(cfg.dms_per_thread, cfg.samples_per_thread / 2);
+      const int32_t sized = std::min(U, presum_chunk(cfg)), held = t.copies[(size_t)chunks.x * (t.copies_max + 1) + t.copies_max].z;
+      if (!wide && held < (sized > 4 ? sized & ~1 : sized))
+        return say("fewer units in a chunk than its stage is sized for", tile, g, held, 0);
+      if (wide && folds > kWideFolds)
         return say("more folds than the wide tile's counts hold", tile, g, folds, 0);
       int32_t chunk = 0, chunk_u0 = 0;  // the unit's chunk and the chunk's first unit
       for (int32_t u = 0; u < U; u++) {

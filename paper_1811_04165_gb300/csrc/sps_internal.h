@@ -240,7 +240,7 @@ int presum_di_pad(const sps_dedisp_config& cfg);
 int presum_chunk(const sps_dedisp_config& cfg);  // units a stage is sized for
 int32_t presum_wide_stage(const sps_dedisp_config& cfg);  // bytes of a wide tile's stage
 int presum_fold_units(const sps_dedisp_config& cfg);  // units a 16-bit lane sums between folds
-constexpr int32_t kPresumChunkUnits = 16;             // most units per chunk
+constexpr int32_t kPresumChunkUnits = 16;             // most units per chunk, unless its stage is sized for more
 // Host tables (presum_tables.cpp): series count over all rows, the largest
 // packed window data of any (tile, group, chunk), and the full tables of one
 // configuration.

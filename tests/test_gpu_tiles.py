@@ -112,3 +112,21 @@ def test_snr_threads(lib, n_dms, n_t, decimate, threads):
     96, 315 with 224; 620 rows of 4500 samples 18.7 us with 64, 14.8 with 128."""
     plan = lib.Plan(16, *BAND, n_t, 1e-3 * np.arange(n_dms), [1, 10], smoothing=decimate)
     assert plan.tiles()[0].snr.threads == threads
+
+
+@pytest.mark.parametrize("tile", [(4, 8, 4, 1, 64, 1), (2, 8, 4, 1, 64, 1), (1, 8, 8, 1, 36, 1), (4, 8, 2, 1, 64, 1)])
+def test_large_chunks(lib, tile):
+    """Chunks of more than 16 series (one stage of them each), against the single-channel kernel."""
+    import torch
+    plan = _plan(lib, 389, 2011, 70, 0.05)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    x = torch.randint(0, 256, (389, plan.pitch), dtype=torch.uint8, device="cuda", generator=gen)
+    out = []
+    for t in (tile, (4, 8, 4, 1, 8, 0)):
+        cfg = plan.config
+        cfg.brute = lib.DedispConfig(*t)
+        plan.config = cfg
+        out.append(torch.full((70, 2011), -1, dtype=torch.int32, device="cuda"))
+        lib.sps_dedisperse(plan, x, out[-1])
+    assert plan.status() == 0
+    assert torch.equal(*out)
