@@ -348,15 +348,17 @@ bool build_copies(const sps_plan* p, double pass_us) {
   return 0.1 * pass_us < 2.5 + 4.0 * p->channels * (double)p->n_in / 6e6;
 }
 
-// Blocks of a pre-summed tile that one SM holds, and the ns a unit takes a round of
-// them (`half`: with at most half of them), as choose_tile says.
-struct PassRate { int64_t per_sm; double full, half; };
+// Blocks of a pre-summed tile that one SM holds, the ns a unit takes a round of
+// them (`half`: with at most half of them), and those of a block's start and end, as
+// choose_tile says.
+struct PassRate { int64_t per_sm; double full, half, ends; };
 
 PassRate pass_rate(const sps_plan* p, const sps_dedisp_config& c) {
   const int64_t warps = c.warps_dm * c.warps_time;
-  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return {16 / warps, 500, 380};
+  if (presum_wide(c.dms_per_thread, c.samples_per_thread / 2)) return {16 / warps, 500, 380, 2000};
   const int64_t fit = p->smem_per_sm / (presum_smem_bytes(cached_presum_stage(p, 0, c)) + 1024);
-  return {std::max<int64_t>(1, std::min<int64_t>(16 / warps, fit)), 370, 290};
+  return {std::max<int64_t>(1, std::min<int64_t>(16 / warps, fit)), 370, 290,
+          2000.0 + 600.0 * std::max(0, presum_chunk(c) - 4)};
 }
 
 int64_t pass_blocks(const sps_plan* p, const sps_dedisp_config& c) {
@@ -378,8 +380,8 @@ int32_t best_splits(const sps_plan* p, const sps_dedisp_config& c, int64_t block
   for (int32_t s : {1, 2, 3, 4, 6, 8, 12, 16}) {
     if (s > 1 && s > units / 8) break;
     const int64_t whole = blocks * s / slots, last = blocks * s % slots;
-    double ns = whole * (units * r.full / s + 2000);
-    if (last) ns += units * (last > slots / 2 ? r.full : r.half) / s + 2000;
+    double ns = whole * (units * r.full / s + r.ends);
+    if (last) ns += units * (last > slots / 2 ? r.full : r.half) / s + r.ends;
     if (s > 1) ns += 0.24 * (s + 1) * out_kb;
     if (ns < *least) {
       *least = ns;
@@ -403,7 +405,9 @@ int32_t best_splits(const sps_plan* p, const sps_dedisp_config& c, int64_t block
 //     along the channels: each split's blocks add their sums into zeroed rows.
 // Constants measured on the 1536-channel band, in ns: a unit takes a round of
 // resident blocks 500 (380 with at most half the SM's blocks), with the default
-// tile 370 (290); a block starts and ends in 2000; a split costs 0.24 per KB of
+// tile 370 (290); a block starts and ends in 2000, and 600 more per unit that its
+// stage holds beyond 4 (pairs of 64 channels, tiles of 16 x 256: 866 us, 1006 in
+// three splits); a split costs 0.24 per KB of
 // output (its additions reach the L2 at 4.3 TB/s).  64 trials x 12500 samples:
 // 131 us with the default tile, 52 wide in eight splits, 47 with the default tile
 // in six; 512 trials (0.4 pc cm^-3 apart): 415 with the default tile, 266 wide and,

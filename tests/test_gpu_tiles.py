@@ -130,3 +130,16 @@ def test_large_chunks(lib, tile):
         lib.sps_dedisperse(plan, x, out[-1])
     assert plan.status() == 0
     assert torch.equal(*out)
+
+
+def test_explicit_tiles_of_large_chunks_are_not_split_for_their_last_round(lib):
+    """A block whose stage holds 32 pairs takes long to fill its ring: in three splits the pass of 1536 channels takes
+    1006 us, in one 866."""
+    plan = _plan(lib, 1536, 12500, 512, 0.1)
+    cfg = plan.config
+    cfg.brute = lib.DedispConfig(4, 8, 4, 1, 64, 1)
+    plan.config = cfg
+    assert plan.tiles()[1] == 1
+    cfg.brute = lib.DedispConfig(8, 8, 4, 1, 16, 2)
+    plan.config = cfg
+    assert plan.tiles()[1] > 1
