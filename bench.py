@@ -472,7 +472,8 @@ def events_ms(torch, fn, reps, warm=2):
 def leg_batched(torch, dev, reps=5):
     """The batched-beam workload: 40 beams (alternately 1536 and 384 channels,
     512-4096 DM trials with steps 0.1-0.5, 1-7 widths) per 1.024 s batch, on the
-    GA-tuned tiles stored per channel count, as one graph launch (sps_batch_*)
+    tiles stored per channel count (GA-tuned, or the default where that is faster),
+    as one graph launch (sps_batch_*)
     against plain per-beam sps_search launches on one stream; every beam's
     batched outputs must equal its own search's."""
     import paper_1811_04165_gb300 as sps
@@ -503,7 +504,7 @@ def leg_batched(torch, dev, reps=5):
            "per_beam_ms_per_batch": t_beam, "speedup_vs_per_beam": t_beam / t_batch,
            "real_time_beams": len(wls) * 1024.0 / t_batch, "exact_vs_per_beam": exact,
            "shared_pass_launches": batch.list_launches,
-           "kernel_configs": f"GA-tuned per channel count (stored), taken by {tuned} of {len(plans)} beams",
+           "kernel_configs": f"stored per channel count (GA-tuned, or the default where faster), taken by {tuned} of {len(plans)} beams",
            "plan_s": plan_s, "inputs": "device-drawn noise (timing and exactness do not depend on values)"}
     del batch
     torch.cuda.empty_cache()

@@ -8,7 +8,9 @@ The beams (``synth.batch_beams``): 1.024 s batches of 12500 samples, alternately
 0.1-0.5, the first 1-7 boxcar widths of 1..64, two pulses each.  Kernel tiles
 per channel count come from a live GA run (`sps_tune`, full gene space, Sec. 4)
 on the beam of that shape with the most DM trials, under a workspace bound;
-beams whose tables do not fit the tuned tiles keep their defaults.  Timing:
+beams whose tables do not fit the tuned tiles keep their defaults, and so does a
+channel count whose defaults are the faster ones (the GA does not see the tiles
+that the library picks for its default configuration).  Timing:
 CUDA events around whole batches, inputs larger than L2.  Every beam's batched
 outputs are checked equal to its own search.
 """
@@ -47,8 +49,9 @@ def _time(fn, n, warm=2):
     return e0.elapsed_time(e1) / n
 
 
-# GA-tuned configurations per channel count for the batched-beam mix, written
-# by `--save-tuned` on a GB300 (applied where a beam's tables fit them).
+# Configurations per channel count for the batched-beam mix, GA-tuned or the
+# default where that is faster, written by `--save-tuned` on a GB300 (applied where
+# a beam's tables fit them).
 TUNED = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned", "gb300_batch_beams_configs.json")
 
 
@@ -76,9 +79,11 @@ def apply_tuned(plans, path=TUNED):
 
 
 def tune_shapes(plans, wls, xs, evals, ws_limit):
-    """GA-tuned configuration per channel count, applied where it fits."""
+    """GA-tuned configuration per channel count, or the default one where that is
+    faster over all its beams; applied where it fits."""
     import torch
     out = {}
+    defaults = [p.config for p in plans]
     for ch in sorted({wl.channels for wl in wls}):
         idx = [b for b, wl in enumerate(wls) if wl.channels == ch]
         rep = max(idx, key=lambda b: wls[b].dms.size)
@@ -87,18 +92,32 @@ def tune_shapes(plans, wls, xs, evals, ws_limit):
         t0 = time.perf_counter()
         best, res, trace = sps_tune(p, xs[rep], which=SPACE_FULL, workspace=ws,
                                     desc=search_desc(algorithm=TUNE_GA, max_evaluations=evals, seed=ch), reps=1)
-        del ws
-        cfg = p.config
+        cfg, default = p.config, defaults[rep]
+        ms = {}
+        for name, c in (("default", default), ("tuned", cfg)):
+            ms[name] = 0.0
+            for b in idx:
+                try:
+                    plans[b].config = c if name == "tuned" else defaults[b]
+                except SpsError:
+                    plans[b].config = defaults[b]
+                o = plans[b].alloc_outputs()
+                w = ws if plans[b].workspace_bytes <= ws.numel() else None
+                ms[name] += _time(lambda: plans[b].search(xs[b], out=o, workspace=w), 5)
+                plans[b]._ws = None
+        if ms["default"] <= ms["tuned"]:
+            cfg = default
         applied = 0
         for b in idx:
             try:
                 plans[b].config = cfg
                 applied += 1
             except SpsError:
-                pass
+                plans[b].config = defaults[b]
+        del ws
         out[str(ch)] = {"tuned_on": wls[rep].name, "evaluations": res.evaluations, "best_ms": res.best_fitness,
-                        "seconds": time.perf_counter() - t0, "config": cfg.as_dict(), "applied_to": applied,
-                        "beams": len(idx)}
+                        "seconds": time.perf_counter() - t0, "per_beam_ms": ms, "config": cfg.as_dict(),
+                        "applied_to": applied, "beams": len(idx)}
     return out
 
 
@@ -109,7 +128,7 @@ def main(argv=None):
     ap.add_argument("--tune-evals", type=int, default=60, help="0 keeps the default configurations")
     ap.add_argument("--ws-limit-gb", type=float, default=1.0, help="workspace bound per beam while tuning")
     ap.add_argument("--reps", type=int, default=5)
-    ap.add_argument("--batch-ws-gb", type=float, default=48.0, help="largest batch workspace to allocate")
+    ap.add_argument("--batch-ws-gb", type=float, default=64.0, help="largest batch workspace to allocate")
     ap.add_argument("--out", default=None)
     ap.add_argument("--save-tuned", default=None, metavar="FILE",
                     help="write the tuned configuration per channel count (JSON) for later batches")
@@ -128,7 +147,7 @@ def main(argv=None):
             import torch
             with open(a.save_tuned, "w") as f:
                 json.dump({"how": "python -m paper_1811_04165_gb300.batch_study (live GA, full space, "
-                                  f"{a.tune_evals} evaluations per channel count)",
+                                  f"{a.tune_evals} evaluations per channel count; the default where faster)",
                            "gpu": torch.cuda.get_device_name(), "workload": "batched beams (synth.batch_beams)",
                            "configs": {ch: r["config"] for ch, r in res["tuning"].items()}}, f, indent=1)
     # plain per-beam launches on one stream, one workspace sized for the largest beam
