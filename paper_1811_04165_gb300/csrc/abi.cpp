@@ -151,7 +151,6 @@ sps_status presum_prepass(const sps_plan* p, const sps_dedisp_config& cfg, const
   a.splits = splits;
   a.n_dm = rows;
   a.n_groups = p->channels / per;
-  a.group_units = (per + K - 1) / K;
   a.fold_units = presum_fold_units(cfg);
   a.max_start = (int32_t)(p->n_in - p->n_t);
   a.n_out = n_out;

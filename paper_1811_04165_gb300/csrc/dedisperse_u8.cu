@@ -56,15 +56,6 @@ __device__ __forceinline__ uint32_t madd(uint32_t a, uint32_t one, uint32_t c) {
   return d;
 }
 
-// NW words at shared address addr + 128 * m, m < NW (immediate offsets).
-template <int NW, int M = 0>
-__device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
-  if constexpr (M < NW) {
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(w[M]) : "r"(addr), "n"(M * 128));
-    lds_row<NW, M + 1>(addr, w);
-  }
-}
-
 // BUILD: copies 1..3 are made here, not staged.
 // WALK: the block walks gpb > 1 groups in turn (subband step one); without it
 // the block has one group, compiled as a plain loop over its chunks.

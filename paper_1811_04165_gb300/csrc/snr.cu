@@ -1154,7 +1154,7 @@ sps_status launch_snr(const SnrArgs& a, const sps_snr_config& c, Stream& st) {
     const size_t smem = pow2_smem(a.n_t + room, a.pow2_widths);
     const bool fits = row_fits(a.max_smem, a.n_t, smem - prefix_smem(a.n_t) + 8192);
     if (aligned && !fits && stream_form(a)) {
-      // rows too long to stage whole: the streaming form, any row length
+      // rows too long to stage whole: the streaming form (16-byte aligned rows)
       const size_t stream = stream_smem(a.pow2_widths, c.threads);
       StreamKernel fn = stream_variant(a.pow2_widths);
       SPS_CUDA(launch(st, fn, dim3(a.n_dms), c.threads, stream, a));

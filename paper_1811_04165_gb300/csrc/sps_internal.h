@@ -121,7 +121,6 @@ struct PresumPassArgs {
   int32_t di_pad;
   int32_t n_dm;            // delay-table rows
   int32_t n_groups;
-  int32_t group_units;     // units per group
   int32_t fold_units;      // units a 16-bit lane sums exactly between folds (presum_fold_units)
   int32_t splits;          // blocks per output tile, each summing a share of its chunks (int32 rows, zeroed before)
   int32_t max_start;       // bound on any staged window's start (the pass's largest delay)
@@ -361,7 +360,7 @@ struct sps_plan {
 
   sps_kernel_config cfg{};
   // the tile the brute-force pass runs with: cfg.brute, or the one the library
-  // picks for the default pre-summed tile (presum_tile in plan.cpp)
+  // picks for the default pre-summed tile (choose_tile in plan.cpp)
   sps_dedisp_config brute_tile{};
   sps_dedisp_config step1_tile{}, step2_tile{};  // likewise of the two steps
   bool build_copies = false;       // the single-channel pass makes its shifted copies itself

@@ -106,4 +106,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
   return mbar_wait_polls(bar, parity, status, kMaxPolls);
 }
 
+// NW words at shared address addr + 128 * m, m < NW (immediate offsets).
+template <int NW, int M = 0>
+__device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
+  if constexpr (M < NW) {
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(w[M]) : "r"(addr), "n"(M * 128));
+    lds_row<NW, M + 1>(addr, w);
+  }
+}
+
 }  // namespace sps

@@ -11,6 +11,7 @@
 #include <cstdint>
 
 #include "sps_internal.h"
+#include "tma.cuh"
 
 namespace sps {
 
@@ -18,16 +19,7 @@ constexpr int kWideTrials = 8;  // trials per thread
 constexpr int kWideWords = 7;   // words per thread and trial
 constexpr int kWideTime = 64 * kWideWords;  // samples of a warp
 
-// NW words at shared address addr + 128 * m (immediate offsets).
-template <int NW, int M = 0>
-__device__ __forceinline__ void lds_row(uint32_t addr, uint32_t (&w)[NW]) {
-  if constexpr (M < NW) {
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(w[M]) : "r"(addr), "n"(M * 128));
-    lds_row<NW, M + 1>(addr, w);
-  }
-}
-
-// The same into `w` only where `load` is set (uniform over the warp); otherwise
+// lds_row (tma.cuh) into `w` only where `load` is set (uniform over the warp); otherwise
 // `w` keeps its words.
 template <int NW, int M = 0>
 __device__ __forceinline__ void lds_row_if(bool load, uint32_t addr, uint32_t (&w)[NW]) {
